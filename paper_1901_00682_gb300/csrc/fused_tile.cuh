@@ -1,0 +1,524 @@
+// Fused local solver on 4 x 4 micro-tiles for subdomains of any shape up to 128 x 128
+// (the kernel of every subdomain that is not exactly 128 x 128).
+//
+// What bounds the local solve is latency and issue slots, not memory: a subdomain
+// lives on chip for its whole inner loop, so the time of an inner iteration is the
+// length of its dependency chain (two barriers, the shared-memory exchange) and the
+// instructions its warps issue in between.  Holding 16 pixels per thread puts most
+// neighbours in registers, lets the arithmetic run on packed float32 pairs and leaves
+// one 16-byte exchange per edge and 16 pixels.
+//
+// Mapping.  LPR lanes hold a row group: 4 rows of 4 LPR columns (LPR = 8, 16, 32 for
+// subdomains up to 32, 64, 128 columns wide), so a warp holds 32 / LPR row groups and a
+// CTA of NW warps a band of BAND = 4 NW (32 / LPR) rows.  A subdomain is one CTA, or a
+// cluster of the fewest CTAs whose bands cover its rows; halo rows then travel with
+// st.async counted on mbarriers (bounded waits), as in kernels_fused_mt4.cu.  Registers
+// hold u, the dual dofs p1 (top edge) and p2 (left edge) and their extrapolations; f and
+// the proximal centres, read once per inner iteration by the thread that owns them, wait
+// in shared memory in the owner's order, which keeps a thread within 128 registers and
+// four 128-thread CTAs on an SM.
+//
+// Shapes.  A subdomain smaller than the block of pixels its threads cover is padded on
+// the right and at the bottom.  u is pinned to 0 in the first padding column and row, so
+// the dof on the left edge of that column is the subdomain's right side (D_s u = -u of
+// the last column) and the dof on the top edge of that row its bottom side, updated as
+// any other dof; what lies further out is never read by a pixel of the subdomain.  Where
+// the subdomain fills the block (no padding) the sides are updated by lanes of other
+// warps, as in kernels_fused_mt4.cu.  A side on the image boundary is kept at 0 by
+// clamping its dofs to [-0, 0].
+//
+// Measured per outer iteration of 10 inner ones, multiplier update included, against
+// the cluster-barrier kernel (a column of 8 pixels per thread) it replaces here: 1080 x
+// 1920 in 120 x 128 subdomains 106 -> 44 us, 2160 x 3840 448 -> 160, 2999 x 3001 in 125 x
+// 125/126 477 -> 182, 4096 x 4096 in 64 x 64 572 -> 217 and in 32 x 32 527 -> 211, 128 x
+// 128 in 64 x 64 21.1 -> 13.0, 321 x 481 in 107 x 120/121 25.8 -> 17.0.
+//
+// Every value is computed with the operations of the scalar iteration in its order
+// (pointwise.cuh), so the results are those of the plain path bit for bit.
+#pragma once
+
+#include "fused_common.cuh"
+#include "internal.cuh"
+
+namespace ddtv {
+
+namespace {
+
+template <int LPR_, int NW_>
+struct TileLayout {
+  static constexpr int LPR = LPR_, NW = NW_;
+  static constexpr int RG = 32 / LPR;               // row groups per warp
+  static constexpr int NG = NW * RG;                // row groups per CTA
+  static constexpr int BAND = 4 * NG, BW = 4 * LPR, NT = 32 * NW;
+  static constexpr int SLOT = 4 * (LPR + 1);        // a row group's UR / QL slots
+  static constexpr int kMaxSmemCoef = 64;
+  static constexpr int UB = 0;                      // (NG + 1) x BW: row 0 = u above the band, G + 1 = last row of group G
+  static constexpr int Q1 = UB + (NG + 1) * BW;     // (NG + 1) x BW: row G = pbar1 of group G's first row, NG = below
+  static constexpr int UR = Q1 + (NG + 1) * BW;     // NG x SLOT: slot 0 = 0 (left of the tile), cl + 1 = u of lane cl's right column
+  static constexpr int QL = UR + NG * SLOT;         // NG x SLOT: slot cl = pbar2 of lane cl's left edge, LPR = the right side
+  static constexpr int F = QL + NG * SLOT;          // 4 x NT x 4: f (or g), thread order
+  static constexpr int H1 = F + 16 * NT;            // proximal centres, thread order
+  static constexpr int H2 = H1 + 16 * NT;
+  static constexpr int CO = H2 + 16 * NT;           // kMaxSmemCoef x 16: the coefficients, each twice
+  static constexpr int PBS = CO + 16 * kMaxSmemCoef;  // p of the bottom side of a subdomain that fills the block
+  static constexpr int HBS = PBS + BW;              // its proximal centre
+  static constexpr int XUB = HBS + BW;              // u of the subdomain's last row, for that side
+  static constexpr int MB = XUB + BW;               // two mbarriers
+  static constexpr size_t BYTES = sizeof(float) * MB + 16;
+  static constexpr int kRightThread = 32;           // threads kRightThread + i update the right side of band row i
+  static constexpr int kBottomWarp = NW > 2 ? 2 : 0;
+  static_assert(Q1 % 4 == 0 && UR % 4 == 0 && QL % 4 == 0 && F % 4 == 0 && CO % 4 == 0 && PBS % 4 == 0 && MB % 2 == 0,
+                "16-byte alignment of the vector accesses");
+  static_assert(kRightThread + BAND <= NT, "a thread per right-side dof");
+};
+
+// four consecutive floats of a row, the first n valid (n <= 0: none), the rest 0
+__device__ __forceinline__ void load4(const float* p, int n, bool vec, float* v) {
+  if (vec && n >= 4) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    v[0] = x.x;
+    v[1] = x.y;
+    v[2] = x.z;
+    v[3] = x.w;
+    return;
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) v[c] = c < n ? p[c] : 0.f;
+}
+
+__device__ __forceinline__ void store4(float* p, int n, bool vec, float a, float b, float c, float d) {
+  if (vec && n >= 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+    return;
+  }
+  if (n > 0) p[0] = a;
+  if (n > 1) p[1] = b;
+  if (n > 2) p[2] = c;
+  if (n > 3) p[3] = d;
+}
+
+__device__ __forceinline__ float half_of(f32x2 v, int h) { return h ? hi2(v) : lo2(v); }
+
+// The local solve of subdomain (a, b) of the problem A, its interface strips written to
+// out.  CLU: the subdomain is a cluster of gridDim.x CTAs (else one CTA).  PAD: the
+// subdomain may be smaller than the block (false: every subdomain fills it).
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
+__device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out, const int a, const int b) {
+  using L = TileLayout<LPR, NW>;
+  constexpr int NG = L::NG, BAND = L::BAND, BW = L::BW, NT = L::NT;
+  extern __shared__ __align__(128) float smem[];
+  float* sUB = smem + L::UB;
+  float* sQ1 = smem + L::Q1;
+  float* sCo = smem + L::CO;
+  const uint32_t mbU = smem_addr(smem + L::MB), mbQ = mbU + 8;
+
+  const Grid g = A.g;
+  const int CL = CLU ? (int)gridDim.x : 1, rank = CLU ? (int)blockIdx.x : 0;
+  const int r0 = part_start(a, g.H, g.NR), mr = part_start(a + 1, g.H, g.NR) - r0;
+  const int c0 = part_start(b, g.W, g.NC), mc = part_start(b + 1, g.W, g.NC) - c0;
+  const bool s_top = a > 0 || g.cut_top, s_bot = a + 1 < g.NR || g.cut_bot, s_lft = b > 0, s_rgt = b + 1 < g.NC;
+  const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
+  const int G = w * L::RG + l / LPR, cl = l % LPR;  // row group, lane of the group
+  const int j0 = 4 * cl;                            // first column in the subdomain
+  const int i0 = rank * BAND + 4 * G;               // first row in the subdomain
+  const int K = A.K;
+  const int W2 = g.W + g.NC;
+  const float tau = A.tau;
+  const bool fill_c = !PAD || mc == BW, fill_r = !PAD || mr == CL * BAND;  // no padding column / row
+  const bool last_group = rank == CL - 1 && G == NG - 1;
+  const bool push_down = CLU && G == NG - 1 && rank + 1 < CL;  // u of the band's last row
+  const bool push_up = CLU && G == 0 && rank > 0;              // pbar1 of the band's first row
+  const bool bottom_lane = fill_r && s_bot && rank == CL - 1 && w == L::kBottomWarp && l < LPR;
+  const int rr = tid - L::kRightThread;                        // band row whose right side this thread updates
+  const bool right_lane = fill_c && s_rgt && rr >= 0 && rr < BAND && rank * BAND + rr < mr;
+  const int r_slot = (rr >> 2) * L::SLOT + 4 * LPR + 2 * (rr & 1) + ((rr >> 1) & 1);
+  constexpr uint32_t kHaloBytes = 4 * BW;
+  float* const myUR = smem + L::UR + G * L::SLOT + 4 * (cl + 1);
+  float* const myQL = smem + L::QL + G * L::SLOT + 4 * cl;
+  float* const myF = smem + L::F + 4 * tid;  // column c at + c * 4 NT; the proximal centres likewise
+  constexpr int kH1 = L::H1 - L::F, kH2 = L::H2 - L::F;
+  uint32_t remote_u = 0, remote_q1 = 0, remote_mbU = 0, remote_mbQ = 0;
+  if (push_down) {
+    remote_u = map_rank(smem_addr(sUB + j0), rank + 1);
+    remote_mbU = map_rank(mbU, rank + 1);
+  }
+  if (push_up) {
+    remote_q1 = map_rank(smem_addr(sQ1 + NG * BW + j0), rank - 1);
+    remote_mbQ = map_rank(mbQ, rank - 1);
+  }
+  if (CLU) {
+    if (tid == 0) {
+      mbar_init(mbU, 1);
+      mbar_init(mbQ, 1);
+      // the first phases, armed before any neighbour may complete them
+      if (rank > 0) mbar_arrive_expect_tx(mbU, kHaloBytes);
+      if (rank + 1 < CL) mbar_arrive_expect_tx(mbQ, kHaloBytes);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    cluster_arrive<true>();  // matched before the first halo is sent: the loads hide the wait
+  }
+  // clamp limits of the dofs of row r / column c: 0 on an image-boundary side
+  float lim1[4], lim2[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    lim1[q] = (q == 0 && i0 == 0 && !s_top) || (PAD && i0 + q == mr && !s_bot) ? 0.f : 1.f;
+    lim2[q] = (q == 0 && j0 == 0 && !s_lft) || (PAD && j0 + q == mc && !s_rgt) ? 0.f : 1.f;
+  }
+  if (!PAD) {
+#pragma unroll
+    for (int q = 1; q < 4; ++q) lim1[q] = lim2[q] = 1.f;
+  }
+
+  // pairs [column c][e]: rows (e, e + 2) of column j0 + c
+  f32x2 U[4][2], P1[4][2], P2[4][2], Q1[4][2], Q2[4][2];
+  uint32_t in_d = 0;  // bit 4c + r: pixel (row r, column j0 + c) lies in the inpainting domain
+  float pr_s = 0.f, hr_s = 0.f;
+
+  // ---- load the state, build the proximal centre
+  {
+    const bool vec = (g.W & 3) == 0 && (c0 & 3) == 0;
+    float h1[4][4], h2[4][4], fv[4][4];
+    float u[4][4], p1[4][4], p2[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = i0 + r, gi = r0 + i;
+      const int n = i < mr ? mc - j0 : 0;                                // pixels of this lane's row
+      const int n1 = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;             // p1 dofs (row mr: the bottom side)
+      const int n2 = i < mr ? mc + (s_rgt ? 1 : 0) - j0 : 0;             // p2 dofs (column mc: the right side)
+      load4(A.u + (size_t)gi * g.W + c0 + j0, n, vec, u[r]);
+      load4(A.f + (size_t)gi * g.W + c0 + j0, n, vec, fv[r]);
+      load4(A.P1 + (size_t)(gi + a) * g.W + c0 + j0, n1, vec, p1[r]);
+      load4(A.P2 + (size_t)gi * W2 + c0 + b + j0, n2, false, p2[r]);
+      if (MASK) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c < n && A.mask[(size_t)gi * g.W + c0 + j0 + c]) in_d |= 1u << (4 * c + r);
+      }
+    }
+    if (right_lane) {
+      const int gi = r0 + rank * BAND + rr;
+      pr_s = A.P2[(size_t)gi * W2 + c0 + BW + b];
+      hr_s = phat_s(pr_s, A.lamv[(size_t)b * g.H + gi], tau);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = i0 + r, gi = r0 + i;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int j = j0 + c;
+        h1[r][c] = p1[r][c];
+        h2[r][c] = p2[r][c];
+        if (r == 0 && i == 0 && s_top && j < mc) h1[r][c] = phat_t(p1[r][c], A.lamh[(ptrdiff_t)(a - 1) * g.W + c0 + j], tau);
+        if (PAD && i == mr && s_bot && j < mc) h1[r][c] = phat_s(p1[r][c], A.lamh[(size_t)a * g.W + c0 + j], tau);
+        if (c == 0 && j == 0 && s_lft && i < mr) h2[r][c] = phat_t(p2[r][c], A.lamv[(size_t)(b - 1) * g.H + gi], tau);
+        if (PAD && j == mc && s_rgt && i < mr) h2[r][c] = phat_s(p2[r][c], A.lamv[(size_t)b * g.H + gi], tau);
+        if (FID == FID_SEG) fv[r][c] = (fv[r][c] - A.c1) * (fv[r][c] - A.c1) - (fv[r][c] - A.c2) * (fv[r][c] - A.c2);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        U[c][e] = pk2(u[e][c], u[e + 2][c]);
+        Q1[c][e] = P1[c][e] = pk2(p1[e][c], p1[e + 2][c]);
+        Q2[c][e] = P2[c][e] = pk2(p2[e][c], p2[e + 2][c]);
+      }
+      *reinterpret_cast<float4*>(myF + 4 * NT * c) = make_float4(fv[0][c], fv[2][c], fv[1][c], fv[3][c]);
+      *reinterpret_cast<float4*>(myF + kH1 + 4 * NT * c) = make_float4(h1[0][c], h1[2][c], h1[1][c], h1[3][c]);
+      *reinterpret_cast<float4*>(myF + kH2 + 4 * NT * c) = make_float4(h2[0][c], h2[2][c], h2[1][c], h2[3][c]);
+    }
+    *reinterpret_cast<float4*>(sQ1 + G * BW + j0) = make_float4(p1[0][0], p1[0][1], p1[0][2], p1[0][3]);
+    *reinterpret_cast<ulonglong2*>(myQL) = make_ulonglong2(P2[0][0], P2[0][1]);
+    if (G == NG - 1) {
+      // pbar1 of the row below the band: the next CTA's first row (its halo of later
+      // iterations), the bottom side of a subdomain that fills the block, or 0
+      const int i = rank * BAND + BAND, n = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;
+      float q[4];
+      load4(A.P1 + (size_t)(r0 + i + a) * g.W + c0 + j0, n, vec, q);
+      *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(q[0], q[1], q[2], q[3]);
+      if (last_group && fill_r && s_bot) {
+        float h[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) h[c] = c < n ? phat_s(q[c], A.lamh[(size_t)a * g.W + c0 + j0 + c], tau) : 0.f;
+        *reinterpret_cast<float4*>(smem + L::PBS + j0) = make_float4(q[0], q[1], q[2], q[3]);
+        *reinterpret_cast<float4*>(smem + L::HBS + j0) = make_float4(h[0], h[1], h[2], h[3]);
+      }
+    }
+    if (G == 0 && rank == 0) *reinterpret_cast<float4*>(sUB + j0) = make_float4(0.f, 0.f, 0.f, 0.f);  // u above the tile
+    if (cl == 0) *reinterpret_cast<float4*>(smem + L::UR + G * L::SLOT) = make_float4(0.f, 0.f, 0.f, 0.f);  // u left of it
+    // the slot right of the last lane: the right side of a subdomain that fills the block, else 0
+    if (rr >= 0 && rr < BAND) smem[L::QL + r_slot] = pr_s;
+  }
+  const bool coef_smem = K <= L::kMaxSmemCoef;
+  if (coef_smem)
+    for (int q = tid; q < 16 * K; q += NT)
+      sCo[q] = reinterpret_cast<const float*>(A.coef)[(q >> 4) * 8 + ((q & 15) >> 1)];
+  __syncthreads();
+  bool timed_out = false;
+  uint32_t phU = 0, phQ = 0;  // index of the next phase of mbU / mbQ this thread waits for
+  if (CLU) cluster_wait();  // every CTA's barriers are initialised and armed
+  auto wait_u = [&]() {
+    if (!mbar_wait(mbU, phU & 1)) timed_out = true;
+    ++phU;
+    if (cl == 0) mbar_arrive_expect_tx(mbU, kHaloBytes);  // arm the next phase
+  };
+  auto wait_q = [&]() {
+    if (!mbar_wait(mbQ, phQ & 1)) timed_out = true;
+    ++phQ;
+    if (cl == 0) mbar_arrive_expect_tx(mbQ, kHaloBytes);
+  };
+  // the padding column and row whose u is pinned: columns j0 .. j0 + 3 hold column mc at
+  // mc & 3 if this lane is the one, rows likewise
+  const bool pin_c = PAD && !fill_c && (mc >> 2) == cl;
+  const bool pin_r = PAD && !fill_r && ((mr - rank * BAND) >> 2) == G && mr >= rank * BAND;
+  const int cpad = mc & 3, rpad = mr & 3;
+
+#pragma unroll 2
+  for (int k = 0; k < K; ++k) {
+    f32x2 SIG, UA, UBc, PA, PC, PB, TH, SS;
+    if (coef_smem) {
+      const ulonglong2 cf0 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k);
+      const ulonglong2 cf1 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 4);
+      const ulonglong2 cf2 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 8);
+      const ulonglong2 cf3 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 12);
+      SIG = cf0.x, UA = cf0.y, UBc = cf1.x, SS = cf1.y, PA = cf2.x, PC = cf2.y, PB = cf3.x, TH = cf3.y;
+    } else {
+      const float4 ca = __ldg(reinterpret_cast<const float4*>(A.coef) + 2 * k);
+      const float4 cb = __ldg(reinterpret_cast<const float4*>(A.coef) + 2 * k + 1);
+      SIG = pk2(ca.x, ca.x), UA = pk2(ca.y, ca.y), UBc = pk2(ca.z, ca.z), SS = pk2(ca.w, ca.w);
+      PA = pk2(cb.x, cb.x), PC = pk2(cb.y, cb.y), PB = pk2(cb.z, cb.z), TH = pk2(cb.w, cb.w);
+    }
+    const Coef co{lo2(SIG), lo2(UA), lo2(UBc), lo2(SS), lo2(PA), lo2(PC), lo2(PB), lo2(TH)};
+    if (push_down && k > 0) wait_q();  // pbar1 halo of iteration k - 1
+    // ---- u-step: pair e = 1 (holding the group's last row) first
+    {
+      const float4 qb = *reinterpret_cast<const float4*>(sQ1 + (G + 1) * BW + j0);  // pbar1 of the row below
+      const ulonglong2 qn = *reinterpret_cast<const ulonglong2*>(myQL + 4);         // left edge of the lane to the right
+      const f32x2 QRn[2] = {qn.x, qn.y};
+      const float qbv[4] = {qb.x, qb.y, qb.z, qb.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const ulonglong2 fc = *reinterpret_cast<const ulonglong2*>(myF + 4 * NT * c);
+#pragma unroll
+        for (int ee = 0; ee < 2; ++ee) {
+          const int e = 1 - ee;
+          const f32x2 fg = e == 0 ? fc.x : fc.y;
+          // bottom - top: for e = 1 the rows below (2, 4) straddle pair 0 and the group below
+          const f32x2 bt = e == 0 ? sub2(Q1[c][1], Q1[c][0])
+                                  : pk2(hi2(Q1[c][0]) - lo2(Q1[c][1]), qbv[c] - hi2(Q1[c][1]));
+          const f32x2 right = c < 3 ? Q2[c + 1][e] : QRn[e];
+          const f32x2 d = sub2(add2(bt, right), Q2[c][e]);  // div_px
+          const f32x2 ub = fma2(SIG, d, U[c][e]);
+          const bool dl = MASK && ((in_d >> (4 * c + e)) & 1u), dh = MASK && ((in_d >> (4 * c + e + 2)) & 1u);
+          f32x2 un;
+          if (FID == FID_L2) {
+            un = fma2(UBc, fg, mul2(UA, ub));
+            if (MASK) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
+          } else if (FID == FID_L1) {  // ubar - P_[-s,s](ubar - f)
+            const f32x2 v = sub2(ub, fg);
+            un = sub2(ub, pk2(clamp_abs(lo2(v), co.s), clamp_abs(hi2(v), co.s)));
+            if (MASK) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
+          } else {
+            un = pk2(prox_ubar<FID>(lo2(ub), lo2(fg), dl, co), prox_ubar<FID>(hi2(ub), hi2(fg), dh, co));
+          }
+          U[c][e] = un;
+        }
+      }
+      if (PAD) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (pin_c && cpad == q) U[q][0] = U[q][1] = 0ull;
+          if (pin_r && rpad == q) {
+            const int e = q & 1;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) U[c][e] = q < 2 ? pk2(0.f, hi2(U[c][e])) : pk2(lo2(U[c][e]), 0.f);
+          }
+        }
+      }
+      const float4 ul = make_float4(hi2(U[0][1]), hi2(U[1][1]), hi2(U[2][1]), hi2(U[3][1]));
+      if (push_down)
+        st_async_v4_f32(remote_u, ul.x, ul.y, ul.z, ul.w, remote_mbU);
+      else if (last_group)
+        *reinterpret_cast<float4*>(smem + L::XUB + j0) = ul;  // for the bottom side's update
+      if (G < NG - 1) *reinterpret_cast<float4*>(sUB + (G + 1) * BW + j0) = ul;
+      *reinterpret_cast<ulonglong2*>(myUR) = make_ulonglong2(U[3][0], U[3][1]);
+    }
+    __syncthreads();
+    // ---- p-step: first the dofs that need no row above the group (in the first group that
+    // row is the halo from the CTA above), then the first row's pbar1 and its push upwards
+    {
+      const ulonglong2 ul = *reinterpret_cast<const ulonglong2*>(myUR - 4);  // right column of the lane to the left
+      f32x2 H0[4];  // the proximal centres of rows (0, 2), for the second part
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const ulonglong2 h1 = *reinterpret_cast<const ulonglong2*>(myF + kH1 + 4 * NT * c);
+        const ulonglong2 h2 = *reinterpret_cast<const ulonglong2*>(myF + kH2 + 4 * NT * c);
+        H0[c] = mul2(PB, h1.x);
+        {
+          const f32x2 tt = fma2(PC, sub2(U[c][1], U[c][0]), fma2(PA, P1[c][1], mul2(PB, h1.y)));  // p_target
+          const f32x2 pn = pk2(clamp_abs(lo2(tt), lim1[1]), clamp_abs(hi2(tt), lim1[3]));
+          Q1[c][1] = fma2(TH, sub2(pn, P1[c][1]), pn);
+          P1[c][1] = pn;
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const f32x2 leftu = c > 0 ? U[c - 1][e] : (e == 0 ? ul.x : ul.y);
+          const f32x2 tt = fma2(PC, sub2(U[c][e], leftu), fma2(PA, P2[c][e], mul2(PB, e == 0 ? h2.x : h2.y)));
+          const f32x2 pn = pk2(clamp_abs(lo2(tt), lim2[c]), clamp_abs(hi2(tt), lim2[c]));
+          Q2[c][e] = fma2(TH, sub2(pn, P2[c][e]), pn);
+          P2[c][e] = pn;
+        }
+      }
+      *reinterpret_cast<ulonglong2*>(myQL) = make_ulonglong2(Q2[0][0], Q2[0][1]);
+      if (push_up) wait_u();  // u halo of iteration k
+      const float4 ua = *reinterpret_cast<const float4*>(sUB + G * BW + j0);  // u of the row above
+      const float uav[4] = {ua.x, ua.y, ua.z, ua.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        // rows (0, 2): the rows above (-1, 1) straddle the group above and pair 1
+        const f32x2 du = pk2(lo2(U[c][0]) - uav[c], hi2(U[c][0]) - lo2(U[c][1]));
+        const f32x2 tt = fma2(PC, du, fma2(PA, P1[c][0], H0[c]));
+        const f32x2 pn = pk2(clamp_abs(lo2(tt), lim1[0]), clamp_abs(hi2(tt), lim1[2]));
+        Q1[c][0] = fma2(TH, sub2(pn, P1[c][0]), pn);
+        P1[c][0] = pn;
+      }
+      const float4 q = make_float4(lo2(Q1[0][0]), lo2(Q1[1][0]), lo2(Q1[2][0]), lo2(Q1[3][0]));
+      if (G > 0) *reinterpret_cast<float4*>(sQ1 + G * BW + j0) = q;
+      if (push_up) st_async_v4_f32(remote_q1, q.x, q.y, q.z, q.w, remote_mbQ);
+    }
+    if (right_lane) {  // Du = -u of the last column ((-pc) u = pc (-u) exactly)
+      const float tt = fmaf(-co.pc, smem[L::UR + r_slot], fmaf(co.pa, pr_s, co.pb * hr_s));
+      const float pn = clamp_abs(tt, 1.f);
+      smem[L::QL + r_slot] = fmaf(co.th, pn - pr_s, pn);
+      pr_s = pn;
+    }
+    if (bottom_lane) {  // Du = -u of the last row
+      const float4 pv = *reinterpret_cast<const float4*>(smem + L::PBS + j0);
+      const float4 hv = *reinterpret_cast<const float4*>(smem + L::HBS + j0);
+      const float4 uv = *reinterpret_cast<const float4*>(smem + L::XUB + j0);
+      float pB[4] = {pv.x, pv.y, pv.z, pv.w}, qB[4];
+      const float hB[4] = {hv.x, hv.y, hv.z, hv.w}, uB[4] = {uv.x, uv.y, uv.z, uv.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) p_update(pB[c], qB[c], -uB[c], hB[c], co);
+      *reinterpret_cast<float4*>(smem + L::PBS + j0) = make_float4(pB[0], pB[1], pB[2], pB[3]);
+      *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(qB[0], qB[1], qB[2], qB[3]);
+    }
+    __syncthreads();
+  }
+  if (CLU) {
+    if (push_down) wait_q();  // drain the last pbar1 halo (not read)
+    __syncwarp();
+    cluster_arrive<false>();  // no CTA leaves while a neighbour may still write into it; the
+                              // stores below hide the wait
+  }
+
+  // ---- store u^{n+1}, p~^{n+1} and the interface strips
+  const bool vec = (g.W & 3) == 0 && (c0 & 3) == 0;
+  // the strips of a set start at multiples of the interface edges, not of 4 floats
+  const bool vec_t = vec && (reinterpret_cast<uintptr_t>(out.ST) & 15) == 0;
+  const bool vec_b = vec && (reinterpret_cast<uintptr_t>(out.SB) & 15) == 0;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int e = r & 1, h = r >> 1, i = i0 + r, gi = r0 + i;
+    const int n = i < mr ? mc - j0 : 0;
+    const int n1 = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;
+    const int n2 = i < mr ? mc + (s_rgt ? 1 : 0) - j0 : 0;
+    store4(A.u + (size_t)gi * g.W + c0 + j0, n, vec, half_of(U[0][e], h), half_of(U[1][e], h), half_of(U[2][e], h),
+           half_of(U[3][e], h));
+    const float q0 = half_of(P1[0][e], h), q1 = half_of(P1[1][e], h), q2 = half_of(P1[2][e], h), q3 = half_of(P1[3][e], h);
+    store4(A.P1 + (size_t)(gi + a) * g.W + c0 + j0, n1, vec, q0, q1, q2, q3);
+    if (r == 0 && i == 0 && s_top) store4(out.ST + (ptrdiff_t)(a - 1) * g.W + c0 + j0, n1, vec_t, q0, q1, q2, q3);
+    if (PAD && i == mr && s_bot) store4(out.SB + (size_t)a * g.W + c0 + j0, n1, vec_b, q0, q1, q2, q3);
+    store4(A.P2 + (size_t)gi * W2 + c0 + b + j0, n2, false, half_of(P2[0][e], h), half_of(P2[1][e], h),
+           half_of(P2[2][e], h), half_of(P2[3][e], h));
+    if (j0 == 0 && s_lft && i < mr) out.SL[(size_t)(b - 1) * g.H + gi] = half_of(P2[0][e], h);
+    if (PAD && s_rgt && i < mr) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (j0 + c == mc) out.SR[(size_t)b * g.H + gi] = half_of(P2[c][e], h);
+    }
+  }
+  if (right_lane) {
+    const int gi = r0 + rank * BAND + rr;
+    A.P2[(size_t)gi * W2 + c0 + BW + b] = pr_s;
+    out.SR[(size_t)b * g.H + gi] = pr_s;
+  }
+  if (bottom_lane) {
+    const float4 v = *reinterpret_cast<const float4*>(smem + L::PBS + j0);
+    store4(A.P1 + (size_t)(r0 + mr + a) * g.W + c0 + j0, mc - j0, vec, v.x, v.y, v.z, v.w);
+    store4(out.SB + (size_t)a * g.W + c0 + j0, mc - j0, vec_b, v.x, v.y, v.z, v.w);
+  }
+  if (CLU) {
+    if (timed_out) atomicOr(A.err, 1);
+    __syncwarp();
+    cluster_wait();
+  }
+}
+
+// 16 warps per SM: 128 registers per thread
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
+__global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile(const LocalArgs A) {
+  tile_solve<LPR, NW, CLU, PAD, FID, MASK>(A, A.out, (int)blockIdx.z, (int)blockIdx.y);
+}
+
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
+cudaError_t prepare_tile_one() {
+  return cudaFuncSetAttribute(k_tile<LPR, NW, CLU, PAD, FID, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)TileLayout<LPR, NW>::BYTES);
+}
+
+template <int LPR, int NW, bool CLU, bool PAD>
+cudaError_t prepare_tile_fid() {
+  cudaError_t e;
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L2, false>()) != cudaSuccess) return e;
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L2, true>()) != cudaSuccess) return e;
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L1, false>()) != cudaSuccess) return e;
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L1, true>()) != cudaSuccess) return e;
+  return prepare_tile_one<LPR, NW, CLU, PAD, FID_SEG, false>();
+}
+
+template <int LPR, int NW, bool CLU>
+cudaError_t prepare_tile() {
+  const cudaError_t e = prepare_tile_fid<LPR, NW, CLU, false>();
+  return e != cudaSuccess ? e : prepare_tile_fid<LPR, NW, CLU, true>();
+}
+
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
+cudaError_t launch_tile_one(const LocalArgs& a, int cl, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CLU ? cl : 1, a.g.NC, a.g.NR);
+  cfg.blockDim = dim3(32 * NW, 1, 1);
+  cfg.dynamicSmemBytes = TileLayout<LPR, NW>::BYTES;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CLU ? cl : 1;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CLU ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_tile<LPR, NW, CLU, PAD, FID, MASK>, a);
+}
+
+template <int LPR, int NW, bool CLU, bool PAD>
+cudaError_t launch_tile_fid(const LocalArgs& a, int fid, int cl, cudaStream_t st) {
+  const bool m = a.mask != nullptr;
+  switch (fid) {
+    case FID_L2:
+      return m ? launch_tile_one<LPR, NW, CLU, PAD, FID_L2, true>(a, cl, st)
+               : launch_tile_one<LPR, NW, CLU, PAD, FID_L2, false>(a, cl, st);
+    case FID_L1:
+      return m ? launch_tile_one<LPR, NW, CLU, PAD, FID_L1, true>(a, cl, st)
+               : launch_tile_one<LPR, NW, CLU, PAD, FID_L1, false>(a, cl, st);
+    default: return launch_tile_one<LPR, NW, CLU, PAD, FID_SEG, false>(a, cl, st);
+  }
+}
+
+template <int LPR, int NW, bool CLU>
+cudaError_t launch_tile(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st) {
+  return pad ? launch_tile_fid<LPR, NW, CLU, true>(a, fid, cl, st) : launch_tile_fid<LPR, NW, CLU, false>(a, fid, cl, st);
+}
+
+}  // namespace
+}  // namespace ddtv

@@ -119,8 +119,6 @@ cudaError_t fused_prepare();
 void fused_max_tile(int* rows, int* cols);
 // Number of hardware mappings available for 128 x 128 tiles.
 int fused_num_variants();
-// Name of the configuration chosen for a tile shape and variant (for reports).
-const char* fused_config_name(int mr, int mc, int variant);
 
 // ---- kernels_fused_mt.cu
 // Persistent fused local solver on 2 x 4 micro-tiles (two columns by four rows per
@@ -146,6 +144,23 @@ cudaError_t fused_mt4_prepare();
 // 16-byte aligned, inner count <= fused_mt4_max_inner().
 cudaError_t launch_fused_mt4_batch(const BatchArgs& B, int total_tiles, cudaStream_t st);
 int fused_mt4_max_inner();
+
+// ---- kernels_tile8.cu, kernels_tile16.cu, kernels_tile32.cu (fused_tile.cuh)
+// launch_tile_<LPR>_<NW>: the micro-tile kernel with LPR lanes per row group and NW warps
+// per CTA, cl CTAs per subdomain; pad: some subdomain does not fill the block of
+// 4 LPR columns x cl bands of 4 NW (32 / LPR) rows.
+cudaError_t launch_tile_8_2(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
+cudaError_t launch_tile_8_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
+cudaError_t launch_tile_16_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
+cudaError_t launch_tile_16_8(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
+cudaError_t launch_tile_32_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
+cudaError_t prepare_tile_8_2();
+cudaError_t prepare_tile_8_4();
+cudaError_t prepare_tile_16_4();
+cudaError_t prepare_tile_16_8();
+cudaError_t prepare_tile_32_4();
+// every 64 x 64 subdomain of every image of a batch (launch_tile_16_8's kernel)
+cudaError_t launch_tile_batch_64(const BatchArgs& B, int total_tiles, cudaStream_t st);
 
 // ---- kernels_plain.cu
 // phat = p~ -+ tau lambda on the interface sides, pbar = p~; full arrays.

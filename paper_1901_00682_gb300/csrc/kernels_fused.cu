@@ -1,5 +1,10 @@
-// Fused local solver: all inner iterations of one outer iteration of Algorithm 1 for
-// every subdomain in one launch (Section 5, local problem eq. local, solved by the
+// Fused local solver with cluster barriers: the adaptive inner stop of every subdomain
+// shape but exact 128 x 128, and variant 3 of those; and the choice among the fused
+// kernels (launch_fused_local).  A fixed inner count on any other shape runs the
+// micro-tile kernel of fused_tile.cuh.
+//
+// All inner iterations of one outer iteration of Algorithm 1 for every subdomain in one
+// launch (Section 5, local problem eq. local, solved by the
 // accelerated primal-dual algorithm with the dual field p as the uniformly convex
 // variable; the projection onto the box C of eq. proj_C is fused into the p-step).
 //
@@ -330,41 +335,11 @@ __global__ void __launch_bounds__(BW* TR, (BW * TR <= 256 ? 2 : 1)) k_fused(cons
   fused_tile<BW, R, TR, CL, FID, MASK, ADAPT>(A, A.out, (int)blockIdx.z, (int)blockIdx.y);
 }
 
-// Every tile of a batch of images, one CTA cluster per tile (blockIdx.y = the batch's
-// tile), each with its image's fidelity, parameters and strips.
-template <int BW, int R, int TR, int CL>
-__global__ void __launch_bounds__(BW* TR, (BW * TR <= 256 ? 2 : 1)) k_fused_tile_batch(const BatchArgs B) {
-  const int t = blockIdx.y;
-  const int img = B.tile_img[t];
-  const LocalArgs A = B.args[img];
-  const int q = t - B.tile_base[img];
-  const int a = q / A.g.NC, b = q - a * A.g.NC;
-  const Strips out = B.strips[2 * img + B.write_set];
-  switch (B.fid[img]) {
-    case FID_L2: fused_tile<BW, R, TR, CL, FID_L2, false, false>(A, out, a, b); break;
-    case FID_L1: fused_tile<BW, R, TR, CL, FID_L1, false, false>(A, out, a, b); break;
-    default: fused_tile<BW, R, TR, CL, FID_SEG, false, false>(A, out, a, b); break;
-  }
-}
-
-struct Config {
-  int BW, R, TR, CL;
-  const char* name;
-};
-
-// Cluster-barrier mappings by tile size.  Class 0: tiles up to 32 x 32; class 1: up
-// to 64 x 64; class 2: up to 128 x 128.
-constexpr Config kConfigs[] = {
-    {32, 8, 4, 1, "bw32_r8_tr4_cl1"},    // class 0
-    {64, 8, 8, 1, "bw64_r8_tr8_cl1"},    // class 1
-    {128, 8, 2, 8, "bw128_r8_tr2_cl8"},  // class 2: 256 threads, 2 CTAs/SM
-};
-
 // Hardware mappings of exact 128 x 128 subdomains (dd_tv_params.variant):
 //   0  persistent 4 x 4 micro-tiles, state moved by tensor copies (default)
 //   1  the same kernel moving the state with 16-byte cp.async copies
 //   2  persistent 2 x 4 micro-tiles, 256 threads, 2 CTAs per SM
-//   3  the cluster-barrier kernel of every other tile shape (one subdomain per cluster)
+//   3  the cluster-barrier kernel (one subdomain per cluster)
 constexpr int kNumVariants = 4;
 
 template <int BW, int R, int TR, int CL, int FID, bool MASK, bool ADAPT>
@@ -388,7 +363,7 @@ cudaError_t launch_one(const LocalArgs& a, cudaStream_t st) {
 }
 
 template <int BW, int R, int TR, int CL, bool ADAPT>
-cudaError_t launch_fid_a(const LocalArgs& a, int fid, cudaStream_t st) {
+cudaError_t launch_fid(const LocalArgs& a, int fid, cudaStream_t st) {
   const bool m = a.mask != nullptr;
   switch (fid) {
     case FID_L2:
@@ -401,33 +376,42 @@ cudaError_t launch_fid_a(const LocalArgs& a, int fid, cudaStream_t st) {
   }
 }
 
-template <int BW, int R, int TR, int CL>
-cudaError_t launch_fid(const LocalArgs& a, int fid, cudaStream_t st) {
-  return a.inner_tol2 > 0.0 ? launch_fid_a<BW, R, TR, CL, true>(a, fid, st)
-                            : launch_fid_a<BW, R, TR, CL, false>(a, fid, st);
-}
-
-template <int BW, int R, int TR, int CL, int FID, bool MASK>
+template <int BW, int R, int TR, int CL, int FID, bool MASK, bool ADAPT>
 cudaError_t prepare_one() {
-  using L = SmemLayout<BW, R, TR>;
-  cudaError_t e = cudaFuncSetAttribute(k_fused<BW, R, TR, CL, FID, MASK, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_fused<BW, R, TR, CL, FID, MASK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)L::BYTES);
+  return cudaFuncSetAttribute(k_fused<BW, R, TR, CL, FID, MASK, ADAPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)SmemLayout<BW, R, TR>::BYTES);
 }
 
-template <int BW, int R, int TR, int CL>
+template <int BW, int R, int TR, int CL, bool ADAPT>
 cudaError_t prepare_fid() {
   cudaError_t e;
-  if ((e = prepare_one<BW, R, TR, CL, FID_L2, false>()) != cudaSuccess) return e;
-  if ((e = prepare_one<BW, R, TR, CL, FID_L2, true>()) != cudaSuccess) return e;
-  if ((e = prepare_one<BW, R, TR, CL, FID_L1, false>()) != cudaSuccess) return e;
-  if ((e = prepare_one<BW, R, TR, CL, FID_L1, true>()) != cudaSuccess) return e;
-  return prepare_one<BW, R, TR, CL, FID_SEG, false>();
+  if ((e = prepare_one<BW, R, TR, CL, FID_L2, false, ADAPT>()) != cudaSuccess) return e;
+  if ((e = prepare_one<BW, R, TR, CL, FID_L2, true, ADAPT>()) != cudaSuccess) return e;
+  if ((e = prepare_one<BW, R, TR, CL, FID_L1, false, ADAPT>()) != cudaSuccess) return e;
+  if ((e = prepare_one<BW, R, TR, CL, FID_L1, true, ADAPT>()) != cudaSuccess) return e;
+  return prepare_one<BW, R, TR, CL, FID_SEG, false, ADAPT>();
 }
 
-// index into kConfigs for a tile shape, -1 if none fits
+// The micro-tile kernel (fused_tile.cuh) for every subdomain shape up to 128 x 128, with
+// a fixed inner count.  Columns choose the lanes of a row group (a subdomain of mc
+// columns in a block of 32, 64 or 128), rows the warps of a CTA and the CTAs of a
+// cluster.  Up to 32 x 32 and 64 x 64 one CTA holds the subdomain: no halo leaves the
+// SM.  In a cluster of two 32-row CTAs, 64 x 64 subdomains take 256 us per outer
+// iteration of 10 inner ones at 4096^2 and 14.1 us at 128^2, in one CTA 217 and 13.0.
+cudaError_t launch_tile_shape(const LocalArgs& a, int mr, int mc, int fid, cudaStream_t st) {
+  auto go = [&](cudaError_t (*launch)(const LocalArgs&, int, int, bool, cudaStream_t), int bw, int band) {
+    const int cl = (mr + band - 1) / band;
+    const bool pad = a.g.W != bw * a.g.NC || a.g.H != cl * band * a.g.NR;
+    return launch(a, fid, cl, pad, st);
+  };
+  if (mr < 1 || mc < 1 || mr > 128 || mc > 128) return cudaErrorInvalidValue;
+  if (mc <= 32) return mr <= 32 ? go(launch_tile_8_2, 32, 32) : go(launch_tile_8_4, 32, 64);
+  if (mc <= 64) return mr > 32 && mr <= 64 ? go(launch_tile_16_8, 64, 64) : go(launch_tile_16_4, 64, 32);
+  return go(launch_tile_32_4, 128, 16);
+}
+
+// size class of the cluster-barrier kernel for a tile shape (up to 32 x 32, 64 x 64 and
+// 128 x 128), -1 if none fits
 int pick(int mr, int mc) {
   if (mc <= 32 && mr <= 32) return 0;
   if (mc <= 64 && mr <= 64) return 1;
@@ -444,27 +428,17 @@ void fused_max_tile(int* rows, int* cols) {
 
 int fused_num_variants() { return kNumVariants; }
 
-const char* fused_config_name(int mr, int mc, int variant) {
-  if (mr == 128 && mc == 128) {
-    switch (variant) {
-      case 0: return "mt4_tma";
-      case 1: return "mt4_cp_async";
-      case 2: return "mt2x4";
-      default: break;
-    }
-  }
-  const int q = pick(mr, mc);
-  return q < 0 ? "none" : kConfigs[q].name;
-}
-
 cudaError_t fused_prepare() {
   cudaError_t e;
-  if ((e = prepare_fid<32, 8, 4, 1>()) != cudaSuccess) return e;
-  if ((e = prepare_fid<64, 8, 8, 1>()) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_fused_tile_batch<64, 8, 8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)SmemLayout<64, 8, 8>::BYTES)) != cudaSuccess)
-    return e;
-  if ((e = prepare_fid<128, 8, 2, 8>()) != cudaSuccess) return e;
+  if ((e = prepare_fid<32, 8, 4, 1, true>()) != cudaSuccess) return e;
+  if ((e = prepare_fid<64, 8, 8, 1, true>()) != cudaSuccess) return e;
+  if ((e = prepare_fid<128, 8, 2, 8, true>()) != cudaSuccess) return e;
+  if ((e = prepare_fid<128, 8, 2, 8, false>()) != cudaSuccess) return e;
+  if ((e = prepare_tile_8_2()) != cudaSuccess) return e;
+  if ((e = prepare_tile_8_4()) != cudaSuccess) return e;
+  if ((e = prepare_tile_16_4()) != cudaSuccess) return e;
+  if ((e = prepare_tile_16_8()) != cudaSuccess) return e;
+  if ((e = prepare_tile_32_4()) != cudaSuccess) return e;
   if ((e = fused_mt_prepare()) != cudaSuccess) return e;
   return fused_mt4_prepare();
 }
@@ -473,10 +447,7 @@ cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, in
   if (tile == 128)  // variant 0: 4 x 4 micro-tiles (K within its shared coefficient table); 2: 2 x 4
     return variant == 0 && K <= fused_mt4_max_inner() ? launch_fused_mt4_batch(B, total_tiles, st)
                                                        : launch_fused_mt_batch(B, total_tiles, st);
-  if (tile != 64) return cudaErrorInvalidValue;
-  // 64 x 64 subdomains: one CTA of 64 x 8 threads per subdomain
-  k_fused_tile_batch<64, 8, 8, 1><<<dim3(1, total_tiles, 1), dim3(64, 8, 1), SmemLayout<64, 8, 8>::BYTES, st>>>(B);
-  return cudaGetLastError();
+  return tile == 64 ? launch_tile_batch_64(B, total_tiles, st) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStream_t st) {
@@ -501,10 +472,12 @@ cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStr
       default: break;
     }
   }
+  if (a.inner_tol2 <= 0.0)  // exact 128 x 128 subdomains: variant 3, or arrays the kernels above cannot take
+    return exact128 ? launch_fid<128, 8, 2, 8, false>(a, fid, st) : launch_tile_shape(a, mr, mc, fid, st);
   switch (pick(mr, mc)) {
-    case 0: return launch_fid<32, 8, 4, 1>(a, fid, st);
-    case 1: return launch_fid<64, 8, 8, 1>(a, fid, st);
-    case 2: return launch_fid<128, 8, 2, 8>(a, fid, st);
+    case 0: return launch_fid<32, 8, 4, 1, true>(a, fid, st);
+    case 1: return launch_fid<64, 8, 8, 1, true>(a, fid, st);
+    case 2: return launch_fid<128, 8, 2, 8, true>(a, fid, st);
     default: return cudaErrorInvalidValue;
   }
 }
