@@ -22,16 +22,19 @@
 // the right and at the bottom.  u is pinned to 0 in the first padding column and row, so
 // the dof on the left edge of that column is the subdomain's right side (D_s u = -u of
 // the last column) and the dof on the top edge of that row its bottom side, updated as
-// any other dof; what lies further out is never read by a pixel of the subdomain.  Where
+// any other dof; what lies further out is never read by a pixel of the subdomain.  (The
+// lane that holds the column or row branches on its place in the micro-tile; as selects the
+// pinning cost half as many instructions again as the iteration.)  Where
 // the subdomain fills the block (no padding) the sides are updated by lanes of other
 // warps, as in kernels_fused_mt4.cu.  A side on the image boundary is kept at 0 by
 // clamping its dofs to [-0, 0].
 //
 // Measured per outer iteration of 10 inner ones, multiplier update included, against
 // the cluster-barrier kernel (a column of 8 pixels per thread) it replaces here: 1080 x
-// 1920 in 120 x 128 subdomains 106 -> 44 us, 2160 x 3840 448 -> 160, 2999 x 3001 in 125 x
-// 125/126 477 -> 182, 4096 x 4096 in 64 x 64 572 -> 217 and in 32 x 32 527 -> 211, 128 x
-// 128 in 64 x 64 21.1 -> 13.0, 321 x 481 in 107 x 120/121 25.8 -> 17.0.
+// 1920 in 120 x 128 subdomains 106 -> 43 us, 2160 x 3840 448 -> 150, 2999 x 3001 in 125 x
+// 125/126 477 -> 176, 4096 x 4096 in 64 x 64 572 -> 217 and in 32 x 32 527 -> 211, 512 x 512
+// in 32 x 32 19.1 -> 10.6, 128 x 128 in 64 x 64 21.1 -> 12.9, 321 x 481 in 107 x 120/121
+// 25.8 -> 17.5.
 //
 // Every value is computed with the operations of the scalar iteration in its order
 // (pointwise.cuh), so the results are those of the plain path bit for bit.
@@ -71,6 +74,15 @@ struct TileLayout {
                 "16-byte alignment of the vector accesses");
   static_assert(kRightThread + BAND <= NT, "a thread per right-side dof");
 };
+
+// four consecutive floats (16-byte aligned)
+__device__ __forceinline__ void load4(const float* p, float* v) {
+  const float4 x = *reinterpret_cast<const float4*>(p);
+  v[0] = x.x;
+  v[1] = x.y;
+  v[2] = x.z;
+  v[3] = x.w;
+}
 
 // four consecutive floats of a row, the first n valid (n <= 0: none), the rest 0
 __device__ __forceinline__ void load4(const float* p, int n, bool vec, float* v) {
@@ -158,17 +170,13 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     __syncthreads();
     cluster_arrive<true>();  // matched before the first halo is sent: the loads hide the wait
   }
-  // clamp limits of the dofs of row r / column c: 0 on an image-boundary side
-  float lim1[4], lim2[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    lim1[q] = (q == 0 && i0 == 0 && !s_top) || (PAD && i0 + q == mr && !s_bot) ? 0.f : 1.f;
-    lim2[q] = (q == 0 && j0 == 0 && !s_lft) || (PAD && j0 + q == mc && !s_rgt) ? 0.f : 1.f;
-  }
-  if (!PAD) {
-#pragma unroll
-    for (int q = 1; q < 4; ++q) lim1[q] = lim2[q] = 1.f;
-  }
+  // the first padding column and row, if this lane holds them
+  const bool pad_c = PAD && !fill_c && (mc >> 2) == cl;
+  const bool pad_r = PAD && !fill_r && mr >= rank * BAND && ((mr - rank * BAND) >> 2) == G;
+  const int cpad = mc & 3, rpad = mr & 3;  // where in the lane's 4 x 4 pixels
+  // clamp limits of the dofs of the lane's first row / column: 0 on an image-boundary side
+  const float lim_top = (i0 == 0 && !s_top) || (pad_r && rpad == 0 && !s_bot) ? 0.f : 1.f;
+  const float lim_left = (j0 == 0 && !s_lft) || (pad_c && cpad == 0 && !s_rgt) ? 0.f : 1.f;
 
   // pairs [column c][e]: rows (e, e + 2) of column j0 + c
   f32x2 U[4][2], P1[4][2], P2[4][2], Q1[4][2], Q2[4][2];
@@ -180,21 +188,42 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     const bool vec = (g.W & 3) == 0 && (c0 & 3) == 0;
     float h1[4][4], h2[4][4], fv[4][4];
     float u[4][4], p1[4][4], p2[4][4];
+    const float* gu = A.u + (size_t)(r0 + i0) * g.W + c0 + j0;
+    const float* gf = A.f + (size_t)(r0 + i0) * g.W + c0 + j0;
+    const float* g1 = A.P1 + (size_t)(r0 + i0 + a) * g.W + c0 + j0;
+    const float* g2 = A.P2 + (size_t)(r0 + i0) * W2 + c0 + b + j0;
+    // every load in flight before the first is used: one latency, not one per array
+    if (vec && i0 + 3 < mr && j0 + 3 < mc) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int i = i0 + r, gi = r0 + i;
-      const int n = i < mr ? mc - j0 : 0;                                // pixels of this lane's row
-      const int n1 = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;             // p1 dofs (row mr: the bottom side)
-      const int n2 = i < mr ? mc + (s_rgt ? 1 : 0) - j0 : 0;             // p2 dofs (column mc: the right side)
-      load4(A.u + (size_t)gi * g.W + c0 + j0, n, vec, u[r]);
-      load4(A.f + (size_t)gi * g.W + c0 + j0, n, vec, fv[r]);
-      load4(A.P1 + (size_t)(gi + a) * g.W + c0 + j0, n1, vec, p1[r]);
-      load4(A.P2 + (size_t)gi * W2 + c0 + b + j0, n2, false, p2[r]);
-      if (MASK) {
+      for (int r = 0; r < 4; ++r) {
+        load4(gu + (size_t)r * g.W, u[r]);
+        load4(gf + (size_t)r * g.W, fv[r]);
+        load4(g1 + (size_t)r * g.W, p1[r]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) p2[r][c] = g2[(size_t)r * W2 + c];
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int i = i0 + r;
+        const int n = i < mr ? mc - j0 : 0;                                // pixels of this lane's row
+        const int n1 = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;             // p1 dofs (row mr: the bottom side)
+        const int n2 = i < mr ? mc + (s_rgt ? 1 : 0) - j0 : 0;             // p2 dofs (column mc: the right side)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          u[r][c] = c < n ? gu[(size_t)r * g.W + c] : 0.f;
+          fv[r][c] = c < n ? gf[(size_t)r * g.W + c] : 0.f;
+          p1[r][c] = c < n1 ? g1[(size_t)r * g.W + c] : 0.f;
+          p2[r][c] = c < n2 ? g2[(size_t)r * W2 + c] : 0.f;
+        }
+      }
+    }
+    if (MASK) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-          if (c < n && A.mask[(size_t)gi * g.W + c0 + j0 + c]) in_d |= 1u << (4 * c + r);
-      }
+          if (i0 + r < mr && j0 + c < mc && A.mask[(size_t)(r0 + i0 + r) * g.W + c0 + j0 + c]) in_d |= 1u << (4 * c + r);
     }
     if (right_lane) {
       const int gi = r0 + rank * BAND + rr;
@@ -268,12 +297,6 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     ++phQ;
     if (cl == 0) mbar_arrive_expect_tx(mbQ, kHaloBytes);
   };
-  // the padding column and row whose u is pinned: columns j0 .. j0 + 3 hold column mc at
-  // mc & 3 if this lane is the one, rows likewise
-  const bool pin_c = PAD && !fill_c && (mc >> 2) == cl;
-  const bool pin_r = PAD && !fill_r && ((mr - rank * BAND) >> 2) == G && mr >= rank * BAND;
-  const int cpad = mc & 3, rpad = mr & 3;
-
 #pragma unroll 2
   for (int k = 0; k < K; ++k) {
     f32x2 SIG, UA, UBc, PA, PC, PB, TH, SS;
@@ -325,15 +348,26 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
           U[c][e] = un;
         }
       }
-      if (PAD) {
+      // u of the first padding column and row: 0 where the side is an interface (D_s u =
+      // -u), u of the pixel before it where it is the image boundary (D_s u = 0: the dof
+      // stays 0; in the lane's first column or row the clamp limit does that)
+      if (PAD && pad_c) {
+        auto pin = [&](int q) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (pin_c && cpad == q) U[q][0] = U[q][1] = 0ull;
-          if (pin_r && rpad == q) {
-            const int e = q & 1;
+          for (int e = 0; e < 2; ++e) U[q][e] = s_rgt || q == 0 ? 0ull : U[q > 0 ? q - 1 : 0][e];
+        };
+        if (cpad == 0) pin(0);
+        else if (cpad == 1) pin(1);
+        else if (cpad == 2) pin(2);
+        else pin(3);
+      }
+      if (PAD && pad_r) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) U[c][e] = q < 2 ? pk2(0.f, hi2(U[c][e])) : pk2(lo2(U[c][e]), 0.f);
-          }
+        for (int c = 0; c < 4; ++c) {
+          if (rpad == 0) U[c][0] = pk2(0.f, hi2(U[c][0]));
+          else if (rpad == 1) U[c][1] = pk2(s_bot ? 0.f : lo2(U[c][0]), hi2(U[c][1]));
+          else if (rpad == 2) U[c][0] = pk2(lo2(U[c][0]), s_bot ? 0.f : lo2(U[c][1]));
+          else U[c][1] = pk2(lo2(U[c][1]), s_bot ? 0.f : hi2(U[c][0]));
         }
       }
       const float4 ul = make_float4(hi2(U[0][1]), hi2(U[1][1]), hi2(U[2][1]), hi2(U[3][1]));
@@ -357,7 +391,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         H0[c] = mul2(PB, h1.x);
         {
           const f32x2 tt = fma2(PC, sub2(U[c][1], U[c][0]), fma2(PA, P1[c][1], mul2(PB, h1.y)));  // p_target
-          const f32x2 pn = pk2(clamp_abs(lo2(tt), lim1[1]), clamp_abs(hi2(tt), lim1[3]));
+          const f32x2 pn = pk2(clamp_abs(lo2(tt), 1.f), clamp_abs(hi2(tt), 1.f));
           Q1[c][1] = fma2(TH, sub2(pn, P1[c][1]), pn);
           P1[c][1] = pn;
         }
@@ -365,7 +399,8 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         for (int e = 0; e < 2; ++e) {
           const f32x2 leftu = c > 0 ? U[c - 1][e] : (e == 0 ? ul.x : ul.y);
           const f32x2 tt = fma2(PC, sub2(U[c][e], leftu), fma2(PA, P2[c][e], mul2(PB, e == 0 ? h2.x : h2.y)));
-          const f32x2 pn = pk2(clamp_abs(lo2(tt), lim2[c]), clamp_abs(hi2(tt), lim2[c]));
+          const float ll = c == 0 ? lim_left : 1.f;
+          const f32x2 pn = pk2(clamp_abs(lo2(tt), ll), clamp_abs(hi2(tt), ll));
           Q2[c][e] = fma2(TH, sub2(pn, P2[c][e]), pn);
           P2[c][e] = pn;
         }
@@ -379,7 +414,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         // rows (0, 2): the rows above (-1, 1) straddle the group above and pair 1
         const f32x2 du = pk2(lo2(U[c][0]) - uav[c], hi2(U[c][0]) - lo2(U[c][1]));
         const f32x2 tt = fma2(PC, du, fma2(PA, P1[c][0], H0[c]));
-        const f32x2 pn = pk2(clamp_abs(lo2(tt), lim1[0]), clamp_abs(hi2(tt), lim1[2]));
+        const f32x2 pn = pk2(clamp_abs(lo2(tt), lim_top), clamp_abs(hi2(tt), 1.f));
         Q1[c][0] = fma2(TH, sub2(pn, P1[c][0]), pn);
         P1[c][0] = pn;
       }

@@ -86,12 +86,15 @@ __device__ __forceinline__ float phat_s(float p, float lam, float tau) { return 
 __device__ __forceinline__ float phat_t(float p, float lam, float tau) { return fmaf(tau, lam, p); }
 
 // first pixel row (column) of tile a when len pixels are split into n tiles
+// (0 <= a <= n <= len; the 64-bit division a long axis needs is some hundred instructions)
 __host__ __device__ __forceinline__ int part_start(int a, int len, int n) {
+  if (len < 65536) return (int)((unsigned)a * (unsigned)len / (unsigned)n);
   return (int)(((long long)a * len) / n);
 }
 
 // the tile that pixel row (column) i belongs to
 __host__ __device__ __forceinline__ int part_of(int i, int len, int n) {
+  if (len < 65536) return (int)(((unsigned)(i + 1) * (unsigned)n - 1u) / (unsigned)len);
   return (int)(((long long)(i + 1) * n - 1) / len);
 }
 
