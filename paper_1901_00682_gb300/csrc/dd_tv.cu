@@ -79,6 +79,10 @@ struct dd_tv {
   Coef* coef = nullptr;
   // plain path: phat and pbar; full-dimension path: pbar (carried across iterations)
   float *Ph1 = nullptr, *Ph2 = nullptr, *Pb1 = nullptr, *Pb2 = nullptr;
+  // full-dimension path: the two sets its launches go back and forth between (u, P1, ...
+  // above point into the one that holds the current iterate); full_mem is set 1
+  FullSet full[2] = {};
+  float* full_mem = nullptr;
   double* partials = nullptr;
   unsigned int* counter = nullptr;
   double* red_out = nullptr;
@@ -259,12 +263,39 @@ struct PhaseMark {
   }
 };
 
+// Full-dimension path: launches of one outer iteration (of inner_iters iterations).
+int full_launches(const dd_tv* h) { return (h->p.inner_iters + full_max_steps() - 1) / full_max_steps(); }
+
+// Points the handle's state at the set that holds iterate h->n (set 0 at n = 0, the other
+// one after every launch).
+void full_select(dd_tv* h) {
+  if (!h->full_mem) return;
+  const FullSet& s = h->full[h->n & full_launches(h) & 1];
+  h->u = s.u;
+  h->P1 = s.P1;
+  h->P2 = s.P2;
+  h->Pb1 = s.Pb1;
+  h->Pb2 = s.Pb2;
+}
+
 // One outer iteration starting from parity `par` (= n mod 2): the strips of p~^n are
 // in set par, those of p~^{n-1} in set 1 - par, and p~^{n+1}'s go to set 1 - par.
 cudaError_t outer_once(dd_tv* h, int par) {
   cudaError_t e;
   const cudaStream_t st = h->stream;
-  if (h->p.path == DD_TV_PATH_FULLDIM) {
+  if (h->p.path == DD_TV_PATH_FULLDIM && h->full_mem) {
+    const int L = full_launches(h), K = h->p.inner_iters;
+    PhaseMark m(h, 1, L);
+    int cur = par & L & 1;
+    for (int q = 0; q < L; ++q, cur ^= 1) {
+      const int n = (int)((long long)(q + 1) * K / L - (long long)q * K / L);
+      const FullArgs a{h->g.H, h->g.W, (float)h->p.c1, (float)h->p.c2, h->f, h->has_mask ? h->mask : nullptr,
+                       h->coef, h->flag, h->full[cur], h->full[1 - cur]};
+      if ((e = launch_full(a, h->fid, n, st)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+  if (h->p.path == DD_TV_PATH_FULLDIM) {  // no room for the second set: a launch per half-step, in place
     LocalArgs a = local_args(h, 0);
     PhaseMark m(h, 1, 2 * a.K);
     for (int k = 0; k < a.K; ++k) {
@@ -344,12 +375,15 @@ int run_outer(dd_tv* h, int count) {
       h->n += 1;
       done += 1;
     }
+    full_select(h);
   }
   return DD_TV_OK;
 }
 
 int reset_state(dd_tv* h) {
   const cudaStream_t st = h->stream;
+  h->n = 0;
+  full_select(h);
   CK(launch_init_u(h->g, h->fid, h->f, h->has_mask ? h->mask : nullptr, h->u, st));
   CK(cudaMemsetAsync(h->P1, 0, h->n1 * sizeof(float), st));
   CK(cudaMemsetAsync(h->P2, 0, h->n2 * sizeof(float), st));
@@ -363,7 +397,6 @@ int reset_state(dd_tv* h) {
   CK(cudaMemsetAsync(h->inner_used, 0, (size_t)h->g.NR * h->g.NC * sizeof(int), st));
   CK(cudaMemsetAsync(h->inner_max, 0, sizeof(int), st));
   CK(cudaMemsetAsync(h->inner_work, 0, sizeof(unsigned long long), st));
-  h->n = 0;
   h->loaded = true;
   return DD_TV_OK;
 }
@@ -840,6 +873,26 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
       return rc;
     }
   }
+  if (p->path == DD_TV_PATH_FULLDIM) {
+    // the second set, every array on a 256-byte boundary; without room for it the path
+    // runs a launch per half-step in place
+    auto up = [](size_t n) { return (n + 63) & ~(size_t)63; };
+    const size_t n = up(h->npx) + 2 * up(h->n1) + 2 * up(h->n2);
+    if (cudaMalloc((void**)&h->full_mem, n * sizeof(float)) != cudaSuccess ||
+        cudaMemset(h->full_mem, 0, n * sizeof(float)) != cudaSuccess || full_prepare() != cudaSuccess) {
+      cudaGetLastError();
+      if (h->full_mem) cudaFree(h->full_mem);
+      h->full_mem = nullptr;
+    } else {
+      float* m = h->full_mem;
+      h->full[0] = FullSet{h->u, h->P1, h->P2, h->Pb1, h->Pb2};
+      h->full[1].u = m;
+      h->full[1].P1 = m += up(h->npx);
+      h->full[1].P2 = m += up(h->n1);
+      h->full[1].Pb1 = m += up(h->n2);
+      h->full[1].Pb2 = m += up(h->n1);
+    }
+  }
   if (p->path == DD_TV_PATH_PLAIN) {
     if ((rc = dalloc(h, &h->Ph1, h->n1)) || (rc = dalloc(h, &h->Ph2, h->n2))) {
       dd_tv_destroy(h);
@@ -896,6 +949,11 @@ int dd_tv_destroy(dd_tv* h) {
   drop_graphs(h);
   adj_free(h->adj);
   h->adj = nullptr;
+  if (h->full_mem) {  // u, P1, ... back to the arrays allocated one by one
+    h->n = 0;
+    full_select(h);
+    cudaFree(h->full_mem);
+  }
   for (auto& m : h->marks) {
     cudaEventDestroy(m.a);
     cudaEventDestroy(m.b);
@@ -1022,12 +1080,13 @@ int dd_tv_set_state(dd_tv* h, const float* u, const float* P1, const float* P2, 
   if (outer_count < 0) return fail(h, DD_TV_EINVAL, "outer_count must be >= 0");
   const cudaStream_t st = h->stream;
   const auto D2D = cudaMemcpyDeviceToDevice;
+  h->n = outer_count;
+  full_select(h);
   CK(cudaMemcpyAsync(h->u, u, h->npx * sizeof(float), D2D, st));
   CK(cudaMemcpyAsync(h->P1, P1, h->n1 * sizeof(float), D2D, st));
   CK(cudaMemcpyAsync(h->P2, P2, h->n2 * sizeof(float), D2D, st));
   if (h->nh) CK(cudaMemcpyAsync(h->lamh, lamh, h->nh * sizeof(float), D2D, st));
   if (h->nv) CK(cudaMemcpyAsync(h->lamv, lamv, h->nv * sizeof(float), D2D, st));
-  h->n = outer_count;
   if (h->p.path == DD_TV_PATH_FULLDIM) {
     CK(cudaMemcpyAsync(h->Pb1, P1prev, h->n1 * sizeof(float), D2D, st));
     CK(cudaMemcpyAsync(h->Pb2, P2prev, h->n2 * sizeof(float), D2D, st));

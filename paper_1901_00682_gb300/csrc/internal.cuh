@@ -51,6 +51,22 @@ struct LocalArgs {
   unsigned long long* inner_work;  // running sum of tile pixels x inner iterations
 };
 
+// One set of the full-dimension path's state: u, p and the extrapolated pbar.
+struct FullSet {
+  float *u, *P1, *P2, *Pb1, *Pb2;  // H x W, (H + 1) x W, H x (W + 1), pbar likewise
+};
+
+// Arguments of one launch of full-dimension iterations (constant steps: coef[0]).
+struct FullArgs {
+  int H, W;
+  float c1, c2;
+  const float* f;
+  const uint8_t* mask;   // or nullptr
+  const Coef* coef;
+  int* err;
+  FullSet in, out;       // distinct arrays
+};
+
 // Batch of images solved together (every image partitioned into exact 128 x 128
 // subdomains).  Device arrays, one entry per image unless stated otherwise.
 struct BatchArgs {
@@ -161,6 +177,13 @@ cudaError_t prepare_tile_16_8();
 cudaError_t prepare_tile_32_4();
 // every 64 x 64 subdomain of every image of a batch (launch_tile_16_8's kernel)
 cudaError_t launch_tile_batch_64(const BatchArgs& B, int total_tiles, cudaStream_t st);
+
+// ---- kernels_full.cu
+// n <= full_max_steps() full-dimension iterations in one launch, a.in -> a.out (the dofs of
+// the image boundary are 0 and not written)
+cudaError_t launch_full(const FullArgs& a, int fidelity, int n, cudaStream_t st);
+int full_max_steps();
+cudaError_t full_prepare();
 
 // ---- kernels_plain.cu
 // phat = p~ -+ tau lambda on the interface sides, pbar = p~; full arrays.
