@@ -82,11 +82,11 @@ typedef struct {
   int energy_every;       /* with outer_tol: evaluate J every energy_every outer iterations  */
   int path;               /* dd_tv_path                                                    */
   int variant;            /* fused path, hardware mapping of exact 128 x 128 subdomains:
-                             0 persistent 4 x 4 micro-tiles, state moved by tensor
-                             copies (default); 1 the same with cp.async copies; 2
-                             persistent 2 x 4 micro-tiles; 3 one cluster per subdomain
-                             with cluster barriers (the kernel of every other tile
-                             shape).  The arithmetic and results do not depend on it  */
+                             0 the micro-tile kernel of every other tile shape
+                             (default); 1 persistent 4 x 4 micro-tiles, state moved by
+                             tensor copies; 2 persistent 2 x 4 micro-tiles; 3 one
+                             cluster per subdomain with cluster barriers.  The
+                             arithmetic and results do not depend on it               */
   double inner_tol;       /* >= 0.  0: every local solve runs inner_iters iterations.  > 0:
                              adaptive inner stopping (Section 5, eq. stop_inner1): a
                              subdomain stops after the first inner iteration k with
@@ -303,9 +303,8 @@ int dd_tv_shard_energy(dd_tv* h, const float* row_below_dev, double* J_out);
  * the subdomain size, the number of inner iterations and the initial inner steps, and
  * advance by the same number of outer iterations.  One outer iteration of the whole
  * batch is two kernel launches (multiplier update of every interface of every image,
- * then the local solves of every subdomain of every image: by default a persistent
- * kernel whose clusters walk the batch's work list of (image, subdomain) pairs with
- * each image's fidelity and parameters).  dd_tv_batch_iterate(b, n) with n > 1 is one
+ * then the local solves of every subdomain of every image, the batch's work list of
+ * (image, subdomain) pairs with each image's fidelity and parameters).  dd_tv_batch_iterate(b, n) with n > 1 is one
  * CUDA-graph launch of the n outer iterations (the graph is captured on the first call
  * with that n and start parity and replayed by later ones).
  * Image sides must be multiples of the subdomain side (64 or 128).  Results are
@@ -321,14 +320,14 @@ typedef struct {
 } dd_tv_batch_image;
 
 typedef struct {
-  int tile;               /* subdomain side: 128 (persistent clusters over the work
-                             list, see variant) or 64 (one CTA per subdomain); other
-                             sides return DD_TV_EUNSUPPORTED                            */
+  int tile;               /* subdomain side: 128 or 64; other sides return
+                             DD_TV_EUNSUPPORTED                                         */
   int inner_iters;        /* 1..DD_TV_MAX_INNER                                        */
   double tau0, sigma0;    /* initial inner steps (Section 5: 10 and 1/80)               */
-  int variant;            /* 0: 4 x 4 pixel micro-tiles per thread (2 x 4 when
-                             inner_iters > 64); 2 (tile 128 only): 2 x 4 micro-tiles.
-                             Both give the same bits; anything else: DD_TV_EINVAL      */
+  int variant;            /* 0: 4 x 4 pixel micro-tiles per thread, one cluster (tile
+                             128) or CTA (64) per subdomain; 2 (tile 128 only):
+                             persistent 2 x 4 micro-tiles.  Both give the same bits;
+                             anything else: DD_TV_EINVAL                               */
 } dd_tv_batch_params;
 
 /* Validates and allocates the batch (images[n], n >= 1); *out = NULL on error. */

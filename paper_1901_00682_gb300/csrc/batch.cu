@@ -108,7 +108,7 @@ cudaError_t outer_once(dd_tv_batch* b, int par) {
   ba.tile_img = b->d_tile_img;
   ba.tile_base = b->d_tile_base;
   ba.write_set = 1 - par;
-  return launch_fused_batch(ba, b->total_tiles, b->p.tile, b->p.variant, b->p.inner_iters, b->stream);
+  return launch_fused_batch(ba, b->total_tiles, b->p.tile, b->p.variant, b->total4 > 0, b->stream);
 }
 
 void drop_batch_graphs(dd_tv_batch* b) {

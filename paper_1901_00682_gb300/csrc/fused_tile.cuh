@@ -1,5 +1,4 @@
-// Fused local solver on 4 x 4 micro-tiles for subdomains of any shape up to 128 x 128
-// (the kernel of every subdomain that is not exactly 128 x 128).
+// Fused local solver on 4 x 4 micro-tiles for subdomains of any shape up to 128 x 128.
 //
 // What bounds the local solve is latency and issue slots, not memory: a subdomain
 // lives on chip for its whole inner loop, so the time of an inner iteration is the
@@ -30,11 +29,13 @@
 // clamping its dofs to [-0, 0].
 //
 // Measured per outer iteration of 10 inner ones, multiplier update included, against
-// the cluster-barrier kernel (a column of 8 pixels per thread) it replaces here: 1080 x
-// 1920 in 120 x 128 subdomains 106 -> 43 us, 2160 x 3840 448 -> 150, 2999 x 3001 in 125 x
-// 125/126 477 -> 176, 4096 x 4096 in 64 x 64 572 -> 217 and in 32 x 32 527 -> 211, 512 x 512
-// in 32 x 32 19.1 -> 10.6, 128 x 128 in 64 x 64 21.1 -> 12.9, 321 x 481 in 107 x 120/121
-// 25.8 -> 17.5.
+// the kernels it replaced (the cluster-barrier kernel, a column of 8 pixels per thread;
+// for exact 128 x 128 subdomains the persistent kernel of kernels_fused_mt4.cu): 1080 x 1920
+// in 120 x 128 subdomains 106 -> 41 us, 2160 x 3840 448 -> 137, 2999 x 3001 in 125 x 125/126
+// 477 -> 158, 4096 x 4096 in 64 x 64 572 -> 214 and in 32 x 32 527 -> 187, 512 x 512 in 32 x 32
+// 19.1 -> 8.9, 128 x 128 in 64 x 64 21.1 -> 11.9, 321 x 481 in 107 x 120/121 25.8 -> 14.5; in 128 x
+// 128 subdomains 512 x 512 14.0 -> 13.0, 1024 x 1024 22.7 -> 18.6, 4096 x 4096 231 -> 216, a
+// batch of 64 images (168 Mpixel) 2730 -> 2280.
 //
 // Every value is computed with the operations of the scalar iteration in its order
 // (pointwise.cuh), so the results are those of the plain path bit for bit.
@@ -111,11 +112,67 @@ __device__ __forceinline__ void store4(float* p, int n, bool vec, float a, float
 
 __device__ __forceinline__ float half_of(f32x2 v, int h) { return h ? hi2(v) : lo2(v); }
 
+// Stores the subdomain's u, p1, p2 and sides.
+template <int LPR, int NW, bool PAD>
+__device__ __forceinline__ void tile_store(const LocalArgs& A, const Strips& out, int a, int b, int tid, int CL, int rank,
+                                           const f32x2 (&U)[4][2], const f32x2 (&P1)[4][2], const f32x2 (&P2)[4][2],
+                                           float pr_s) {
+  using L = TileLayout<LPR, NW>;
+  constexpr int BAND = L::BAND, BW = L::BW;
+  extern __shared__ __align__(128) float smem[];
+  const Grid g = A.g;
+  const int r0 = PAD ? part_start(a, g.H, g.NR) : a * CL * BAND, mr = PAD ? part_start(a + 1, g.H, g.NR) - r0 : CL * BAND;
+  const int c0 = PAD ? part_start(b, g.W, g.NC) : b * BW, mc = PAD ? part_start(b + 1, g.W, g.NC) - c0 : BW;
+  const bool s_top = a > 0 || g.cut_top, s_bot = a + 1 < g.NR || g.cut_bot, s_lft = b > 0, s_rgt = b + 1 < g.NC;
+  const bool fill_c = !PAD || mc == BW, fill_r = !PAD || mr == CL * BAND;
+  const int w = tid >> 5, l = tid & 31, G = w * L::RG + l / LPR, j0 = 4 * (l % LPR), i0 = rank * BAND + 4 * G;
+  const int W2 = g.W + g.NC;
+  const int rr = tid - L::kRightThread;
+  const bool right_lane = fill_c && s_rgt && rr >= 0 && rr < BAND && rank * BAND + rr < mr;
+  const bool bottom_lane = fill_r && s_bot && rank == CL - 1 && w == L::kBottomWarp && l < LPR;
+  const bool vec = (g.W & 3) == 0 && (c0 & 3) == 0;
+  // the strips of a set start at multiples of the interface edges, not of 4 floats
+  const bool vec_t = vec && (reinterpret_cast<uintptr_t>(out.ST) & 15) == 0;
+  const bool vec_b = vec && (reinterpret_cast<uintptr_t>(out.SB) & 15) == 0;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int e = r & 1, h = r >> 1, i = i0 + r, gi = r0 + i;
+    const int n = i < mr ? mc - j0 : 0;
+    const int n1 = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;
+    const int n2 = i < mr ? mc + (s_rgt ? 1 : 0) - j0 : 0;
+    store4(A.u + (size_t)gi * g.W + c0 + j0, n, vec, half_of(U[0][e], h), half_of(U[1][e], h), half_of(U[2][e], h),
+           half_of(U[3][e], h));
+    const float q0 = half_of(P1[0][e], h), q1 = half_of(P1[1][e], h), q2 = half_of(P1[2][e], h), q3 = half_of(P1[3][e], h);
+    store4(A.P1 + (size_t)(gi + a) * g.W + c0 + j0, n1, vec, q0, q1, q2, q3);
+    if (r == 0 && i == 0 && s_top) store4(out.ST + (ptrdiff_t)(a - 1) * g.W + c0 + j0, n1, vec_t, q0, q1, q2, q3);
+    if (PAD && i == mr && s_bot) store4(out.SB + (size_t)a * g.W + c0 + j0, n1, vec_b, q0, q1, q2, q3);
+    store4(A.P2 + (size_t)gi * W2 + c0 + b + j0, n2, false, half_of(P2[0][e], h), half_of(P2[1][e], h),
+           half_of(P2[2][e], h), half_of(P2[3][e], h));
+    if (j0 == 0 && s_lft && i < mr) out.SL[(size_t)(b - 1) * g.H + gi] = half_of(P2[0][e], h);
+    if (PAD && s_rgt && i < mr) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (j0 + c == mc) out.SR[(size_t)b * g.H + gi] = half_of(P2[c][e], h);
+    }
+  }
+  if (right_lane) {
+    const int gi = r0 + rank * BAND + rr;
+    A.P2[(size_t)gi * W2 + c0 + BW + b] = pr_s;
+    out.SR[(size_t)b * g.H + gi] = pr_s;
+  }
+  if (bottom_lane) {
+    const float4 v = *reinterpret_cast<const float4*>(smem + L::PBS + j0);
+    store4(A.P1 + (size_t)(r0 + mr + a) * g.W + c0 + j0, mc - j0, vec, v.x, v.y, v.z, v.w);
+    store4(out.SB + (size_t)a * g.W + c0 + j0, mc - j0, vec_b, v.x, v.y, v.z, v.w);
+  }
+}
+
 // The local solve of subdomain (a, b) of the problem A, its interface strips written to
-// out.  CLU: the subdomain is a cluster of gridDim.x CTAs (else one CTA).  PAD: the
-// subdomain may be smaller than the block (false: every subdomain fills it).
+// out, by CTA rank of CL.  CLU: the subdomain is a cluster (else one CTA: rank 0 of 1).
+// PAD: the subdomain may be smaller than the block (false: every subdomain fills it).
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
-__device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out, const int a, const int b) {
+__device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out, const int a, const int b,
+                                           const int rank, const int CL) {
   using L = TileLayout<LPR, NW>;
   constexpr int NG = L::NG, BAND = L::BAND, BW = L::BW, NT = L::NT;
   extern __shared__ __align__(128) float smem[];
@@ -125,9 +182,8 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   const uint32_t mbU = smem_addr(smem + L::MB), mbQ = mbU + 8;
 
   const Grid g = A.g;
-  const int CL = CLU ? (int)gridDim.x : 1, rank = CLU ? (int)blockIdx.x : 0;
-  const int r0 = part_start(a, g.H, g.NR), mr = part_start(a + 1, g.H, g.NR) - r0;
-  const int c0 = part_start(b, g.W, g.NC), mc = part_start(b + 1, g.W, g.NC) - c0;
+  const int r0 = PAD ? part_start(a, g.H, g.NR) : a * CL * BAND, mr = PAD ? part_start(a + 1, g.H, g.NR) - r0 : CL * BAND;
+  const int c0 = PAD ? part_start(b, g.W, g.NC) : b * BW, mc = PAD ? part_start(b + 1, g.W, g.NC) - c0 : BW;
   const bool s_top = a > 0 || g.cut_top, s_bot = a + 1 < g.NR || g.cut_bot, s_lft = b > 0, s_rgt = b + 1 < g.NC;
   const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
   const int G = w * L::RG + l / LPR, cl = l % LPR;  // row group, lane of the group
@@ -149,15 +205,10 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   float* const myQL = smem + L::QL + G * L::SLOT + 4 * cl;
   float* const myF = smem + L::F + 4 * tid;  // column c at + c * 4 NT; the proximal centres likewise
   constexpr int kH1 = L::H1 - L::F, kH2 = L::H2 - L::F;
-  uint32_t remote_u = 0, remote_q1 = 0, remote_mbU = 0, remote_mbQ = 0;
-  if (push_down) {
-    remote_u = map_rank(smem_addr(sUB + j0), rank + 1);
-    remote_mbU = map_rank(mbU, rank + 1);
-  }
-  if (push_up) {
-    remote_q1 = map_rank(smem_addr(sQ1 + NG * BW + j0), rank - 1);
-    remote_mbQ = map_rank(mbQ, rank - 1);
-  }
+  // the neighbour's shared memory: every array lies where it does here
+  const uint32_t s0 = smem_addr(smem);
+  const uint32_t remote = push_down ? map_rank(s0, rank + 1) : (push_up ? map_rank(s0, rank - 1) : 0u);
+  pdl_trigger();
   if (CLU) {
     if (tid == 0) {
       mbar_init(mbU, 1);
@@ -183,7 +234,13 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   uint32_t in_d = 0;  // bit 4c + r: pixel (row r, column j0 + c) lies in the inpainting domain
   float pr_s = 0.f, hr_s = 0.f;
 
-  // ---- load the state, build the proximal centre
+  // ---- load the state, build the proximal centre.  Every load is in flight before the first
+  // is used: one latency, not one per array (the loads were 3.8 of 16 us per subdomain).
+  const bool coef_smem = K <= L::kMaxSmemCoef;
+  if (coef_smem)
+    for (int q = tid; q < 16 * K; q += NT)
+      cp_async4(sCo + q, reinterpret_cast<const float*>(A.coef) + (q >> 4) * 8 + ((q & 15) >> 1));
+  cp_async_commit();
   {
     const bool vec = (g.W & 3) == 0 && (c0 & 3) == 0;
     float h1[4][4], h2[4][4], fv[4][4];
@@ -192,13 +249,15 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     const float* gf = A.f + (size_t)(r0 + i0) * g.W + c0 + j0;
     const float* g1 = A.P1 + (size_t)(r0 + i0 + a) * g.W + c0 + j0;
     const float* g2 = A.P2 + (size_t)(r0 + i0) * W2 + c0 + b + j0;
-    // every load in flight before the first is used: one latency, not one per array
+    const uint8_t* gm = MASK ? A.mask + (size_t)(r0 + i0) * g.W + c0 + j0 : nullptr;
+    uint32_t mb[4] = {0, 0, 0, 0};  // mask bytes of the lane's rows
     if (vec && i0 + 3 < mr && j0 + 3 < mc) {
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         load4(gu + (size_t)r * g.W, u[r]);
         load4(gf + (size_t)r * g.W, fv[r]);
         load4(g1 + (size_t)r * g.W, p1[r]);
+        if (MASK) mb[r] = *reinterpret_cast<const uint32_t*>(gm + (size_t)r * g.W);
 #pragma unroll
         for (int c = 0; c < 4; ++c) p2[r][c] = g2[(size_t)r * W2 + c];
       }
@@ -215,34 +274,44 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
           fv[r][c] = c < n ? gf[(size_t)r * g.W + c] : 0.f;
           p1[r][c] = c < n1 ? g1[(size_t)r * g.W + c] : 0.f;
           p2[r][c] = c < n2 ? g2[(size_t)r * W2 + c] : 0.f;
+          if (MASK && c < n) mb[r] |= (uint32_t)gm[(size_t)r * g.W + c] << (8 * c);
         }
       }
     }
-    if (MASK) {
+    // pbar1 of the row below the band: the next CTA's first row (its halo of later
+    // iterations), the bottom side of a subdomain that fills the block, or 0
+    const int ib = rank * BAND + BAND;
+    const int nb = G == NG - 1 && ib < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;
+    const bool bottom_fill = last_group && fill_r && s_bot;
+    float qb[4], lb[4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+    for (int c = 0; c < 4; ++c) qb[c] = c < nb ? A.P1[(size_t)(r0 + ib + a) * g.W + c0 + j0 + c] : 0.f;
+    if (right_lane) pr_s = A.P2[(size_t)(r0 + rank * BAND + rr) * W2 + c0 + BW + b];
+
+    pdl_wait();  // the multipliers, of the sides this lane holds
+    const bool top = i0 == 0 && s_top, left = j0 == 0 && s_lft, bot = pad_r && s_bot, rgt = pad_c && s_rgt;
+    float lt[4], ll[4], lr[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (i0 + r < mr && j0 + c < mc && A.mask[(size_t)(r0 + i0 + r) * g.W + c0 + j0 + c]) in_d |= 1u << (4 * c + r);
+    for (int c = 0; c < 4; ++c) {
+      lt[c] = top && c < mc - j0 ? A.lamh[(ptrdiff_t)(a - 1) * g.W + c0 + j0 + c] : 0.f;
+      lb[c] = (bot || bottom_fill) && c < mc - j0 ? A.lamh[(size_t)a * g.W + c0 + j0 + c] : 0.f;
+      ll[c] = left && i0 + c < mr ? A.lamv[(size_t)(b - 1) * g.H + r0 + i0 + c] : 0.f;
+      lr[c] = rgt && i0 + c < mr ? A.lamv[(size_t)b * g.H + r0 + i0 + c] : 0.f;
     }
-    if (right_lane) {
-      const int gi = r0 + rank * BAND + rr;
-      pr_s = A.P2[(size_t)gi * W2 + c0 + BW + b];
-      hr_s = phat_s(pr_s, A.lamv[(size_t)b * g.H + gi], tau);
-    }
+    if (right_lane) hr_s = phat_s(pr_s, A.lamv[(size_t)b * g.H + r0 + rank * BAND + rr], tau);
+
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      const int i = i0 + r, gi = r0 + i;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const int j = j0 + c;
         h1[r][c] = p1[r][c];
         h2[r][c] = p2[r][c];
-        if (r == 0 && i == 0 && s_top && j < mc) h1[r][c] = phat_t(p1[r][c], A.lamh[(ptrdiff_t)(a - 1) * g.W + c0 + j], tau);
-        if (PAD && i == mr && s_bot && j < mc) h1[r][c] = phat_s(p1[r][c], A.lamh[(size_t)a * g.W + c0 + j], tau);
-        if (c == 0 && j == 0 && s_lft && i < mr) h2[r][c] = phat_t(p2[r][c], A.lamv[(size_t)(b - 1) * g.H + gi], tau);
-        if (PAD && j == mc && s_rgt && i < mr) h2[r][c] = phat_s(p2[r][c], A.lamv[(size_t)b * g.H + gi], tau);
+        if (r == 0 && top) h1[r][c] = phat_t(p1[r][c], lt[c], tau);
+        if (PAD && bot && rpad == r) h1[r][c] = phat_s(p1[r][c], lb[c], tau);
+        if (c == 0 && left) h2[r][c] = phat_t(p2[r][c], ll[r], tau);
+        if (PAD && rgt && cpad == c) h2[r][c] = phat_s(p2[r][c], lr[r], tau);
         if (FID == FID_SEG) fv[r][c] = (fv[r][c] - A.c1) * (fv[r][c] - A.c1) - (fv[r][c] - A.c2) * (fv[r][c] - A.c2);
+        if (MASK && ((mb[r] >> (8 * c)) & 0xffu)) in_d |= 1u << (4 * c + r);
       }
     }
 #pragma unroll
@@ -260,18 +329,12 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     *reinterpret_cast<float4*>(sQ1 + G * BW + j0) = make_float4(p1[0][0], p1[0][1], p1[0][2], p1[0][3]);
     *reinterpret_cast<ulonglong2*>(myQL) = make_ulonglong2(P2[0][0], P2[0][1]);
     if (G == NG - 1) {
-      // pbar1 of the row below the band: the next CTA's first row (its halo of later
-      // iterations), the bottom side of a subdomain that fills the block, or 0
-      const int i = rank * BAND + BAND, n = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;
-      float q[4];
-      load4(A.P1 + (size_t)(r0 + i + a) * g.W + c0 + j0, n, vec, q);
-      *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(q[0], q[1], q[2], q[3]);
-      if (last_group && fill_r && s_bot) {
-        float h[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) h[c] = c < n ? phat_s(q[c], A.lamh[(size_t)a * g.W + c0 + j0 + c], tau) : 0.f;
-        *reinterpret_cast<float4*>(smem + L::PBS + j0) = make_float4(q[0], q[1], q[2], q[3]);
-        *reinterpret_cast<float4*>(smem + L::HBS + j0) = make_float4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(qb[0], qb[1], qb[2], qb[3]);
+      if (bottom_fill) {
+        *reinterpret_cast<float4*>(smem + L::PBS + j0) = make_float4(qb[0], qb[1], qb[2], qb[3]);
+        *reinterpret_cast<float4*>(smem + L::HBS + j0) =
+            make_float4(phat_s(qb[0], lb[0], tau), phat_s(qb[1], lb[1], tau), phat_s(qb[2], lb[2], tau),
+                        phat_s(qb[3], lb[3], tau));
       }
     }
     if (G == 0 && rank == 0) *reinterpret_cast<float4*>(sUB + j0) = make_float4(0.f, 0.f, 0.f, 0.f);  // u above the tile
@@ -279,10 +342,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     // the slot right of the last lane: the right side of a subdomain that fills the block, else 0
     if (rr >= 0 && rr < BAND) smem[L::QL + r_slot] = pr_s;
   }
-  const bool coef_smem = K <= L::kMaxSmemCoef;
-  if (coef_smem)
-    for (int q = tid; q < 16 * K; q += NT)
-      sCo[q] = reinterpret_cast<const float*>(A.coef)[(q >> 4) * 8 + ((q & 15) >> 1)];
+  cp_async_wait_all();
   __syncthreads();
   bool timed_out = false;
   uint32_t phU = 0, phQ = 0;  // index of the next phase of mbU / mbQ this thread waits for
@@ -297,22 +357,23 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     ++phQ;
     if (cl == 0) mbar_arrive_expect_tx(mbQ, kHaloBytes);
   };
-#pragma unroll 2
+  // Two iterations per trip save the moves of the new dual values; with padding or a mask
+  // the doubled code no longer fits the registers and the instruction cache (per outer
+  // iteration, 2160 x 3840 in 120 x 128 subdomains: 144 us unrolled, 138 not; 4096 x 4096 in
+  // 64 x 64: 207 and 219, with a mask 248 and 229).
+#pragma unroll(PAD || MASK ? 1 : 2)
   for (int k = 0; k < K; ++k) {
-    f32x2 SIG, UA, UBc, PA, PC, PB, TH, SS;
+    // (the coefficients of each half-step are loaded when it begins: registers)
+    f32x2 SIG, UA, UBc, SS;
     if (coef_smem) {
       const ulonglong2 cf0 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k);
       const ulonglong2 cf1 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 4);
-      const ulonglong2 cf2 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 8);
-      const ulonglong2 cf3 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 12);
-      SIG = cf0.x, UA = cf0.y, UBc = cf1.x, SS = cf1.y, PA = cf2.x, PC = cf2.y, PB = cf3.x, TH = cf3.y;
+      SIG = cf0.x, UA = cf0.y, UBc = cf1.x, SS = cf1.y;
     } else {
       const float4 ca = __ldg(reinterpret_cast<const float4*>(A.coef) + 2 * k);
-      const float4 cb = __ldg(reinterpret_cast<const float4*>(A.coef) + 2 * k + 1);
       SIG = pk2(ca.x, ca.x), UA = pk2(ca.y, ca.y), UBc = pk2(ca.z, ca.z), SS = pk2(ca.w, ca.w);
-      PA = pk2(cb.x, cb.x), PC = pk2(cb.y, cb.y), PB = pk2(cb.z, cb.z), TH = pk2(cb.w, cb.w);
     }
-    const Coef co{lo2(SIG), lo2(UA), lo2(UBc), lo2(SS), lo2(PA), lo2(PC), lo2(PB), lo2(TH)};
+    const Coef cu{lo2(SIG), lo2(UA), lo2(UBc), lo2(SS), 0.f, 0.f, 0.f, 0.f};
     if (push_down && k > 0) wait_q();  // pbar1 halo of iteration k - 1
     // ---- u-step: pair e = 1 (holding the group's last row) first
     {
@@ -340,10 +401,10 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
             if (MASK) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
           } else if (FID == FID_L1) {  // ubar - P_[-s,s](ubar - f)
             const f32x2 v = sub2(ub, fg);
-            un = sub2(ub, pk2(clamp_abs(lo2(v), co.s), clamp_abs(hi2(v), co.s)));
+            un = sub2(ub, pk2(clamp_abs(lo2(v), cu.s), clamp_abs(hi2(v), cu.s)));
             if (MASK) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
           } else {
-            un = pk2(prox_ubar<FID>(lo2(ub), lo2(fg), dl, co), prox_ubar<FID>(hi2(ub), hi2(fg), dh, co));
+            un = pk2(prox_ubar<FID>(lo2(ub), lo2(fg), dl, cu), prox_ubar<FID>(hi2(ub), hi2(fg), dh, cu));
           }
           U[c][e] = un;
         }
@@ -372,13 +433,23 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       }
       const float4 ul = make_float4(hi2(U[0][1]), hi2(U[1][1]), hi2(U[2][1]), hi2(U[3][1]));
       if (push_down)
-        st_async_v4_f32(remote_u, ul.x, ul.y, ul.z, ul.w, remote_mbU);
+        st_async_v4_f32(remote + 4 * (L::UB + j0), ul.x, ul.y, ul.z, ul.w, remote + 4 * L::MB);
       else if (last_group)
         *reinterpret_cast<float4*>(smem + L::XUB + j0) = ul;  // for the bottom side's update
       if (G < NG - 1) *reinterpret_cast<float4*>(sUB + (G + 1) * BW + j0) = ul;
       *reinterpret_cast<ulonglong2*>(myUR) = make_ulonglong2(U[3][0], U[3][1]);
     }
     __syncthreads();
+    f32x2 PA, PC, PB, TH;
+    if (coef_smem) {
+      const ulonglong2 cf2 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 8);
+      const ulonglong2 cf3 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 12);
+      PA = cf2.x, PC = cf2.y, PB = cf3.x, TH = cf3.y;
+    } else {
+      const float4 cb = __ldg(reinterpret_cast<const float4*>(A.coef) + 2 * k + 1);
+      PA = pk2(cb.x, cb.x), PC = pk2(cb.y, cb.y), PB = pk2(cb.z, cb.z), TH = pk2(cb.w, cb.w);
+    }
+    const Coef co{0.f, 0.f, 0.f, 0.f, lo2(PA), lo2(PC), lo2(PB), lo2(TH)};
     // ---- p-step: first the dofs that need no row above the group (in the first group that
     // row is the halo from the CTA above), then the first row's pbar1 and its push upwards
     {
@@ -420,7 +491,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       }
       const float4 q = make_float4(lo2(Q1[0][0]), lo2(Q1[1][0]), lo2(Q1[2][0]), lo2(Q1[3][0]));
       if (G > 0) *reinterpret_cast<float4*>(sQ1 + G * BW + j0) = q;
-      if (push_up) st_async_v4_f32(remote_q1, q.x, q.y, q.z, q.w, remote_mbQ);
+      if (push_up) st_async_v4_f32(remote + 4 * (L::Q1 + NG * BW + j0), q.x, q.y, q.z, q.w, remote + 4 * L::MB + 8);
     }
     if (right_lane) {  // Du = -u of the last column ((-pc) u = pc (-u) exactly)
       const float tt = fmaf(-co.pc, smem[L::UR + r_slot], fmaf(co.pa, pr_s, co.pb * hr_s));
@@ -448,42 +519,12 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
                               // stores below hide the wait
   }
 
-  // ---- store u^{n+1}, p~^{n+1} and the interface strips
-  const bool vec = (g.W & 3) == 0 && (c0 & 3) == 0;
-  // the strips of a set start at multiples of the interface edges, not of 4 floats
-  const bool vec_t = vec && (reinterpret_cast<uintptr_t>(out.ST) & 15) == 0;
-  const bool vec_b = vec && (reinterpret_cast<uintptr_t>(out.SB) & 15) == 0;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int e = r & 1, h = r >> 1, i = i0 + r, gi = r0 + i;
-    const int n = i < mr ? mc - j0 : 0;
-    const int n1 = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;
-    const int n2 = i < mr ? mc + (s_rgt ? 1 : 0) - j0 : 0;
-    store4(A.u + (size_t)gi * g.W + c0 + j0, n, vec, half_of(U[0][e], h), half_of(U[1][e], h), half_of(U[2][e], h),
-           half_of(U[3][e], h));
-    const float q0 = half_of(P1[0][e], h), q1 = half_of(P1[1][e], h), q2 = half_of(P1[2][e], h), q3 = half_of(P1[3][e], h);
-    store4(A.P1 + (size_t)(gi + a) * g.W + c0 + j0, n1, vec, q0, q1, q2, q3);
-    if (r == 0 && i == 0 && s_top) store4(out.ST + (ptrdiff_t)(a - 1) * g.W + c0 + j0, n1, vec_t, q0, q1, q2, q3);
-    if (PAD && i == mr && s_bot) store4(out.SB + (size_t)a * g.W + c0 + j0, n1, vec_b, q0, q1, q2, q3);
-    store4(A.P2 + (size_t)gi * W2 + c0 + b + j0, n2, false, half_of(P2[0][e], h), half_of(P2[1][e], h),
-           half_of(P2[2][e], h), half_of(P2[3][e], h));
-    if (j0 == 0 && s_lft && i < mr) out.SL[(size_t)(b - 1) * g.H + gi] = half_of(P2[0][e], h);
-    if (PAD && s_rgt && i < mr) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (j0 + c == mc) out.SR[(size_t)b * g.H + gi] = half_of(P2[c][e], h);
-    }
-  }
-  if (right_lane) {
-    const int gi = r0 + rank * BAND + rr;
-    A.P2[(size_t)gi * W2 + c0 + BW + b] = pr_s;
-    out.SR[(size_t)b * g.H + gi] = pr_s;
-  }
-  if (bottom_lane) {
-    const float4 v = *reinterpret_cast<const float4*>(smem + L::PBS + j0);
-    store4(A.P1 + (size_t)(r0 + mr + a) * g.W + c0 + j0, mc - j0, vec, v.x, v.y, v.z, v.w);
-    store4(out.SB + (size_t)a * g.W + c0 + j0, mc - j0, vec_b, v.x, v.y, v.z, v.w);
-  }
+  // ---- store u^{n+1}, p~^{n+1} and the interface strips.  The geometry is worked out again
+  // rather than kept in registers through the loop (the asm hides that it is the same).
+  int tid2 = tid, a2 = a, b2 = b;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid2));
+  asm volatile("" : "+r"(a2), "+r"(b2));
+  tile_store<LPR, NW, PAD>(A, out, a2, b2, tid2, CL, rank, U, P1, P2, pr_s);
   if (CLU) {
     if (timed_out) atomicOr(A.err, 1);
     __syncwarp();
@@ -493,8 +534,11 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
 
 // 16 warps per SM: 128 registers per thread
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
-__global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile(const LocalArgs A) {
-  tile_solve<LPR, NW, CLU, PAD, FID, MASK>(A, A.out, (int)blockIdx.z, (int)blockIdx.y);
+__global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile(const LocalArgs A, const int cl) {
+  // block x = CTA x % cl of subdomain x / cl (a 1-D grid: any number of subdomains)
+  const unsigned t = CLU ? blockIdx.x / (unsigned)cl : blockIdx.x, rank = CLU ? blockIdx.x - t * (unsigned)cl : 0u;
+  const unsigned a = t / (unsigned)A.g.NC;
+  tile_solve<LPR, NW, CLU, PAD, FID, MASK>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank, CLU ? cl : 1);
 }
 
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
@@ -522,18 +566,20 @@ cudaError_t prepare_tile() {
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
 cudaError_t launch_tile_one(const LocalArgs& a, int cl, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CLU ? cl : 1, a.g.NC, a.g.NR);
+  cfg.gridDim = dim3((unsigned)(CLU ? cl : 1) * a.g.NC * a.g.NR, 1, 1);
   cfg.blockDim = dim3(32 * NW, 1, 1);
   cfg.dynamicSmemBytes = TileLayout<LPR, NW>::BYTES;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CLU ? cl : 1;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
   cfg.attrs = attr;
-  cfg.numAttrs = CLU ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_tile<LPR, NW, CLU, PAD, FID, MASK>, a);
+  if (has_interfaces(a.g)) pdl_attr(&attr[cfg.numAttrs++]);
+  if (CLU) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = cl;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, k_tile<LPR, NW, CLU, PAD, FID, MASK>, a, cl);
 }
 
 template <int LPR, int NW, bool CLU, bool PAD>
@@ -553,6 +599,48 @@ cudaError_t launch_tile_fid(const LocalArgs& a, int fid, int cl, cudaStream_t st
 template <int LPR, int NW, bool CLU>
 cudaError_t launch_tile(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st) {
   return pad ? launch_tile_fid<LPR, NW, CLU, true>(a, fid, cl, st) : launch_tile_fid<LPR, NW, CLU, false>(a, fid, cl, st);
+}
+
+// Every subdomain of a batch of images (all of them fill their block), CL CTAs each, with
+// its image's fidelity, parameters and strips.
+template <int LPR, int NW, int CL>
+__global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile_batch(const BatchArgs B) {
+  const int t = (int)blockIdx.x / CL, rank = (int)blockIdx.x % CL;
+  const int img = B.tile_img[t];
+  const LocalArgs A = B.args[img];
+  const int q = t - B.tile_base[img];
+  const int a = q / A.g.NC, b = q - a * A.g.NC;
+  const Strips out = B.strips[2 * img + B.write_set];
+  switch (B.fid[img]) {
+    case FID_L2: tile_solve<LPR, NW, (CL > 1), false, FID_L2, false>(A, out, a, b, rank, CL); break;
+    case FID_L1: tile_solve<LPR, NW, (CL > 1), false, FID_L1, false>(A, out, a, b, rank, CL); break;
+    default: tile_solve<LPR, NW, (CL > 1), false, FID_SEG, false>(A, out, a, b, rank, CL); break;
+  }
+}
+
+template <int LPR, int NW, int CL>
+cudaError_t prepare_tile_batch() {
+  return cudaFuncSetAttribute(k_tile_batch<LPR, NW, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)TileLayout<LPR, NW>::BYTES);
+}
+
+template <int LPR, int NW, int CL>
+cudaError_t launch_tile_batch(const BatchArgs& B, int total_tiles, bool overlap, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CL * total_tiles, 1, 1);
+  cfg.blockDim = dim3(32 * NW, 1, 1);
+  cfg.dynamicSmemBytes = TileLayout<LPR, NW>::BYTES;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  cfg.attrs = attr;
+  if (overlap) pdl_attr(&attr[cfg.numAttrs++]);
+  if (CL > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = CL;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, k_tile_batch<LPR, NW, CL>, B);
 }
 
 }  // namespace

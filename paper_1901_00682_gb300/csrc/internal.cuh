@@ -108,6 +108,27 @@ struct AdjArgs {
   float* tape;             // tile-fused reverse kernel: adj_fused_tape_floats(g, K) floats
 };
 
+// Programmatic dependent launch.  A kernel launched with pdl_attr may start while its
+// predecessor in the stream still runs, once every block of that one has called
+// pdl_trigger or ended; pdl_wait returns when the predecessor has completed and its
+// writes are visible (at once in a kernel launched without the attribute).
+//
+// The outer iteration is a chain of short kernels: multiplier update, local solves, update,
+// ...  The update waits before its first access and triggers after that wait, so a
+// local solve that starts early knows the previous local solve complete: it loads its
+// state at once and waits only before it reads the multipliers and before it ends.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+inline void pdl_attr(cudaLaunchAttribute* attr) {
+  attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr->val.programmaticStreamSerializationAllowed = 1;
+}
+
+// whether a multiplier update precedes the local solves of grid g (otherwise their
+// predecessor is the previous local solve itself, whose results they load)
+inline bool has_interfaces(const Grid& g) { return g.NR > 1 || g.NC > 1 || g.cut_top || g.cut_bot; }
+
 // ---- kernels_interface.cu
 // lambda += sigma ((2 cur_s - prev_s) - (2 cur_t - prev_t)) on every interface edge.
 cudaError_t launch_interface(const Grid& g, float sigma, Strips cur, Strips prev, float* lamh, float* lamv,
@@ -121,10 +142,12 @@ cudaError_t launch_interface_batch(const BatchIfaceArgs& a, int total4, cudaStre
 
 // ---- kernels_fused.cu
 // All tiles of all images of a batch, one launch (BatchArgs.write_set selects the strips);
-// tile: the subdomain side, 128 (persistent micro-tile kernels: variant 0 the 4 x 4 one
-// when K <= fused_mt4_max_inner(), else and for variant 2 the 2 x 4 one) or 64 (one CTA
-// per subdomain).
-cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, int variant, int K, cudaStream_t st);
+// tile: the subdomain side, 128 or 64; variant 2 (128 only): the persistent 2 x 4
+// micro-tile kernel instead of the micro-tile kernel of fused_tile.cuh.  overlap: a
+// multiplier update precedes it in the stream (the batch has interfaces), so it may start
+// early.
+cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, int variant, bool overlap,
+                               cudaStream_t st);
 // One outer iteration's local solves, all tiles, fused (returns cudaErrorInvalidValue
 // if no fused configuration fits the tile shape).
 cudaError_t launch_fused_local(const LocalArgs& a, int fidelity, int variant, cudaStream_t st);
@@ -147,19 +170,12 @@ cudaError_t launch_fused_mt_batch(const BatchArgs& B, int total_tiles, cudaStrea
 
 // ---- kernels_fused_mt4.cu
 // Persistent fused local solver on 4 x 4 micro-tiles, one warp per thread row, three
-// 128-thread CTAs per SM; 128 x 128 tiles with 16-byte aligned rows
-// (fused_mt4_supported).
+// 128-thread CTAs per SM, the state moved by tensor copies; 128 x 128 tiles with 16-byte
+// aligned rows (fused_mt4_supported), fixed inner count or (a.inner_tol2 > 0) the adaptive
+// stop.  cudaErrorNotSupported if the tensor maps cannot be encoded.
 bool fused_mt4_supported(const LocalArgs& a);
-// tma: move the state with tensor copies (falls back to cp.async if the tensor maps
-// cannot be encoded).  With a.inner_tol2 > 0 (adaptive inner stop) the tensor-copy
-// kernel runs whatever tma says, and cudaErrorNotSupported comes back if its maps
-// cannot be encoded.
-cudaError_t launch_fused_mt4(const LocalArgs& a, int fidelity, bool tma, cudaStream_t st);
+cudaError_t launch_fused_mt4(const LocalArgs& a, int fidelity, cudaStream_t st);
 cudaError_t fused_mt4_prepare();
-// The same kernel (cp.async copies) over the work list of a batch: every image's arrays
-// 16-byte aligned, inner count <= fused_mt4_max_inner().
-cudaError_t launch_fused_mt4_batch(const BatchArgs& B, int total_tiles, cudaStream_t st);
-int fused_mt4_max_inner();
 
 // ---- kernels_tile8.cu, kernels_tile16.cu, kernels_tile32.cu (fused_tile.cuh)
 // launch_tile_<LPR>_<NW>: the micro-tile kernel with LPR lanes per row group and NW warps
@@ -175,8 +191,9 @@ cudaError_t prepare_tile_8_4();
 cudaError_t prepare_tile_16_4();
 cudaError_t prepare_tile_16_8();
 cudaError_t prepare_tile_32_4();
-// every 64 x 64 subdomain of every image of a batch (launch_tile_16_8's kernel)
-cudaError_t launch_tile_batch_64(const BatchArgs& B, int total_tiles, cudaStream_t st);
+// every subdomain of every image of a batch, 64 x 64 or 128 x 128
+cudaError_t launch_tile_batch_128(const BatchArgs& B, int total_tiles, bool overlap, cudaStream_t st);
+cudaError_t launch_tile_batch_64(const BatchArgs& B, int total_tiles, bool overlap, cudaStream_t st);
 
 // ---- kernels_full.cu
 // n <= full_max_steps() full-dimension iterations in one launch, a.in -> a.out (the dofs of

@@ -58,9 +58,11 @@ __global__ void __launch_bounds__(FL::NT, 4) k_full(const FullArgs A, const Axis
   float* sUB = smem + FL::UB;
   float* sQ1 = smem + FL::Q1;
   const uint32_t mbU = smem_addr(smem + FL::MB), mbQ = mbU + 8;
-  const int CL = (int)gridDim.x, rank = (int)blockIdx.x;
+  // a 1-D grid: CTA x % CL of block x / CL, row by row
+  const int CL = (ar.size() + BAND - 1) / BAND, rank = (int)(blockIdx.x % (unsigned)CL);
+  const int by = (int)(blockIdx.x / (unsigned)CL) / ac.m, bx = (int)(blockIdx.x / (unsigned)CL) - by * ac.m;
   const int W = A.W, W2 = A.W + 1;
-  const int c0 = ac.start(blockIdx.y), mc = ac.size(), r0 = ar.start(blockIdx.z), mr = ar.size();
+  const int c0 = ac.start(bx), mc = ac.size(), r0 = ar.start(by), mr = ar.size();
   const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
   const int j0 = 4 * l, i0 = rank * BAND + 4 * w;
   const bool push_down = w == NG - 1 && rank + 1 < CL, push_up = w == 0 && rank > 0;
@@ -86,6 +88,8 @@ __global__ void __launch_bounds__(FL::NT, 4) k_full(const FullArgs A, const Axis
   }
   __syncthreads();
   cluster_arrive<true>();  // matched before the first halo is sent: the loads hide the wait
+  pdl_trigger();
+  pdl_wait();  // the launch before, whose results this one reads
 
   // clamp limits: 0 on the image boundary
   float lim1[4], lim2[4];
@@ -256,7 +260,7 @@ __global__ void __launch_bounds__(FL::NT, 4) k_full(const FullArgs A, const Axis
   cluster_arrive<false>();  // no CTA leaves while a neighbour may still write into it
 
   // ---- store what n iterations leave exact
-  const int ra = ar.from(blockIdx.z), rb = ar.to(blockIdx.z), ca = ac.from(blockIdx.y), cb = ac.to(blockIdx.y);
+  const int ra = ar.from(by), rb = ar.to(by), ca = ac.from(bx), cb = ac.to(bx);
   const int ja = c0 + j0;
   const bool whole = ja >= ca && ja + 4 <= cb;
   const bool vec = whole && (W & 3) == 0 && (ja & 3) == 0;
@@ -291,17 +295,18 @@ cudaError_t launch_full_one(const FullArgs& a, int n, cudaStream_t st) {
   const Axis ar = axis_for(a.H, n), ac = axis_for(a.W, n);
   const int cl = (ar.size() + FL::BAND - 1) / FL::BAND;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cl, ac.m, ar.m);
+  cfg.gridDim = dim3((unsigned)cl * ac.m * ar.m, 1, 1);
   cfg.blockDim = dim3(FL::NT, 1, 1);
   cfg.dynamicSmemBytes = FL::BYTES;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  pdl_attr(&attr[1]);
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_full<FID, MASK>, a, ar, ac, n);
 }
 

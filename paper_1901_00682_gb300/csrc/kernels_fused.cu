@@ -1,7 +1,7 @@
 // Fused local solver with cluster barriers: the adaptive inner stop of every subdomain
 // shape but exact 128 x 128, and variant 3 of those; and the choice among the fused
-// kernels (launch_fused_local).  A fixed inner count on any other shape runs the
-// micro-tile kernel of fused_tile.cuh.
+// kernels (launch_fused_local).  A fixed inner count runs the micro-tile kernel of
+// fused_tile.cuh.
 //
 // All inner iterations of one outer iteration of Algorithm 1 for every subdomain in one
 // launch (Section 5, local problem eq. local, solved by the
@@ -336,8 +336,8 @@ __global__ void __launch_bounds__(BW* TR, (BW * TR <= 256 ? 2 : 1)) k_fused(cons
 }
 
 // Hardware mappings of exact 128 x 128 subdomains (dd_tv_params.variant):
-//   0  persistent 4 x 4 micro-tiles, state moved by tensor copies (default)
-//   1  the same kernel moving the state with 16-byte cp.async copies
+//   0  the micro-tile kernel of every other shape (fused_tile.cuh)
+//   1  persistent 4 x 4 micro-tiles, state moved by tensor copies
 //   2  persistent 2 x 4 micro-tiles, 256 threads, 2 CTAs per SM
 //   3  the cluster-barrier kernel (one subdomain per cluster)
 constexpr int kNumVariants = 4;
@@ -398,6 +398,9 @@ cudaError_t prepare_fid() {
 // cluster.  Up to 32 x 32 and 64 x 64 one CTA holds the subdomain: no halo leaves the
 // SM.  In a cluster of two 32-row CTAs, 64 x 64 subdomains take 256 us per outer
 // iteration of 10 inner ones at 4096^2 and 14.1 us at 128^2, in one CTA 217 and 13.0.
+// 128 columns run 16-row CTAs in clusters of up to 8: with 32 rows in 8 warps and
+// clusters of 4, 4096^2 takes 233 us instead of 215, and 120 x 128 subdomains (2160 x
+// 3840) 146 instead of 137.
 cudaError_t launch_tile_shape(const LocalArgs& a, int mr, int mc, int fid, cudaStream_t st) {
   auto go = [&](cudaError_t (*launch)(const LocalArgs&, int, int, bool, cudaStream_t), int bw, int band) {
     const int cl = (mr + band - 1) / band;
@@ -443,43 +446,39 @@ cudaError_t fused_prepare() {
   return fused_mt4_prepare();
 }
 
-cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, int variant, int K, cudaStream_t st) {
-  if (tile == 128)  // variant 0: 4 x 4 micro-tiles (K within its shared coefficient table); 2: 2 x 4
-    return variant == 0 && K <= fused_mt4_max_inner() ? launch_fused_mt4_batch(B, total_tiles, st)
-                                                       : launch_fused_mt_batch(B, total_tiles, st);
-  return tile == 64 ? launch_tile_batch_64(B, total_tiles, st) : cudaErrorInvalidValue;
+cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, int variant, bool overlap,
+                               cudaStream_t st) {
+  if (tile == 128)
+    return variant == 2 ? launch_fused_mt_batch(B, total_tiles, st) : launch_tile_batch_128(B, total_tiles, overlap, st);
+  return tile == 64 ? launch_tile_batch_64(B, total_tiles, overlap, st) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStream_t st) {
   // largest tile of the (ragged) partition
   const int mr = (a.g.H + a.g.NR - 1) / a.g.NR, mc = (a.g.W + a.g.NC - 1) / a.g.NC;
   const bool exact128 = a.g.H == 128 * a.g.NR && a.g.W == 128 * a.g.NC;  // every tile exactly 128 x 128
-  if (a.inner_tol2 > 0.0 && exact128 && variant == 0 && fused_mt4_supported(a)) {
-    // adaptive inner stop in the default kernel (the other variants: the cluster-barrier kernel)
-    const cudaError_t e = launch_fused_mt4(a, fid, true, st);
-    if (e != cudaErrorNotSupported) return e;
-  }
-  if (a.inner_tol2 <= 0.0 && exact128) {
-    switch (variant) {
-      case 0:  // default: persistent 4 x 4 micro-tiles, tensor copies
-      case 1:  // the same with cp.async copies
-        if (fused_mt4_supported(a)) return launch_fused_mt4(a, fid, variant == 0, st);
-        if (fused_mt_supported(a)) return launch_fused_mt(a, fid, st);  // W + N_c not a multiple of 4
-        break;
-      case 2:
-        if (fused_mt_supported(a)) return launch_fused_mt(a, fid, st);
-        break;
-      default: break;
+  if (a.inner_tol2 > 0.0) {
+    // the adaptive stop: in the persistent micro-tile kernel where it applies (variant 0)
+    if (exact128 && variant == 0 && fused_mt4_supported(a)) {
+      const cudaError_t e = launch_fused_mt4(a, fid, st);
+      if (e != cudaErrorNotSupported) return e;
+    }
+    switch (pick(mr, mc)) {
+      case 0: return launch_fid<32, 8, 4, 1, true>(a, fid, st);
+      case 1: return launch_fid<64, 8, 8, 1, true>(a, fid, st);
+      case 2: return launch_fid<128, 8, 2, 8, true>(a, fid, st);
+      default: return cudaErrorInvalidValue;
     }
   }
-  if (a.inner_tol2 <= 0.0)  // exact 128 x 128 subdomains: variant 3, or arrays the kernels above cannot take
-    return exact128 ? launch_fid<128, 8, 2, 8, false>(a, fid, st) : launch_tile_shape(a, mr, mc, fid, st);
-  switch (pick(mr, mc)) {
-    case 0: return launch_fid<32, 8, 4, 1, true>(a, fid, st);
-    case 1: return launch_fid<64, 8, 8, 1, true>(a, fid, st);
-    case 2: return launch_fid<128, 8, 2, 8, true>(a, fid, st);
-    default: return cudaErrorInvalidValue;
+  if (exact128) {
+    if (variant == 1 && fused_mt4_supported(a)) {
+      const cudaError_t e = launch_fused_mt4(a, fid, st);
+      if (e != cudaErrorNotSupported) return e;
+    }
+    if (variant == 2 && fused_mt_supported(a)) return launch_fused_mt(a, fid, st);
+    if (variant == 3) return launch_fid<128, 8, 2, 8, false>(a, fid, st);
   }
+  return launch_tile_shape(a, mr, mc, fid, st);
 }
 
 }  // namespace ddtv

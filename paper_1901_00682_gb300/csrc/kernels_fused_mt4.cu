@@ -16,25 +16,23 @@
 // the lane to its left), and its warp's last-row u and first-row pbar1 with the warps
 // above and below; two CTA barriers order them.  Rows crossing CTAs travel with
 // st.async and mbarrier complete_tx (bounded waits, the same phase protocol as
-// kernels_fused_mt.cu), and the next subdomain is prefetched with 16-byte cp.async copies
-// (p2 as a window starting on a 16-byte boundary: W + N_c must be a multiple of 4).
-// Rows are packed in pairs (r, r + 2) for the `*.f32x2` arithmetic; every value is
-// computed with the operations of the scalar iteration in the same order, so the
-// results are bit-identical to the other mappings.
+// kernels_fused_mt.cu).  Rows are packed in pairs (r, r + 2) for the `*.f32x2` arithmetic;
+// every value is computed with the operations of the scalar iteration in the same order,
+// so the results are bit-identical to the other mappings.
 //
-// TMA: the same kernel moving the state with the tensor memory accelerator.  One thread
-// loads the next subdomain's u, f, p1 bands and p2 window as four 2-D tensor copies
-// (cp.async.bulk.tensor, completion counted on an mbarrier), and stores the previous
-// subdomain's u and p1 bands from an out-buffer in shared memory as two tensor copies
-// (bulk group, issued after the barrier that follows the out-buffer writes; the buffer
-// is rewritten only after a wait for the copies to have read it); p2 and the sides go
-// out with ordinary stores.
+// The state moves with the tensor memory accelerator.  One thread loads the next
+// subdomain's u, f, p1 bands and p2 window (starting on a 16-byte boundary: W + N_c must be
+// a multiple of 4) as four 2-D tensor copies (cp.async.bulk.tensor, completion counted on
+// an mbarrier), and stores the previous subdomain's u and p1 bands from an out-buffer in
+// shared memory as two tensor copies (bulk group, issued after the barrier that follows
+// the out-buffer writes; the buffer is rewritten only after a wait for the copies to have
+// read it); p2 and the sides go out with ordinary stores.
 //
-// Batch: k_fused_mt4_batch runs the cp.async form of the body over the work list of a
-// batch of images (BatchTiles), every subdomain with its image's descriptor (kept in
-// shared memory while the image does not change), fidelity and coefficients.
+// With a fixed inner count this is variant 1; the default there is the micro-tile kernel
+// of fused_tile.cuh, whose f and proximal centres in shared memory leave room for a fourth
+// CTA per SM (4096 x 4096, 10 inner iterations: 215 us against 231 here).
 //
-// ADAPT (tensor-copy kernel only): adaptive inner stopping (Section 5, eq. stop_inner1).
+// ADAPT: adaptive inner stopping (Section 5, eq. stop_inner1).
 // Every thread sums (p^{k+1} - p^k)^2 and (p^{k+1})^2 over its dofs in the p-step of
 // iteration k (packed float32 pairs) and leaves them in the P1 out-buffer, idle during
 // the inner loop.  At the start of iteration k + 1 one warp adds the CTA's 128 pairs
@@ -87,9 +85,7 @@ struct Mt4Layout {
   static constexpr int XLR = XLL + BAND;             // lamv right of the band rows (BAND)
   static constexpr int PBS = XLR + BAND;             // bottom side p of the tile (128; last CTA)
   static constexpr int HBS = PBS + BW;               // bottom side phat (128)
-  static constexpr int MB = HBS + BW;                // two mbarriers
-  static constexpr size_t BYTES = sizeof(float) * MB + 16;
-  // tensor-copy variant: out-buffers of u and p1 (128-byte aligned), three mbarriers
+  // out-buffers of u and p1 (128-byte aligned), five mbarriers
   static constexpr int OU = (HBS + BW + 31) & ~31;
   static constexpr int OP1 = OU + BAND * BW;
   // adaptive inner stop: during the inner loop OP1 holds every thread's residual sums (4
@@ -108,11 +104,11 @@ struct Mt4Layout {
 #endif
   static constexpr int kReduceWarp = MT4_REDUCE_WARP;  // adds the CTA's residual sums and sends them
   static constexpr int kDecideWarp = MT4_DECIDE_WARP;  // takes the stop decision
-  static constexpr size_t BYTES_TMA = sizeof(float) * MBT + 48;
+  static constexpr size_t BYTES = sizeof(float) * MBT + 48;
   static constexpr uint32_t kTmaBytes = 4 * (3 * BAND * BW + BAND * P2S);  // one subdomain's four tensor loads
   static_assert(Q1 % 4 == 0 && UR % 4 == 0 && QL % 4 == 0 && F % 4 == 0 && CO % 4 == 0 && SU % 4 == 0 &&
                     SP2 % 4 == 0 && XLT % 4 == 0 && XLL % 4 == 0 && XLR % 4 == 0 && PBS % 4 == 0 &&
-                    HBS % 4 == 0 && MB % 2 == 0,
+                    HBS % 4 == 0,
                 "16-byte alignment of the vector and cp.async buffers");
   static_assert(CL * BAND == 128, "a cluster of CTAs covers the 128 rows of a tile");
   static_assert(SU % 32 == 0 && SP2 % 32 == 0 && (BAND * BW) % 32 == 0 && OU % 32 == 0 && OP1 % 32 == 0,
@@ -146,83 +142,34 @@ __device__ __forceinline__ void tma_fence_smem() { asm volatile("fence.proxy.asy
 
 __device__ __forceinline__ float lane4(f32x2 v, int h) { return h ? hi2(v) : lo2(v); }
 
-// The subdomains of one image (tile t = a N_c + b), its fidelity fixed at compile time.
-// The batch kernel runs the same body over BatchTiles (fused_common.cuh): every
-// subdomain with its image's geometry, parameters, strips and fidelity.
-template <int FID>
-struct Mt4One {
-  const LocalArgs& A;
-  static constexpr bool kBatch = false;
-  __device__ int count() const { return A.g.NR * A.g.NC; }
-  __device__ int inner() const { return A.K; }
-  __device__ int image(int) const { return 0; }
-  __device__ const LocalArgs& args(int) const { return A; }
-  __device__ int local(int t) const { return t; }
-  __device__ Strips out(int) const { return A.out; }
-  __device__ int* err() const { return A.err; }
-  template <class Body>
-  __device__ void dispatch(int, Body&& body) const {
-    body(FidC<FID>{});
-  }
-};
-
-// A batch image's descriptor as the batch kernel keeps it in shared memory: its
-// LocalArgs, the strips it writes this launch, its first tile in the work list, its
-// fidelity and its index.
-struct Mt4BatchDesc {
-  LocalArgs A;
-  Strips out;
-  int base, fid, img, pad;
-};
-static_assert(sizeof(LocalArgs) % 4 == 0 && sizeof(Strips) % 4 == 0 && sizeof(Mt4BatchDesc) % 16 == 0,
-              "descriptors copied word by word");
-
-// every thread of the CTA copies words of image img's descriptor into d (a barrier must
-// follow before d is read)
-__device__ __forceinline__ void load_batch_desc(Mt4BatchDesc* d, const BatchArgs& B, int img, int tid, int nt) {
-  constexpr int kA = sizeof(LocalArgs) / 4, kS = sizeof(Strips) / 4, kN = sizeof(Mt4BatchDesc) / 4;
-  const uint32_t* a = reinterpret_cast<const uint32_t*>(B.args + img);
-  const uint32_t* st = reinterpret_cast<const uint32_t*>(B.strips + 2 * img + B.write_set);
-  uint32_t* dst = reinterpret_cast<uint32_t*>(d);
-  for (int q = tid; q < kN; q += nt) {
-    uint32_t v = 0;
-    if (q < kA) v = a[q];
-    else if (q < kA + kS) v = st[q - kA];
-    else if (q == kA + kS) v = (uint32_t)B.tile_base[img];
-    else if (q == kA + kS + 1) v = (uint32_t)B.fid[img];
-    else if (q == kA + kS + 2) v = (uint32_t)img;
-    dst[q] = v;
-  }
-}
-
 // the coefficient sets of an image into shared memory, each coefficient twice
 __device__ __forceinline__ void load_coef_dup(float* sCo, const Coef* coef, int K, int tid, int nt) {
   for (int q = tid; q < 16 * K; q += nt)  // K <= kMaxSmemCoef
     sCo[q] = reinterpret_cast<const float*>(coef)[(q >> 4) * 8 + ((q & 15) >> 1)];
 }
 
-template <bool MASK, bool TMA, bool ADAPT, class Src>
-__device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, const int first, const int stride) {
+template <int FID, bool MASK, bool ADAPT>
+__device__ __forceinline__ void fused_mt4_body(const LocalArgs& A, const Mt4Maps* M, const int first, const int stride) {
   using L = Mt4Layout;
   constexpr int NW = L::NW, CL = L::CL, BAND = L::BAND, NT = L::NT, BW = L::BW;
   extern __shared__ __align__(128) float smem[];
   float* sUB = smem + L::UB;
   float* sQ1 = smem + L::Q1;
   float* sCo = smem + L::CO;
-  const uint32_t mbU = smem_addr(smem + (TMA ? L::MBT : L::MB));
+  const uint32_t mbU = smem_addr(smem + L::MBT);
   const uint32_t mbQ = mbU + 8;
-  const uint32_t mbL = mbU + 16;  // tensor loads of the staged subdomain (TMA)
+  const uint32_t mbL = mbU + 16;  // tensor loads of the staged subdomain
   const uint32_t mbR = mbU + 24;  // reduction phases of the adaptive stop, two mbarriers (parity)
-  static_assert(!ADAPT || TMA, "the adaptive stop keeps the rolled-back u in the tensor-copy out-buffer");
-  static_assert(!(Src::kBatch && (TMA || ADAPT || MASK)), "the batch runs the cp.async kernel, fixed counts, no mask");
-
-  const int T = S.count();
+  const Grid g = A.g;
+  const int T = g.NR * g.NC, W2 = g.W + g.NC;
+  const float tau = A.tau;
+  const Strips out = A.out;
   const int rank = (int)blockIdx.x;
   const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
   const int j0 = 4 * l;              // the lane's first column in the tile
   const int lr0 = 4 * w;             // the warp's first row in the band
   const int i0 = rank * BAND + lr0;  // ... in the tile
-  const int K = S.inner();
+  const int K = A.K;
   const bool last_row_here = rank == CL - 1 && w == NW - 1;
   // the tile's bottom side is updated by warp 2 of the last CTA (the last warp, which
   // holds the last row, already waits for halos and pushes rows); warp 1 updates the
@@ -245,27 +192,19 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
     remote_q1 = map_rank(smem_addr(sQ1 + NW * BW + j0), rank - 1);
     remote_mbQ = map_rank(mbQ, rank - 1);
   }
+  pdl_trigger();  // (the next update; this grid itself starts after the one before it: were its
+                  // clusters placed beside an update's blocks, some would wait for a second round)
   if (tid == 0) {
     mbar_init(mbU, 1);
     mbar_init(mbQ, 1);
-    if (TMA) mbar_init(mbL, 1);
+    mbar_init(mbL, 1);
     if (ADAPT) {
       mbar_init(mbR, 1);
       mbar_init(mbR + 8, 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (!Src::kBatch) load_coef_dup(sCo, S.args(0).coef, K, tid, NT);
-  int cur_img = Src::kBatch ? -1 : 0;  // image whose coefficients are in sCo
-  // batch: the descriptors of the current and of the next subdomain's image, in the P1
-  // out-buffer region (unused by the cp.async kernel); a subdomain of the image already
-  // held reuses its slot, so the work list is read from global memory once per subdomain
-  // (its image index, loaded a subdomain ahead) and a descriptor once per image change
-  Mt4BatchDesc* const dsc = reinterpret_cast<Mt4BatchDesc*>(smem + L::OP1);
-  int cur = 0;  // slot of the current subdomain's descriptor
-  if constexpr (Src::kBatch) {
-    if (first < T) load_batch_desc(&dsc[0], S.B, S.B.tile_img[first], tid, NT);
-  }
+  load_coef_dup(sCo, A.coef, K, tid, NT);
   if (rank == 0 && w == 0) *reinterpret_cast<float4*>(sUB + j0) = make_float4(0.f, 0.f, 0.f, 0.f);  // u above the tile
   if (l < 4) smem[L::UR + w * L::SLOT + l] = 0.f;  // u left of the tile
   __syncthreads();
@@ -278,48 +217,16 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
   cluster_arrive<true>();  // barriers initialised and armed everywhere before any halo is sent
   cluster_wait();
 
-  auto prefetch = [&](int t, const LocalArgs& A, const int lt) {
-    const Grid g = A.g;
-    const int W2 = g.W + g.NC;
-    const int a = lt / g.NC, b = lt - a * g.NC;
+  auto prefetch = [&](int t) {
+    const int a = t / g.NC, b = t - a * g.NC;
     const int c0 = b * 128;
     const int gb = a * 128 + rank * BAND;  // image row of the band's first row
-    if (TMA) {
-      if (tid == 0) {
-        mbar_arrive_expect_tx(mbL, L::kTmaBytes);
-        tma_load_2d(smem + L::SU, &M->u, c0, gb, mbL);
-        tma_load_2d(smem + L::SU + BAND * BW, &M->f, c0, gb, mbL);
-        tma_load_2d(smem + L::SU + 2 * BAND * BW, &M->p1, c0, gb + a, mbL);
-        tma_load_2d(smem + L::SP2, &M->p2, c0 + b - (b & 3), gb, mbL);
-      }
-    } else {
-#pragma unroll
-      for (int m = 0; m < 12; ++m) {  // u, f, p1: 3 x BAND rows x 32 chunks of 16 bytes
-        const int fld = m >> 2;
-        const int q = tid + NT * (m & 3);
-        const int row = q >> 5, ch = q & 31;
-        const float* base = fld == 0 ? A.u : (fld == 1 ? A.f : A.P1);
-        const int grow = gb + row + (fld == 2 ? a : 0);
-        cp_async16(smem + L::SU + fld * BAND * BW + row * BW + 4 * ch, base + (size_t)grow * g.W + c0 + 4 * ch);
-      }
-      if (!Src::kBatch || (W2 & 3) == 0) {
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {  // p2 window: BAND rows x 33 chunks
-          const int q = tid + NT * m;
-          if (q < BAND * 33) {
-            const int row = q / 33, ch = q - row * 33;
-            cp_async16(smem + L::SP2 + row * L::P2S + 4 * ch,
-                       A.P2 + (size_t)(gb + row) * W2 + c0 + b - (b & 3) + 4 * ch);
-          }
-        }
-      } else {  // rows not 16-byte aligned (a batch image with W + N_c not a multiple of 4):
-                // the tile's 129 p2 columns one by one, at the same place in the window
-        const int o = b & 3;
-        for (int q = tid; q < BAND * 129; q += NT) {
-          const int row = q / 129, col = q - row * 129;
-          cp_async4(smem + L::SP2 + row * L::P2S + o + col, A.P2 + (size_t)(gb + row) * W2 + c0 + b + col);
-        }
-      }
+    if (tid == 0) {
+      mbar_arrive_expect_tx(mbL, L::kTmaBytes);
+      tma_load_2d(smem + L::SU, &M->u, c0, gb, mbL);
+      tma_load_2d(smem + L::SU + BAND * BW, &M->f, c0, gb, mbL);
+      tma_load_2d(smem + L::SU + 2 * BAND * BW, &M->p1, c0, gb + a, mbL);
+      tma_load_2d(smem + L::SP2, &M->p2, c0 + b - (b & 3), gb, mbL);
     }
     if (tid < 32) {
       if (rank == 0 && (a > 0 || g.cut_top)) cp_async16(smem + L::XLT + 4 * tid, A.lamh + (ptrdiff_t)(a - 1) * g.W + c0 + 4 * tid);
@@ -352,26 +259,13 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
     if (l == 0) mbar_arrive_expect_tx(mbQ, kHaloBytes);
   };
 
-  if (first < T) {
-    if constexpr (Src::kBatch)
-      prefetch(first, dsc[0].A, first - dsc[0].base);
-    else
-      prefetch(first, S.args(first), S.local(first));
-  }
+  if (first < T) prefetch(first);
   uint32_t nsub = 0;             // subdomains started (phase of mbL)
-  int pa = -1, pc0 = 0, pgb = 0;  // previous subdomain, whose u and p1 wait in the out-buffer (TMA)
+  int pa = -1, pc0 = 0, pgb = 0;  // previous subdomain, whose u and p1 wait in the out-buffer
   uint32_t gred = 0;              // adaptive stop: reduction phases sent (and consumed) so far
 
   for (int t = first; t < T; t += stride, ++nsub) {
-    const LocalArgs& A = Src::kBatch ? dsc[cur].A : S.args(t);
-    const Grid g = A.g;
-    const int W2 = g.W + g.NC;
-    const float tau = A.tau;
-    const Strips out = Src::kBatch ? dsc[cur].out : S.out(t);
-    const int lt = Src::kBatch ? t - dsc[cur].base : S.local(t);
-    // batch: the next subdomain's image, loaded while this one's staging lands
-    const int img_next = (Src::kBatch && t + stride < T) ? S.image(t + stride) : 0;
-    const int a = lt / g.NC, b = lt - a * g.NC;
+    const int a = t / g.NC, b = t - a * g.NC;
     const int c0 = b * 128;
     const int gb = a * 128 + rank * BAND;
     const int o = b & 3;
@@ -386,21 +280,15 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
     const bool right_rows = s_rgt && w == 1 && l < BAND;
     const int r_slot = (l >> 2) * L::SLOT + 4 * 32 + 2 * (l & 1) + ((l >> 1) & 1);
     float pr_s = 0.f, hr_s = 0.f;
-    auto body = [&](auto fidc) {
-    constexpr int FID = decltype(fidc)::value;
     // pairs [column c][e]: rows (e, e + 2) of column j0 + c
     f32x2 U[4][2], P1[4][2], P2[4][2], H1[4][2], H2[4][2], Q1[4][2], Q2[4][2];
     uint32_t in_d = 0;  // bit 4c + r: pixel (row r, column j0 + c) lies in the inpainting domain
     int k_run = K;  // adaptive stop: inner iterations kept (< K: u of the last u-step undone)
 
     cp_async_wait_all();
-    if (TMA && !mbar_wait(mbL, nsub & 1)) timed_out = true;
+    if (!mbar_wait(mbL, nsub & 1)) timed_out = true;
     __syncthreads();  // staging landed; the previous subdomain's shared arrays are free
-    if (Src::kBatch && dsc[cur].img != cur_img) {  // visible after the barrier that follows the unpack
-      load_coef_dup(sCo, A.coef, K, tid, NT);
-      cur_img = dsc[cur].img;
-    }
-    if (TMA && tid == 0 && pa >= 0) {  // the previous subdomain's u and p1 bands
+    if (tid == 0 && pa >= 0) {  // the previous subdomain's u and p1 bands
       tma_store_2d(&M->u, smem + L::OU, pc0, pgb);
       tma_store_2d(&M->p1, smem + L::OP1, pc0, pgb + pa);
       tma_commit();
@@ -488,17 +376,7 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
       }
     }
     __syncthreads();  // staging consumed by every thread
-    int nxt = cur;  // slot of the next subdomain's descriptor
-    if constexpr (Src::kBatch) {
-      if (t + stride < T && img_next != dsc[cur].img) {
-        nxt = cur ^ 1;
-        load_batch_desc(&dsc[nxt], S.B, img_next, tid, NT);
-        __syncthreads();
-      }
-      if (t + stride < T) prefetch(t + stride, dsc[nxt].A, t + stride - dsc[nxt].base);
-    } else {
-      if (t + stride < T) prefetch(t + stride, S.args(t + stride), S.local(t + stride));
-    }
+    if (t + stride < T) prefetch(t + stride);
 
     // unrolled by two: the new dual values then land in the registers the old ones of
     // the previous iteration held, instead of being moved back every iteration
@@ -691,7 +569,7 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
       }
       if (ADAPT && k + 1 < K)  // this thread's residual sums, added up at the start of iteration k + 1
         *reinterpret_cast<float4*>(smem + L::PS + 4 * tid) = make_float4(lo2(AD), hi2(AD), lo2(AP), hi2(AP));
-      if (!ADAPT && TMA && k == K - 1 && tid == 0) tma_wait_read();  // the out-buffer is free for this subdomain's bands
+      if (!ADAPT && k == K - 1 && tid == 0) tma_wait_read();  // the out-buffer is free for this subdomain's bands
       __syncthreads();
     }
     const bool stopped = ADAPT && k_run < K;
@@ -708,13 +586,8 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
       const int gi = gb + lr0 + r;
       const float4 uv = make_float4(lane4(U[0][e], h), lane4(U[1][e], h), lane4(U[2][e], h), lane4(U[3][e], h));
       const float4 pv = make_float4(lane4(P1[0][e], h), lane4(P1[1][e], h), lane4(P1[2][e], h), lane4(P1[3][e], h));
-      if (TMA) {
-        if (!stopped) *reinterpret_cast<float4*>(smem + L::OU + (lr0 + r) * BW + j0) = uv;
-        *reinterpret_cast<float4*>(smem + L::OP1 + (lr0 + r) * BW + j0) = pv;
-      } else {
-        *reinterpret_cast<float4*>(A.u + (size_t)gi * g.W + c0 + j0) = uv;
-        *reinterpret_cast<float4*>(A.P1 + (size_t)(gi + a) * g.W + c0 + j0) = pv;
-      }
+      if (!stopped) *reinterpret_cast<float4*>(smem + L::OU + (lr0 + r) * BW + j0) = uv;
+      *reinterpret_cast<float4*>(smem + L::OP1 + (lr0 + r) * BW + j0) = pv;
       float* p2row = A.P2 + (size_t)gi * W2 + c0 + b + j0;
 #pragma unroll
       for (int c = 0; c < 4; ++c) p2row[c] = lane4(P2[c][e], h);
@@ -733,25 +606,12 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
       *reinterpret_cast<float4*>(A.P1 + (size_t)(a * 128 + 128 + a) * g.W + c0 + j0) = v;
       *reinterpret_cast<float4*>(out.SB + (size_t)a * g.W + c0 + j0) = v;
     }
-    if (TMA) {
-      tma_fence_smem();  // the out-buffer writes become visible to the tensor stores
-      pa = a;
-      pc0 = c0;
-      pgb = gb;
-    }
-    cur = nxt;
-    };  // body
-    if constexpr (Src::kBatch) {
-      switch (dsc[cur].fid) {
-        case FID_L2: body(FidC<FID_L2>{}); break;
-        case FID_L1: body(FidC<FID_L1>{}); break;
-        default: body(FidC<FID_SEG>{}); break;
-      }
-    } else {
-      S.dispatch(t, body);
-    }
+    tma_fence_smem();  // the out-buffer writes become visible to the tensor stores
+    pa = a;
+    pc0 = c0;
+    pgb = gb;
   }
-  if (TMA && pa >= 0) {  // the last subdomain's bands
+  if (pa >= 0) {  // the last subdomain's bands
     __syncthreads();
     if (tid == 0) {
       tma_store_2d(&M->u, smem + L::OU, pc0, pgb);
@@ -759,42 +619,29 @@ __device__ __forceinline__ void fused_mt4_body(const Src& S, const Mt4Maps* M, c
       tma_commit();
     }
   }
-  if (TMA && tid == 0) tma_wait_all();  // the stores are complete before the CTA's shared memory is released
+  if (tid == 0) tma_wait_all();  // the stores are complete before the CTA's shared memory is released
   cp_async_wait_all();
   cluster_arrive<true>();  // no CTA leaves while a neighbour may still write into it
   cluster_wait();
-  if (timed_out) atomicOr(S.err(), 1);
-}
-
-template <int FID, bool MASK>
-__global__ void __launch_bounds__(Mt4Layout::NT, 3) k_fused_mt4(const LocalArgs A) {
-  fused_mt4_body<MASK, false, false>(Mt4One<FID>{A}, nullptr, blockIdx.y, gridDim.y);
+  if (timed_out) atomicOr(A.err, 1);
 }
 
 template <int FID, bool MASK, bool ADAPT>
 __global__ void __launch_bounds__(Mt4Layout::NT, 3) k_fused_mt4t(const LocalArgs A, const __grid_constant__ Mt4Maps M) {
-  fused_mt4_body<MASK, true, ADAPT>(Mt4One<FID>{A}, &M, blockIdx.y, gridDim.y);
+  fused_mt4_body<FID, MASK, ADAPT>(A, &M, blockIdx.y, gridDim.y);
 }
 
-// the batch's work list: every subdomain with its image's descriptor and fidelity
-__global__ void __launch_bounds__(Mt4Layout::NT, 3) k_fused_mt4_batch(const BatchArgs B, int total) {
-  fused_mt4_body<false, false, false>(BatchTiles{B, total}, nullptr, blockIdx.y, gridDim.y);
+// clusters of each kernel resident at once, per device: [adaptive][FID * 2 + MASK]
+int& mt4_clusters(int dev, bool adapt, int fid, bool mask) {
+  static int n[64][2][6] = {};
+  return n[dev & 63][adapt ? 1 : 0][fid * 2 + (mask ? 1 : 0)];
 }
 
-// kernel kinds: cp.async copies, tensor copies, tensor copies with the adaptive stop
-enum Mt4Kind { kMt4Cp = 0, kMt4Tma = 1, kMt4TmaAdapt = 2 };
-
-// clusters of each kernel resident at once, per device: [kind][FID * 2 + MASK]
-int& mt4_clusters(int dev, int kind, int fid, bool mask) {
-  static int n[64][3][6] = {};
-  return n[dev & 63][kind][fid * 2 + (mask ? 1 : 0)];
-}
-
-cudaLaunchConfig_t mt4_config(int clusters, bool tma, cudaLaunchAttribute* attr) {
+cudaLaunchConfig_t mt4_config(int clusters, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(Mt4Layout::CL, clusters, 1);
   cfg.blockDim = dim3(Mt4Layout::NT, 1, 1);
-  cfg.dynamicSmemBytes = tma ? Mt4Layout::BYTES_TMA : Mt4Layout::BYTES;
+  cfg.dynamicSmemBytes = Mt4Layout::BYTES;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = Mt4Layout::CL;
   attr[0].val.clusterDim.y = 1;
@@ -804,14 +651,13 @@ cudaLaunchConfig_t mt4_config(int clusters, bool tma, cudaLaunchAttribute* attr)
   return cfg;
 }
 
-template <class Kern>
-cudaError_t prepare_kernel(Kern kern, int kind, int fid, bool mask) {
-  const bool tma = kind != kMt4Cp;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(tma ? Mt4Layout::BYTES_TMA : Mt4Layout::BYTES));
+template <int FID, bool MASK, bool ADAPT>
+cudaError_t prepare_mt4t() {
+  auto kern = k_fused_mt4t<FID, MASK, ADAPT>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Mt4Layout::BYTES);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = mt4_config(1024, tma, attr);
+  cudaLaunchConfig_t cfg = mt4_config(1024, attr);
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
     cudaGetLastError();
@@ -819,67 +665,23 @@ cudaError_t prepare_kernel(Kern kern, int kind, int fid, bool mask) {
   }
   int dev = 0;
   cudaGetDevice(&dev);
-  mt4_clusters(dev, kind, fid, mask) = n;
-  return cudaSuccess;
-}
-
-// clusters of the batch kernel resident at once, per device
-int& mt4_batch_clusters(int dev) {
-  static int n[64] = {};
-  return n[dev & 63];
-}
-
-// the batch kernel keeps its descriptors in the P1 out-buffer region: it is launched with
-// the tensor-copy kernel's shared-memory size
-static_assert(2 * sizeof(Mt4BatchDesc) <= sizeof(float) * Mt4Layout::BAND * Mt4Layout::BW &&
-                  Mt4Layout::OP1 >= Mt4Layout::MB + 6,
-              "two descriptors fit the P1 out-buffer, clear of the cp.async kernel's mbarriers");
-
-cudaError_t prepare_mt4_batch() {
-  cudaError_t e = cudaFuncSetAttribute(k_fused_mt4_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)Mt4Layout::BYTES_TMA);
-  if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = mt4_config(1024, true, attr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_fused_mt4_batch, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    n = 0;
-  }
-  int dev = 0;
-  cudaGetDevice(&dev);
-  mt4_batch_clusters(dev) = n;
+  mt4_clusters(dev, ADAPT, FID, MASK) = n;
   return cudaSuccess;
 }
 
 template <int FID, bool MASK>
 cudaError_t prepare_mt4_one() {
-  cudaError_t e = prepare_kernel(k_fused_mt4<FID, MASK>, kMt4Cp, FID, MASK);
-  if (e != cudaSuccess) return e;
-  if ((e = prepare_kernel(k_fused_mt4t<FID, MASK, false>, kMt4Tma, FID, MASK)) != cudaSuccess) return e;
-  return prepare_kernel(k_fused_mt4t<FID, MASK, true>, kMt4TmaAdapt, FID, MASK);
-}
-
-int mt4_grid(const LocalArgs& a, int kind, int fid, bool mask) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const int tiles = a.g.NR * a.g.NC;
-  int nc = mt4_clusters(dev, kind, fid, mask);
-  return (nc <= 0 || nc > tiles) ? tiles : nc;
-}
-
-template <int FID, bool MASK>
-cudaError_t launch_mt4_one(const LocalArgs& a, cudaStream_t st) {
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = mt4_config(mt4_grid(a, kMt4Cp, FID, MASK), false, attr);
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, k_fused_mt4<FID, MASK>, a);
+  const cudaError_t e = prepare_mt4t<FID, MASK, false>();
+  return e != cudaSuccess ? e : prepare_mt4t<FID, MASK, true>();
 }
 
 template <int FID, bool MASK, bool ADAPT>
 cudaError_t launch_mt4t_one(const LocalArgs& a, const Mt4Maps& maps, cudaStream_t st) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const int tiles = a.g.NR * a.g.NC, nc = mt4_clusters(dev, ADAPT, FID, MASK);
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = mt4_config(mt4_grid(a, ADAPT ? kMt4TmaAdapt : kMt4Tma, FID, MASK), true, attr);
+  cudaLaunchConfig_t cfg = mt4_config(nc <= 0 || nc > tiles ? tiles : nc, attr);
   cfg.stream = st;
   return cudaLaunchKernelEx(&cfg, k_fused_mt4t<FID, MASK, ADAPT>, a, maps);
 }
@@ -947,21 +749,8 @@ bool fused_mt4_supported(const LocalArgs& a) {
          al16(a.P1) && al16(a.P2) && al16(a.lamh) && al16(a.lamv) && al16(a.out.ST) && al16(a.out.SB);
 }
 
-int fused_mt4_max_inner() { return Mt4Layout::kMaxSmemCoef; }
-
-cudaError_t launch_fused_mt4_batch(const BatchArgs& B, int total_tiles, cudaStream_t st) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const int nc = mt4_batch_clusters(dev);
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = mt4_config((nc <= 0 || nc > total_tiles) ? total_tiles : nc, true, attr);  // smem size
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, k_fused_mt4_batch, B, total_tiles);
-}
-
 cudaError_t fused_mt4_prepare() {
   cudaError_t e;
-  if ((e = prepare_mt4_batch()) != cudaSuccess) return e;
   if ((e = prepare_mt4_one<FID_L2, false>()) != cudaSuccess) return e;
   if ((e = prepare_mt4_one<FID_L2, true>()) != cudaSuccess) return e;
   if ((e = prepare_mt4_one<FID_L1, false>()) != cudaSuccess) return e;
@@ -969,19 +758,10 @@ cudaError_t fused_mt4_prepare() {
   return prepare_mt4_one<FID_SEG, false>();
 }
 
-cudaError_t launch_fused_mt4(const LocalArgs& a, int fid, bool tma, cudaStream_t st) {
-  const bool m = a.mask != nullptr;
+cudaError_t launch_fused_mt4(const LocalArgs& a, int fid, cudaStream_t st) {
   Mt4Maps maps;
-  if (a.inner_tol2 > 0.0) {  // the adaptive stop exists in the tensor-copy kernel only
-    if (!encode_maps(a, &maps)) return cudaErrorNotSupported;
-    return launch_mt4t_fid<true>(a, maps, fid, st);
-  }
-  if (tma && encode_maps(a, &maps)) return launch_mt4t_fid<false>(a, maps, fid, st);
-  switch (fid) {
-    case FID_L2: return m ? launch_mt4_one<FID_L2, true>(a, st) : launch_mt4_one<FID_L2, false>(a, st);
-    case FID_L1: return m ? launch_mt4_one<FID_L1, true>(a, st) : launch_mt4_one<FID_L1, false>(a, st);
-    default: return launch_mt4_one<FID_SEG, false>(a, st);
-  }
+  if (!encode_maps(a, &maps)) return cudaErrorNotSupported;
+  return a.inner_tol2 > 0.0 ? launch_mt4t_fid<true>(a, maps, fid, st) : launch_mt4t_fid<false>(a, maps, fid, st);
 }
 
 }  // namespace ddtv

@@ -24,6 +24,8 @@ __global__ void k_interface_v4(int nh4, int nv4, float sigma, const float4* __re
                                const float4* __restrict__ cSR, const float4* __restrict__ cSL,
                                const float4* __restrict__ pSR, const float4* __restrict__ pSL,
                                float4* __restrict__ lamv) {
+  pdl_wait();     // the previous local solves
+  pdl_trigger();  // the next ones may start: they wait for this kernel before they read lambda
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nh4 + nv4; e += gridDim.x * blockDim.x) {
     const bool h = e < nh4;
     const int q = h ? e : e - nh4;
@@ -47,6 +49,8 @@ __global__ void k_interface_v1(int nh, int nv, float sigma, const float* __restr
                                const float* __restrict__ cSR, const float* __restrict__ cSL,
                                const float* __restrict__ pSR, const float* __restrict__ pSL,
                                float* __restrict__ lamv) {
+  pdl_wait();     // the previous local solves
+  pdl_trigger();  // the next ones may start: they wait for this kernel before they read lambda
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nh + nv; e += gridDim.x * blockDim.x) {
     if (e < nh) {
       lamh[e] = lam_step(lamh[e], sigma, cSB[e], pSB[e], cST[e], pST[e]);
@@ -97,6 +101,8 @@ __global__ void k_scatter(Grid g, Strips s, float* __restrict__ P1, float* __res
 // Batched multiplier update over every image of a batch (W, H multiples of 4): the
 // float4 elements of all images are numbered consecutively, image by image.
 __global__ void k_interface_batch(BatchIfaceArgs B, int total4) {
+  pdl_wait();     // the previous local solves
+  pdl_trigger();  // the next ones may start: they wait for this kernel before they read lambda
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total4; e += gridDim.x * blockDim.x) {
     int lo = 0, hi = B.n_img;  // find the image: elem_base[img] <= e < elem_base[img + 1]
     while (hi - lo > 1) {
@@ -125,6 +131,20 @@ __global__ void k_interface_batch(BatchIfaceArgs B, int total4) {
   }
 }
 
+// launches an update that may start while the previous kernel of the stream ends
+template <class... P, class... X>
+cudaError_t launch_pdl(void (*kern)(P...), int grid, int block, cudaStream_t st, X... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  pdl_attr(attr);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 int grid_for(long long n, int block) {
   long long b = (n + block - 1) / block;
   if (b < 1) b = 1;
@@ -141,21 +161,18 @@ cudaError_t launch_interface(const Grid& g, float sigma, Strips cur, Strips prev
   const int block = 256;
   if (g.W % 4 == 0 && g.H % 4 == 0) {
     const int nh4 = nh / 4, nv4 = nv / 4;
-    k_interface_v4<<<grid_for(nh4 + nv4, block), block, 0, st>>>(
-        nh4, nv4, sigma, (const float4*)cur.SB, (const float4*)cur.ST, (const float4*)prev.SB,
-        (const float4*)prev.ST, (float4*)lamh, (const float4*)cur.SR, (const float4*)cur.SL, (const float4*)prev.SR,
-        (const float4*)prev.SL, (float4*)lamv);
-  } else {
-    k_interface_v1<<<grid_for(nh + nv, block), block, 0, st>>>(nh, nv, sigma, cur.SB, cur.ST, prev.SB, prev.ST,
-                                                                lamh, cur.SR, cur.SL, prev.SR, prev.SL, lamv);
+    return launch_pdl(k_interface_v4, grid_for(nh4 + nv4, block), block, st, nh4, nv4, sigma, (const float4*)cur.SB,
+                      (const float4*)cur.ST, (const float4*)prev.SB, (const float4*)prev.ST, (float4*)lamh,
+                      (const float4*)cur.SR, (const float4*)cur.SL, (const float4*)prev.SR, (const float4*)prev.SL,
+                      (float4*)lamv);
   }
-  return cudaGetLastError();
+  return launch_pdl(k_interface_v1, grid_for(nh + nv, block), block, st, nh, nv, sigma, cur.SB, cur.ST, prev.SB,
+                    prev.ST, lamh, cur.SR, cur.SL, prev.SR, prev.SL, lamv);
 }
 
 cudaError_t launch_interface_batch(const BatchIfaceArgs& a, int total4, cudaStream_t st) {
   if (total4 == 0) return cudaSuccess;
-  k_interface_batch<<<grid_for(total4, 256), 256, 0, st>>>(a, total4);
-  return cudaGetLastError();
+  return launch_pdl(k_interface_batch, grid_for(total4, 256), 256, st, a, total4);
 }
 
 cudaError_t launch_extract_strips(const Grid& g, const float* P1, const float* P2, Strips s, cudaStream_t st) {
