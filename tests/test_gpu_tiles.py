@@ -42,3 +42,28 @@ def test_tile_kernel_equals_plain_path(cuda_lib, H, W, NR, NC):
         a, b = (_state(L, H, W, NR, NC, fid, mask, K, 3, path) for path in ("fused", "plain"))
         for k in a:
             assert torch.equal(a[k], b[k]), (fid, mask, K, k)
+
+
+@pytest.mark.parametrize("path", ["fused", "fulldim"])
+def test_loads_share_the_captured_loop(cuda_lib, path):
+    """The captured outer loop outlives a load: other data, and a mask that comes, changes
+    and goes, give what a new handle gives."""
+    from paper_1901_00682_gb300 import _lib as L
+    H, W, n = 200, 140, 9
+    rng = np.random.default_rng(5)
+    grid = (2, 2) if path == "fused" else (1, 1)
+    p = dict(sub_rows=grid[0], sub_cols=grid[1], alpha=8.0, inner_iters=6, path=path)
+    loads = [(torch.from_numpy(rng.random((H, W), dtype=np.float32)).cuda(),
+              torch.from_numpy((rng.random((H, W)) < 0.3).astype(np.uint8)).cuda() if m else None)
+             for m in (False, False, True, True, False)]
+    with L.Solver(L.make_params(H, W, **p)) as kept:
+        for f, m in loads:
+            kept.load(f, m)
+            kept.iterate(n)
+            with L.Solver(L.make_params(H, W, **p)) as new:
+                new.load(f, m)
+                new.iterate(n)
+                a, b = kept.get_state(), new.get_state()
+                torch.cuda.synchronize()
+            for k in a:
+                assert torch.equal(a[k], b[k]), k
