@@ -167,12 +167,28 @@ __device__ __forceinline__ void tile_store(const LocalArgs& A, const Strips& out
   }
 }
 
+// all bits set if -1 <= x <= 1 (not for NaN), else 0
+__device__ __forceinline__ uint32_t in_box(float x) {
+  uint32_t m;
+  asm("set.le.u32.f32 %0, %1, 0f3F800000;" : "=r"(m) : "f"(fabsf(x)));
+  return m;
+}
+
+constexpr int kTapeWords = 18;  // of the reverse pass, per thread and inner iteration
+
+// Reverse of the K iterations whose tape lies at `tape` (adj_tile.cuh).
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
+__device__ __forceinline__ void tile_reverse(const LocalArgs& A, const AdjArgs& Z, const int a, const int b, const int tid,
+                                             const int rank, const int CL, const float* tape, const uint32_t in_d,
+                                             bool& timed_out);
+
 // The local solve of subdomain (a, b) of the problem A, its interface strips written to
 // out, by CTA rank of CL.  CLU: the subdomain is a cluster (else one CTA: rank 0 of 1).
 // PAD: the subdomain may be smaller than the block (false: every subdomain fills it).
-template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
+// ADJ: record the tape (Z->tape) and run the reverse pass instead of the store.
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK, bool ADJ = false>
 __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out, const int a, const int b,
-                                           const int rank, const int CL) {
+                                           const int rank, const int CL, const AdjArgs* Z = nullptr) {
   using L = TileLayout<LPR, NW>;
   constexpr int NG = L::NG, BAND = L::BAND, BW = L::BW, NT = L::NT;
   extern __shared__ __align__(128) float smem[];
@@ -357,11 +373,25 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     ++phQ;
     if (cl == 0) mbar_arrive_expect_tx(mbQ, kHaloBytes);
   };
+  // tape of one CTA: 16 K NT words of ubar in thread order, K NT words of pass bits (bit 4c +
+  // r: the p1 dof of row r, column c; bit 16 + 4c + r: p2), K NT of the sides that other
+  // lanes update; `live`: the bits of active dofs
+  float* tape = nullptr;
+  uint32_t live = 0;
+  if (ADJ) {
+    tape = Z->tape + ((size_t)(a * g.NC + b) * CL + rank) * kTapeWords * K * NT;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int i = i0 + (q & 3), j = j0 + (q >> 2);
+      if (i < mr + (s_bot ? 1 : 0) && (i > 0 || s_top) && j < mc) live |= 1u << q;
+      if (i < mr && j < mc + (s_rgt ? 1 : 0) && (j > 0 || s_lft)) live |= 1u << (16 + q);
+    }
+  }
   // Two iterations per trip save the moves of the new dual values; with padding or a mask
   // the doubled code no longer fits the registers and the instruction cache (per outer
   // iteration, 2160 x 3840 in 120 x 128 subdomains: 144 us unrolled, 138 not; 4096 x 4096 in
   // 64 x 64: 207 and 219, with a mask 248 and 229).
-#pragma unroll(PAD || MASK ? 1 : 2)
+#pragma unroll(PAD || MASK || ADJ ? 1 : 2)
   for (int k = 0; k < K; ++k) {
     // (the coefficients of each half-step are loaded when it begins: registers)
     f32x2 SIG, UA, UBc, SS;
@@ -384,6 +414,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const ulonglong2 fc = *reinterpret_cast<const ulonglong2*>(myF + 4 * NT * c);
+        f32x2 ubar[2];
 #pragma unroll
         for (int ee = 0; ee < 2; ++ee) {
           const int e = 1 - ee;
@@ -394,6 +425,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
           const f32x2 right = c < 3 ? Q2[c + 1][e] : QRn[e];
           const f32x2 d = sub2(add2(bt, right), Q2[c][e]);  // div_px
           const f32x2 ub = fma2(SIG, d, U[c][e]);
+          ubar[e] = ub;
           const bool dl = MASK && ((in_d >> (4 * c + e)) & 1u), dh = MASK && ((in_d >> (4 * c + e + 2)) & 1u);
           f32x2 un;
           if (FID == FID_L2) {
@@ -408,6 +440,8 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
           }
           U[c][e] = un;
         }
+        if (ADJ)
+          *reinterpret_cast<ulonglong2*>(tape + ((size_t)(4 * k + c) * NT + tid) * 4) = make_ulonglong2(ubar[0], ubar[1]);
       }
       // u of the first padding column and row: 0 where the side is an interface (D_s u =
       // -u), u of the pixel before it where it is the image boundary (D_s u = 0: the dof
@@ -450,6 +484,10 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       PA = pk2(cb.x, cb.x), PC = pk2(cb.y, cb.y), PB = pk2(cb.z, cb.z), TH = pk2(cb.w, cb.w);
     }
     const Coef co{0.f, 0.f, 0.f, 0.f, lo2(PA), lo2(PC), lo2(PB), lo2(TH)};
+    uint32_t bits = 0;
+    auto record = [&](f32x2 t, int n) {  // pass bits n (low half) and n + 2 (high half)
+      if (ADJ) bits |= (in_box(lo2(t)) & (1u << n)) | (in_box(hi2(t)) & (4u << n));
+    };
     // ---- p-step: first the dofs that need no row above the group (in the first group that
     // row is the halo from the CTA above), then the first row's pbar1 and its push upwards
     {
@@ -462,6 +500,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         H0[c] = mul2(PB, h1.x);
         {
           const f32x2 tt = fma2(PC, sub2(U[c][1], U[c][0]), fma2(PA, P1[c][1], mul2(PB, h1.y)));  // p_target
+          record(tt, 4 * c + 1);
           const f32x2 pn = pk2(clamp_abs(lo2(tt), 1.f), clamp_abs(hi2(tt), 1.f));
           Q1[c][1] = fma2(TH, sub2(pn, P1[c][1]), pn);
           P1[c][1] = pn;
@@ -470,6 +509,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         for (int e = 0; e < 2; ++e) {
           const f32x2 leftu = c > 0 ? U[c - 1][e] : (e == 0 ? ul.x : ul.y);
           const f32x2 tt = fma2(PC, sub2(U[c][e], leftu), fma2(PA, P2[c][e], mul2(PB, e == 0 ? h2.x : h2.y)));
+          record(tt, 16 + 4 * c + e);
           const float ll = c == 0 ? lim_left : 1.f;
           const f32x2 pn = pk2(clamp_abs(lo2(tt), ll), clamp_abs(hi2(tt), ll));
           Q2[c][e] = fma2(TH, sub2(pn, P2[c][e]), pn);
@@ -485,6 +525,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         // rows (0, 2): the rows above (-1, 1) straddle the group above and pair 1
         const f32x2 du = pk2(lo2(U[c][0]) - uav[c], hi2(U[c][0]) - lo2(U[c][1]));
         const f32x2 tt = fma2(PC, du, fma2(PA, P1[c][0], H0[c]));
+        record(tt, 4 * c);
         const f32x2 pn = pk2(clamp_abs(lo2(tt), lim_top), clamp_abs(hi2(tt), 1.f));
         Q1[c][0] = fma2(TH, sub2(pn, P1[c][0]), pn);
         P1[c][0] = pn;
@@ -493,8 +534,12 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       if (G > 0) *reinterpret_cast<float4*>(sQ1 + G * BW + j0) = q;
       if (push_up) st_async_v4_f32(remote + 4 * (L::Q1 + NG * BW + j0), q.x, q.y, q.z, q.w, remote + 4 * L::MB + 8);
     }
+    uint32_t* const tapeM = ADJ ? reinterpret_cast<uint32_t*>(tape) + (size_t)(16 * K + k) * NT + tid : nullptr;
+    if (ADJ) *tapeM = bits & live;
+    uint32_t xbits = 0;
     if (right_lane) {  // Du = -u of the last column ((-pc) u = pc (-u) exactly)
       const float tt = fmaf(-co.pc, smem[L::UR + r_slot], fmaf(co.pa, pr_s, co.pb * hr_s));
+      if (ADJ) xbits |= in_box(tt) & 1u;
       const float pn = clamp_abs(tt, 1.f);
       smem[L::QL + r_slot] = fmaf(co.th, pn - pr_s, pn);
       pr_s = pn;
@@ -506,14 +551,30 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       float pB[4] = {pv.x, pv.y, pv.z, pv.w}, qB[4];
       const float hB[4] = {hv.x, hv.y, hv.z, hv.w}, uB[4] = {uv.x, uv.y, uv.z, uv.w};
 #pragma unroll
-      for (int c = 0; c < 4; ++c) p_update(pB[c], qB[c], -uB[c], hB[c], co);
+      for (int c = 0; c < 4; ++c) {
+        if (ADJ) xbits |= in_box(p_target(pB[c], -uB[c], hB[c], co)) & (2u << c);
+        p_update(pB[c], qB[c], -uB[c], hB[c], co);
+      }
       *reinterpret_cast<float4*>(smem + L::PBS + j0) = make_float4(pB[0], pB[1], pB[2], pB[3]);
       *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(qB[0], qB[1], qB[2], qB[3]);
     }
+    if (ADJ && (right_lane || bottom_lane)) tapeM[(size_t)K * NT] = xbits;
     __syncthreads();
   }
+  if (CLU && push_down) wait_q();  // drain the last pbar1 halo (not read)
+  if constexpr (ADJ) {
+    int tid2, a2 = a, b2 = b;  // the geometry again rather than in registers, as below
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid2));
+    asm volatile("" : "+r"(a2), "+r"(b2));
+    tile_reverse<LPR, NW, CLU, PAD, FID, MASK>(A, *Z, a2, b2, tid2, rank, CL, tape, in_d, timed_out);
+    if (CLU) {
+      if (timed_out) atomicOr(A.err, 1);
+      __syncwarp();
+      cluster_wait();
+    }
+    return;
+  }
   if (CLU) {
-    if (push_down) wait_q();  // drain the last pbar1 halo (not read)
     __syncwarp();
     cluster_arrive<false>();  // no CTA leaves while a neighbour may still write into it; the
                               // stores below hide the wait

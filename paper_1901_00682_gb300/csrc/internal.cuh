@@ -178,9 +178,17 @@ cudaError_t launch_fused_mt4(const LocalArgs& a, int fidelity, cudaStream_t st);
 cudaError_t fused_mt4_prepare();
 
 // ---- kernels_tile8.cu, kernels_tile16.cu, kernels_tile32.cu (fused_tile.cuh)
-// launch_tile_<LPR>_<NW>: the micro-tile kernel with LPR lanes per row group and NW warps
-// per CTA, cl CTAs per subdomain; pad: some subdomain does not fill the block of
-// 4 LPR columns x cl bands of 4 NW (32 / LPR) rows.
+// How the micro-tile kernels cover the subdomains of a grid: lpr lanes per row group (a
+// block 4 lpr columns wide), nw warps per CTA (bands of 4 nw (32 / lpr) rows), cl CTAs per
+// subdomain; pad: some subdomain does not fill the block.
+struct TilePlan {
+  int lpr, nw, cl;
+  bool pad;
+};
+// false if a subdomain is larger than 128 x 128
+bool tile_plan(const Grid& g, TilePlan* p);
+
+// launch_tile_<lpr>_<nw>
 cudaError_t launch_tile_8_2(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
 cudaError_t launch_tile_8_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
 cudaError_t launch_tile_16_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
@@ -247,9 +255,10 @@ int sum_f64_partials_count();
 // number of float64 partial sums the reverse u-kernel keeps for an image grid
 long long adj_alpha_slots(const Grid& g);
 
-// ---- kernels_adjoint_fused.cu
-// Reverse of one outer iteration's local solves, tape in shared memory: a = the local
-// solve's arguments (state after the multiplier update), z = the adjoint fields (Au,
+// ---- kernels_adjoint_fused.cu, kernels_adj_tile8.cu, kernels_adj_tile16.cu,
+// kernels_adj_tile32.cu (adj_tile.cuh)
+// Recomputation and reverse of one outer iteration's local solves: a = the local solve's
+// arguments (state after the multiplier update, not written), z = the adjoint fields (Au,
 // AP1/AP2 in: adjoints of u^{n+1}, p~^{n+1}; out: of u^n and of p~^n through the local
 // solve; APh1/APh2 out on the subdomain sides; Af +=; Aal += per (tile, CTA) slot).
 cudaError_t launch_adj_fused(const LocalArgs& a, const AdjArgs& z, int fidelity, cudaStream_t st);
@@ -259,6 +268,15 @@ size_t adj_fused_tape_floats(const Grid& g, int K);
 cudaError_t adj_fused_prepare();
 // alpha partial-sum slots the fused reverse kernel uses
 long long adj_alpha_slots_fused(const Grid& g);
+// launch_adj_tile_<lpr>_<nw>
+cudaError_t launch_adj_tile_8_2(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st);
+cudaError_t launch_adj_tile_8_4(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st);
+cudaError_t launch_adj_tile_16_4(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st);
+cudaError_t launch_adj_tile_16_8(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st);
+cudaError_t launch_adj_tile_32_4(const LocalArgs& a, const AdjArgs& z, int fid, int cl, bool pad, cudaStream_t st);
+cudaError_t prepare_adj_tile_8();
+cudaError_t prepare_adj_tile_16();
+cudaError_t prepare_adj_tile_32();
 
 // ---- kernels_misc.cu
 // u0 = f (0 on D) for L2/L1, 1/2 for SEG

@@ -392,25 +392,14 @@ cudaError_t prepare_fid() {
   return prepare_one<BW, R, TR, CL, FID_SEG, false, ADAPT>();
 }
 
-// The micro-tile kernel (fused_tile.cuh) for every subdomain shape up to 128 x 128, with
-// a fixed inner count.  Columns choose the lanes of a row group (a subdomain of mc
-// columns in a block of 32, 64 or 128), rows the warps of a CTA and the CTAs of a
-// cluster.  Up to 32 x 32 and 64 x 64 one CTA holds the subdomain: no halo leaves the
-// SM.  In a cluster of two 32-row CTAs, 64 x 64 subdomains take 256 us per outer
-// iteration of 10 inner ones at 4096^2 and 14.1 us at 128^2, in one CTA 217 and 13.0.
-// 128 columns run 16-row CTAs in clusters of up to 8: with 32 rows in 8 warps and
-// clusters of 4, 4096^2 takes 233 us instead of 215, and 120 x 128 subdomains (2160 x
-// 3840) 146 instead of 137.
-cudaError_t launch_tile_shape(const LocalArgs& a, int mr, int mc, int fid, cudaStream_t st) {
-  auto go = [&](cudaError_t (*launch)(const LocalArgs&, int, int, bool, cudaStream_t), int bw, int band) {
-    const int cl = (mr + band - 1) / band;
-    const bool pad = a.g.W != bw * a.g.NC || a.g.H != cl * band * a.g.NR;
-    return launch(a, fid, cl, pad, st);
-  };
-  if (mr < 1 || mc < 1 || mr > 128 || mc > 128) return cudaErrorInvalidValue;
-  if (mc <= 32) return mr <= 32 ? go(launch_tile_8_2, 32, 32) : go(launch_tile_8_4, 32, 64);
-  if (mc <= 64) return mr > 32 && mr <= 64 ? go(launch_tile_16_8, 64, 64) : go(launch_tile_16_4, 64, 32);
-  return go(launch_tile_32_4, 128, 16);
+// The micro-tile kernel (fused_tile.cuh), fixed inner count.
+cudaError_t launch_tile_shape(const LocalArgs& a, int fid, cudaStream_t st) {
+  TilePlan p;
+  if (!tile_plan(a.g, &p)) return cudaErrorInvalidValue;
+  if (p.lpr == 8) return p.nw == 2 ? launch_tile_8_2(a, fid, p.cl, p.pad, st) : launch_tile_8_4(a, fid, p.cl, p.pad, st);
+  if (p.lpr == 16)
+    return p.nw == 8 ? launch_tile_16_8(a, fid, p.cl, p.pad, st) : launch_tile_16_4(a, fid, p.cl, p.pad, st);
+  return launch_tile_32_4(a, fid, p.cl, p.pad, st);
 }
 
 // size class of the cluster-barrier kernel for a tile shape (up to 32 x 32, 64 x 64 and
@@ -423,6 +412,25 @@ int pick(int mr, int mc) {
 }
 
 }  // namespace
+
+// Columns choose the lanes of a row group (a subdomain of mc
+// columns in a block of 32, 64 or 128), rows the warps of a CTA and the CTAs of a
+// cluster.  Up to 32 x 32 and 64 x 64 one CTA holds the subdomain: no halo leaves the
+// SM.  In a cluster of two 32-row CTAs, 64 x 64 subdomains take 256 us per outer
+// iteration of 10 inner ones at 4096^2 and 14.1 us at 128^2, in one CTA 217 and 13.0.
+// 128 columns run 16-row CTAs in clusters of up to 8: with 32 rows in 8 warps and
+// clusters of 4, 4096^2 takes 233 us instead of 215, and 120 x 128 subdomains (2160 x
+// 3840) 146 instead of 137.
+bool tile_plan(const Grid& g, TilePlan* p) {
+  const int mr = (g.H + g.NR - 1) / g.NR, mc = (g.W + g.NC - 1) / g.NC;  // the largest subdomain
+  if (mr > 128 || mc > 128) return false;
+  p->lpr = mc <= 32 ? 8 : (mc <= 64 ? 16 : 32);
+  p->nw = p->lpr == 8 && mr <= 32 ? 2 : (p->lpr == 16 && mr > 32 && mr <= 64 ? 8 : 4);
+  const int bw = 4 * p->lpr, band = 4 * p->nw * (32 / p->lpr);
+  p->cl = (mr + band - 1) / band;
+  p->pad = g.W != bw * g.NC || g.H != p->cl * band * g.NR;
+  return true;
+}
 
 void fused_max_tile(int* rows, int* cols) {
   *rows = 128;
@@ -478,7 +486,7 @@ cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStr
     if (variant == 2 && fused_mt_supported(a)) return launch_fused_mt(a, fid, st);
     if (variant == 3) return launch_fid<128, 8, 2, 8, false>(a, fid, st);
   }
-  return launch_tile_shape(a, mr, mc, fid, st);
+  return launch_tile_shape(a, fid, st);
 }
 
 }  // namespace ddtv
