@@ -247,6 +247,9 @@ int dd_tv_batch_create(dd_tv_batch** out, const dd_tv_batch_image* images, int n
     A.u = (float*)(b->arena + off_u[i]);
     A.P1 = (float*)(b->arena + off_p1[i]);
     A.P2 = (float*)(b->arena + off_p2[i]);
+    A.u0 = A.u;
+    A.P10 = A.P1;
+    A.P20 = A.P2;
     A.lamh = (const float*)(b->arena + off_lh[i]);
     A.lamv = (const float*)(b->arena + off_lv[i]);
     A.coef = (const Coef*)(b->arena + off_co[i]);

@@ -54,6 +54,8 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+// (the assembler fuses a packed product into a packed sum that uses it; where the product is to
+// be rounded first, round2)
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   f32x2 r;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -65,6 +67,10 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+
+// a * b rounded: nz is a pair of -0 that the assembler cannot see to be one (it would turn the
+// operation into the product again); it keeps every product, its sign included
+__device__ __forceinline__ f32x2 round2(f32x2 a, f32x2 b, f32x2 nz) { return fma2(a, b, nz); }
 
 template <bool RELEASE>
 __device__ __forceinline__ void cluster_arrive() {

@@ -261,10 +261,10 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     const bool vec = (g.W & 3) == 0 && (c0 & 3) == 0;
     float h1[4][4], h2[4][4], fv[4][4];
     float u[4][4], p1[4][4], p2[4][4];
-    const float* gu = A.u + (size_t)(r0 + i0) * g.W + c0 + j0;
+    const float* gu = A.u0 + (size_t)(r0 + i0) * g.W + c0 + j0;
     const float* gf = A.f + (size_t)(r0 + i0) * g.W + c0 + j0;
-    const float* g1 = A.P1 + (size_t)(r0 + i0 + a) * g.W + c0 + j0;
-    const float* g2 = A.P2 + (size_t)(r0 + i0) * W2 + c0 + b + j0;
+    const float* g1 = A.P10 + (size_t)(r0 + i0 + a) * g.W + c0 + j0;
+    const float* g2 = A.P20 + (size_t)(r0 + i0) * W2 + c0 + b + j0;
     const uint8_t* gm = MASK ? A.mask + (size_t)(r0 + i0) * g.W + c0 + j0 : nullptr;
     uint32_t mb[4] = {0, 0, 0, 0};  // mask bytes of the lane's rows
     if (vec && i0 + 3 < mr && j0 + 3 < mc) {
@@ -301,8 +301,8 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     const bool bottom_fill = last_group && fill_r && s_bot;
     float qb[4], lb[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) qb[c] = c < nb ? A.P1[(size_t)(r0 + ib + a) * g.W + c0 + j0 + c] : 0.f;
-    if (right_lane) pr_s = A.P2[(size_t)(r0 + rank * BAND + rr) * W2 + c0 + BW + b];
+    for (int c = 0; c < 4; ++c) qb[c] = c < nb ? A.P10[(size_t)(r0 + ib + a) * g.W + c0 + j0 + c] : 0.f;
+    if (right_lane) pr_s = A.P20[(size_t)(r0 + rank * BAND + rr) * W2 + c0 + BW + b];
 
     pdl_wait();  // the multipliers, of the sides this lane holds
     const bool top = i0 == 0 && s_top, left = j0 == 0 && s_lft, bot = pad_r && s_bot, rgt = pad_c && s_rgt;
@@ -373,9 +373,9 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     ++phQ;
     if (cl == 0) mbar_arrive_expect_tx(mbQ, kHaloBytes);
   };
-  // tape of one CTA: 16 K NT words of ubar in thread order, K NT words of pass bits (bit 4c +
-  // r: the p1 dof of row r, column c; bit 16 + 4c + r: p2), K NT of the sides that other
-  // lanes update; `live`: the bits of active dofs
+  // tape of one CTA, per iteration: 16 NT words of ubar in thread order, NT words of pass bits
+  // (bit 4c + r: the p1 dof of row r, column c; bit 16 + 4c + r: p2), NT of the sides that
+  // other lanes update; `live`: the bits of active dofs
   float* tape = nullptr;
   uint32_t live = 0;
   if (ADJ) {
@@ -441,7 +441,8 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
           U[c][e] = un;
         }
         if (ADJ)
-          *reinterpret_cast<ulonglong2*>(tape + ((size_t)(4 * k + c) * NT + tid) * 4) = make_ulonglong2(ubar[0], ubar[1]);
+          *reinterpret_cast<ulonglong2*>(tape + (size_t)k * kTapeWords * NT + 4 * NT * c + 4 * tid) =
+              make_ulonglong2(ubar[0], ubar[1]);
       }
       // u of the first padding column and row: 0 where the side is an interface (D_s u =
       // -u), u of the pixel before it where it is the image boundary (D_s u = 0: the dof
@@ -534,7 +535,8 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       if (G > 0) *reinterpret_cast<float4*>(sQ1 + G * BW + j0) = q;
       if (push_up) st_async_v4_f32(remote + 4 * (L::Q1 + NG * BW + j0), q.x, q.y, q.z, q.w, remote + 4 * L::MB + 8);
     }
-    uint32_t* const tapeM = ADJ ? reinterpret_cast<uint32_t*>(tape) + (size_t)(16 * K + k) * NT + tid : nullptr;
+    uint32_t* const tapeM =
+        ADJ ? reinterpret_cast<uint32_t*>(tape) + (size_t)k * kTapeWords * NT + 16 * NT + tid : nullptr;
     if (ADJ) *tapeM = bits & live;
     uint32_t xbits = 0;
     if (right_lane) {  // Du = -u of the last column ((-pc) u = pc (-u) exactly)
@@ -558,7 +560,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       *reinterpret_cast<float4*>(smem + L::PBS + j0) = make_float4(pB[0], pB[1], pB[2], pB[3]);
       *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(qB[0], qB[1], qB[2], qB[3]);
     }
-    if (ADJ && (right_lane || bottom_lane)) tapeM[(size_t)K * NT] = xbits;
+    if (ADJ && (right_lane || bottom_lane)) tapeM[NT] = xbits;
     __syncthreads();
   }
   if (CLU && push_down) wait_q();  // drain the last pbar1 halo (not read)

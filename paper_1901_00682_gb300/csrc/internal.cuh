@@ -39,6 +39,9 @@ struct LocalArgs {
   float* u;              // H x W
   float* P1;             // (H + NR) x W torn
   float* P2;             // H x (W + NC) torn
+  // the state the micro-tile kernel starts from (u, P1, P2 themselves, or another set of
+  // arrays with zeros on the image boundary); the other kernels work in place
+  const float *u0, *P10, *P20;
   const float* lamh;     // (NR-1) x W
   const float* lamv;     // (NC-1) x H
   Strips out;            // strips of p~^{n+1} (written at the end)
@@ -106,6 +109,7 @@ struct AdjArgs {
   float *ALh, *ALv;        // lambda
   Strips APp;              // interface values of p~^{n-1}
   float* tape;             // tile-fused reverse kernel: adj_fused_tape_floats(g, K) floats
+  float neg_zero;          // -0.0f (fused_common.cuh round2)
 };
 
 // Programmatic dependent launch.  A kernel launched with pdl_attr may start while its
@@ -154,6 +158,9 @@ cudaError_t launch_fused_local(const LocalArgs& a, int fidelity, int variant, cu
 // Sets the shared-memory opt-in of every fused configuration on the current device
 // (called at handle creation, outside any stream capture).
 cudaError_t fused_prepare();
+// Whether launch_fused_local(a, ., variant) with a fixed inner count reads a.u0, a.P10, a.P20
+// (rather than working in place on a.u, a.P1, a.P2).
+bool fused_out_of_place(const Grid& g, int variant);
 // Largest tile (rows, cols) the fused kernel supports.
 void fused_max_tile(int* rows, int* cols);
 // Number of hardware mappings available for 128 x 128 tiles.

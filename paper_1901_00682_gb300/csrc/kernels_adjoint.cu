@@ -264,6 +264,8 @@ __global__ void __launch_bounds__(kBlock) k_adj_p(Grid g, const int4* __restrict
 __global__ void k_adj_interface(Grid g, float sigma, float tau, float* __restrict__ AP1, float* __restrict__ AP2,
                                 const float* __restrict__ APh1, const float* __restrict__ APh2,
                                 float* __restrict__ ALh, float* __restrict__ ALv, Strips APp) {
+  pdl_wait();     // the reverse of the local solves
+  pdl_trigger();  // the next outer iteration's recomputation may start
   const int nh = (g.NR - 1) * g.W, nv = (g.NC - 1) * g.H;
   const int W2 = g.W + g.NC;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nh + nv; e += gridDim.x * blockDim.x) {
@@ -324,12 +326,22 @@ __global__ void __launch_bounds__(kBlock) k_sum_f64(const double* __restrict__ x
     last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (last) {
+    // the last block adds the partials: thread t takes t, t + blockDim, ..., then as above (one
+    // thread adding them in a row took 30 us)
     __threadfence();
     double t = 0.0;
-    for (int q = 0; q < (int)gridDim.x; ++q) t += ((volatile double*)partials)[q];
-    out[0] = t;
-    *counter = 0u;
+    for (int q = threadIdx.x; q < (int)gridDim.x; q += blockDim.x) t += ((volatile double*)partials)[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double total = 0.0;
+      for (int w = 0; w < kBlock / 32; ++w) total += sw[w];
+      out[0] = total;
+      *counter = 0u;
+    }
   }
 }
 
@@ -388,8 +400,16 @@ cudaError_t launch_adj_interface(const AdjArgs& r, float sigma, float tau, cudaS
   const Grid& g = r.g;
   const int n = (g.NR - 1) * g.W + (g.NC - 1) * g.H;
   if (n == 0) return cudaSuccess;
-  k_adj_interface<<<nblocks(n), kBlock, 0, st>>>(g, sigma, tau, r.AP1, r.AP2, r.APh1, r.APh2, r.ALh, r.ALv, r.APp);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nblocks(n), 1, 1);
+  cfg.blockDim = dim3(kBlock, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  pdl_attr(attr);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_adj_interface, g, sigma, tau, r.AP1, r.AP2, (const float*)r.APh1,
+                            (const float*)r.APh2, r.ALh, r.ALv, r.APp);
 }
 
 cudaError_t launch_adj_initial(const AdjArgs& r, cudaStream_t st) {

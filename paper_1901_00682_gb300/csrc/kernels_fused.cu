@@ -461,6 +461,10 @@ cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, in
   return tile == 64 ? launch_tile_batch_64(B, total_tiles, overlap, st) : cudaErrorInvalidValue;
 }
 
+bool fused_out_of_place(const Grid& g, int variant) {
+  return variant == 0 || !(g.H == 128 * g.NR && g.W == 128 * g.NC);  // the micro-tile kernel
+}
+
 cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStream_t st) {
   // largest tile of the (ragged) partition
   const int mr = (a.g.H + a.g.NR - 1) / a.g.NR, mc = (a.g.W + a.g.NC - 1) / a.g.NC;
