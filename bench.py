@@ -170,7 +170,7 @@ def kernel_source_sha():
     """First 16 hex digits of the SHA-256 of the fused kernel's sources (the kernel file
     and the device headers it includes), to tell whether a capture is still current."""
     h = hashlib.sha256()
-    for name in ("kernels_fused_mt4.cu", "fused_common.cuh", "pointwise.cuh"):
+    for name in ("fused_tile.cuh", "fused_common.cuh", "pointwise.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1901_00682_gb300", "csrc", name), "rb").read())
     return h.hexdigest()[:16]
 
@@ -273,7 +273,7 @@ def measure_tvl1(dev, stream):
             "ms_500_outer": ms, "value": S * S * INNER * OUT / (ms * 1e-3) / 1e6, "unit": UNIT,
             "energy_500": J500,
             "roofline": {"bound": "smem", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-                         "avg_launch_ms": local_ms, "kernel": "k_fused_mt4t<L1, mask>"},
+                         "avg_launch_ms": local_ms, "kernel": "k_tile<L1, mask>"},
             "energy_vs_oracle_20_outer": {"gpu": J20, "oracle": Jo, "rel_diff": abs(J20 - Jo) / abs(Jo)}}
 
 
@@ -412,7 +412,7 @@ def run_sharded(args, rank, world, local, dev, stream, pg):
     achieved = bytes_per_launch / (local_avg_ms * 1e-3) / 1e9
     roofline = {"bound": "smem", "achieved": achieved, "peak": smem_peak, "unit": "GB/s",
                 "frac": achieved / smem_peak, "traffic": None,
-                "kernel": "fused local solver of the rank's 4096x4096 block (k_fused_mt4t)",
+                "kernel": "fused local solver of the rank's 4096x4096 block (k_tile)",
                 "peak_source": "measured live: ld.shared probe kernel (dd_tv_measure_smem_bandwidth)",
                 "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_ms": local_avg_ms}
     row_tv = args.steps // ENERGY_EVERY if rank < world - 1 else 0   # the cut's TV kernel of each energy
@@ -547,7 +547,7 @@ def run_ours(args):
         "traffic_note": ("DRAM bytes per launch from the committed ncu capture; the bound is shared memory, "
                          "the HBM state stream is hbm_state_stream below (writes still in L2 at kernel exit "
                          "are not counted by ncu)") if traffic else None,
-        "kernel": "fused local solver (k_fused_mt4t: persistent clusters of 8 CTAs x 128 threads, 3 CTAs per SM, one 128x128 subdomain per cluster at a time, 4x4 pixel micro-tile per thread, state moved by tensor copies)",
+        "kernel": "fused local solver (k_tile: a cluster of 8 CTAs x 128 threads per 128x128 subdomain, 4 CTAs per SM, 4x4 pixel micro-tile per thread)",
         "peak_source": "measured live: ld.shared probe kernel (dd_tv_measure_smem_bandwidth)",
         "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_ms": local_avg_ms,
         "occupancy": ({"achieved_warps_frac": prof.get("warps_active_frac"),
@@ -698,9 +698,8 @@ def run_ours(args):
                  "ms_per_outer": ms_b,
                  "value": bt.pixels() * INNER / (ms_b * 1e-3) / 1e6, "unit": UNIT,
                  "launch": f"one CUDA graph of {n_b} outer iterations (2 kernels per outer iteration: batched "
-                           "multiplier update, persistent clusters over the (image, subdomain) work list)",
-                 "kernel": "k_fused_mt4_batch: the 4x4 micro-tile kernel over the work list (cp.async copies, "
-                           "per-image descriptors cached in shared memory)"}
+                           "multiplier update, a cluster per entry of the (image, subdomain) work list)",
+                 "kernel": "k_tile_batch: the 4x4 micro-tile kernel over the work list"}
         smem_peak_b = L.measure_smem_bandwidth()
         ach_b = SMEM_BYTES_PER_PX_ITER * bt.pixels() * INNER / (ms_b * 1e-3) / 1e9
         batch["roofline"] = {"bound": "smem", "achieved": ach_b, "peak": smem_peak_b, "unit": "GB/s",

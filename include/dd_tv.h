@@ -83,9 +83,8 @@ typedef struct {
   int path;               /* dd_tv_path                                                    */
   int variant;            /* fused path, hardware mapping of exact 128 x 128 subdomains:
                              0 the micro-tile kernel of every other tile shape
-                             (default); 1 persistent 4 x 4 micro-tiles, state moved by
-                             tensor copies; 2 persistent 2 x 4 micro-tiles; 3 one
-                             cluster per subdomain with cluster barriers.  The
+                             (default); 1 the same; 2 persistent 2 x 4 micro-tiles; 3
+                             one cluster per subdomain with cluster barriers.  The
                              arithmetic and results do not depend on it               */
   double inner_tol;       /* >= 0.  0: every local solve runs inner_iters iterations.  > 0:
                              adaptive inner stopping (Section 5, eq. stop_inner1): a

@@ -11,7 +11,7 @@
 // subdomains up to 32, 64, 128 columns wide), so a warp holds 32 / LPR row groups and a
 // CTA of NW warps a band of BAND = 4 NW (32 / LPR) rows.  A subdomain is one CTA, or a
 // cluster of the fewest CTAs whose bands cover its rows; halo rows then travel with
-// st.async counted on mbarriers (bounded waits), as in kernels_fused_mt4.cu.  Registers
+// st.async counted on mbarriers (bounded waits), as in kernels_fused_mt.cu.  Registers
 // hold u, the dual dofs p1 (top edge) and p2 (left edge) and their extrapolations; f and
 // the proximal centres, read once per inner iteration by the thread that owns them, wait
 // in shared memory in the owner's order, which keeps a thread within 128 registers and
@@ -25,17 +25,19 @@
 // lane that holds the column or row branches on its place in the micro-tile; as selects the
 // pinning cost half as many instructions again as the iteration.)  Where
 // the subdomain fills the block (no padding) the sides are updated by lanes of other
-// warps, as in kernels_fused_mt4.cu.  A side on the image boundary is kept at 0 by
+// warps.  A side on the image boundary is kept at 0 by
 // clamping its dofs to [-0, 0].
 //
 // Measured per outer iteration of 10 inner ones, multiplier update included, against
 // the kernels it replaced (the cluster-barrier kernel, a column of 8 pixels per thread;
-// for exact 128 x 128 subdomains the persistent kernel of kernels_fused_mt4.cu): 1080 x 1920
+// for exact 128 x 128 subdomains persistent clusters with three CTAs per SM that moved the
+// state by tensor copies): 1080 x 1920
 // in 120 x 128 subdomains 106 -> 41 us, 2160 x 3840 448 -> 137, 2999 x 3001 in 125 x 125/126
 // 477 -> 158, 4096 x 4096 in 64 x 64 572 -> 214 and in 32 x 32 527 -> 187, 512 x 512 in 32 x 32
 // 19.1 -> 8.9, 128 x 128 in 64 x 64 21.1 -> 11.9, 321 x 481 in 107 x 120/121 25.8 -> 14.5; in 128 x
 // 128 subdomains 512 x 512 14.0 -> 13.0, 1024 x 1024 22.7 -> 18.6, 4096 x 4096 231 -> 216, a
-// batch of 64 images (168 Mpixel) 2730 -> 2280.
+// batch of 64 images (168 Mpixel) 2730 -> 2280; with the adaptive stop, 1024 x 1024 and 18.7
+// inner iterations on average, 54 -> 43.
 //
 // Every value is computed with the operations of the scalar iteration in its order
 // (pointwise.cuh), so the results are those of the plain path bit for bit.
@@ -74,6 +76,22 @@ struct TileLayout {
   static_assert(Q1 % 4 == 0 && UR % 4 == 0 && QL % 4 == 0 && F % 4 == 0 && CO % 4 == 0 && PBS % 4 == 0 && MB % 2 == 0,
                 "16-byte alignment of the vector accesses");
   static_assert(kRightThread + BAND <= NT, "a thread per right-side dof");
+};
+
+// Shared memory of the adaptive inner stop, behind the layout above.
+template <int LPR, int NW>
+struct AdaptTileLayout {
+  using L = TileLayout<LPR, NW>;
+  static constexpr int kMaxCL = 8;
+  static constexpr int OU = (L::MB + 4 + 3) & ~3;    // u of the iteration before, thread order
+  static constexpr int PS = OU + 16 * L::NT;         // every thread's residual sums
+  static constexpr int RED = PS + 4 * L::NT;         // two buffers (parity of the phase) of a pair per CTA
+  static constexpr int STOP = RED + 2 * 2 * kMaxCL;  // the CTA's decision
+  static constexpr int MBR = STOP + 2;               // two mbarriers, one per parity
+  static constexpr size_t BYTES = sizeof(float) * MBR + 16;
+  static constexpr int kReduceWarp = NW - 1;         // adds the CTA's residual sums and sends them
+  static constexpr int kDecideWarp = 1;              // takes the stop decision
+  static_assert(RED % 2 == 0 && MBR % 2 == 0, "8-byte alignment of the pairs and mbarriers");
 };
 
 // four consecutive floats (16-byte aligned)
@@ -186,7 +204,19 @@ __device__ __forceinline__ void tile_reverse(const LocalArgs& A, const AdjArgs& 
 // out, by CTA rank of CL.  CLU: the subdomain is a cluster (else one CTA: rank 0 of 1).
 // PAD: the subdomain may be smaller than the block (false: every subdomain fills it).
 // ADJ: record the tape (Z->tape) and run the reverse pass instead of the store.
-template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK, bool ADJ = false>
+//
+// ADAPT: adaptive inner stopping (Section 5, eq. stop_inner1).  Every thread sums (p^{k+1} -
+// p^k)^2 and (p^{k+1})^2 over its dofs in the p-step of iteration k (packed float32 pairs) and
+// leaves the sums in shared memory.  At the start of iteration k + 1 one warp adds the CTA's
+// sums (float32, fixed order) and sends the CTA's pair with st.async to slot `rank` of every
+// CTA of the cluster, counted on one of two mbarriers (by the parity of the phase, so that a
+// phase is always consumed everywhere before its barrier is armed again).  Before the
+// barrier between the u-step and the p-step of iteration k + 1, one warp per CTA waits for the
+// pairs and adds them in a fixed tree: every CTA takes the same decision without a cluster
+// barrier.  On "stop" the u-step of iteration k + 1 is undone (each iteration first copies u
+// to shared memory), its u halo is drained and the p-step is skipped: the solve keeps k + 1
+// inner iterations, as the rule prescribes.
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK, bool ADJ = false, bool ADAPT = false>
 __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out, const int a, const int b,
                                            const int rank, const int CL, const AdjArgs* Z = nullptr) {
   using L = TileLayout<LPR, NW>;
@@ -196,6 +226,9 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   float* sQ1 = smem + L::Q1;
   float* sCo = smem + L::CO;
   const uint32_t mbU = smem_addr(smem + L::MB), mbQ = mbU + 8;
+  using AD = AdaptTileLayout<LPR, NW>;
+  const uint32_t mbR = smem_addr(smem + AD::MBR);
+  static_assert(!ADAPT || (CLU && !PAD && !ADJ && NW > 2), "the adaptive stop: clusters of full blocks");
 
   const Grid g = A.g;
   const int r0 = PAD ? part_start(a, g.H, g.NR) : a * CL * BAND, mr = PAD ? part_start(a + 1, g.H, g.NR) - r0 : CL * BAND;
@@ -232,6 +265,12 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       // the first phases, armed before any neighbour may complete them
       if (rank > 0) mbar_arrive_expect_tx(mbU, kHaloBytes);
       if (rank + 1 < CL) mbar_arrive_expect_tx(mbQ, kHaloBytes);
+      if (ADAPT) {
+        for (int q = 0; q < 2; ++q) {
+          mbar_init(mbR + 8 * q, 1);
+          mbar_arrive_expect_tx(mbR + 8 * q, 8 * CL);
+        }
+      }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -391,8 +430,40 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   // the doubled code no longer fits the registers and the instruction cache (per outer
   // iteration, 2160 x 3840 in 120 x 128 subdomains: 144 us unrolled, 138 not; 4096 x 4096 in
   // 64 x 64: 207 and 219, with a mask 248 and 229).
-#pragma unroll(PAD || MASK || ADJ ? 1 : 2)
+  int k_run = K;  // inner iterations kept (ADAPT; < K: u of the last u-step undone)
+#pragma unroll(PAD || MASK || ADJ || ADAPT ? 1 : 2)
   for (int k = 0; k < K; ++k) {
+    // this thread's sums of (p^{k+1} - p^k)^2 and (p^{k+1})^2
+    f32x2 SD = 0ull, SP = 0ull;
+    auto residual = [&](f32x2 pn, f32x2 po) {
+      if (ADAPT) {
+        const f32x2 d = sub2(pn, po);
+        SD = fma2(d, d, SD);
+        SP = fma2(pn, pn, SP);
+      }
+    };
+    if (ADAPT && k > 0) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<ulonglong2*>(smem + AD::OU + 4 * (NT * c + tid)) = make_ulonglong2(U[c][0], U[c][1]);
+      if (w == AD::kReduceWarp) {
+        // the CTA's residual sums of iteration k - 1 to every CTA of the cluster
+        f32x2 D = 0ull, P = 0ull;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+          const float4 r = *reinterpret_cast<const float4*>(smem + AD::PS + 4 * (l + 32 * q));
+          D = add2(D, pk2(r.x, r.y));
+          P = add2(P, pk2(r.z, r.w));
+        }
+        f32x2 v = pk2(lo2(D) + hi2(D), lo2(P) + hi2(P));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = add2(v, __shfl_xor_sync(0xffffffffu, v, o));
+        const uint32_t par = (k - 1) & 1;
+        if (l < CL)  // lane l to CTA l, slot rank
+          st_async_v2(map_rank(s0 + 4 * (AD::RED + 2 * AD::kMaxCL * par + 2 * rank), l), lo2(v), hi2(v),
+                      map_rank(mbR + 8 * par, l));
+      }
+    }
     // (the coefficients of each half-step are loaded when it begins: registers)
     f32x2 SIG, UA, UBc, SS;
     if (coef_smem) {
@@ -474,7 +545,25 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       if (G < NG - 1) *reinterpret_cast<float4*>(sUB + (G + 1) * BW + j0) = ul;
       *reinterpret_cast<ulonglong2*>(myUR) = make_ulonglong2(U[3][0], U[3][1]);
     }
+    if (ADAPT && k > 0 && w == AD::kDecideWarp) {  // on iteration k - 1
+      const uint32_t par = (k - 1) & 1;
+      if (!mbar_wait(mbR + 8 * par, ((k - 1) >> 1) & 1)) timed_out = true;
+      f32x2 v = l < CL ? *reinterpret_cast<const f32x2*>(smem + AD::RED + 2 * AD::kMaxCL * par + 2 * l) : 0ull;
+#pragma unroll
+      for (int o = AD::kMaxCL / 2; o > 0; o >>= 1) v = add2(v, __shfl_xor_sync(0xffffffffu, v, o));
+      if (l == 0) {
+        mbar_arrive_expect_tx(mbR + 8 * par, 8 * CL);  // the barrier's next phase
+        const float td = lo2(v), tp = hi2(v);
+        *reinterpret_cast<int*>(smem + AD::STOP) = (timed_out || tp == 0.f || td < (float)A.inner_tol2 * tp) ? 1 : 0;
+      }
+    }
     __syncthreads();
+    if (ADAPT && k > 0 && *reinterpret_cast<const int*>(smem + AD::STOP)) {
+      // keep iterations 0 .. k - 1; the u halo this u-step sent is drained
+      k_run = k;
+      if (push_up) wait_u();
+      break;
+    }
     f32x2 PA, PC, PB, TH;
     if (coef_smem) {
       const ulonglong2 cf2 = *reinterpret_cast<const ulonglong2*>(sCo + 16 * k + 8);
@@ -494,27 +583,43 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     {
       const ulonglong2 ul = *reinterpret_cast<const ulonglong2*>(myUR - 4);  // right column of the lane to the left
       f32x2 H0[4];  // the proximal centres of rows (0, 2), for the second part
+      auto p1_odd = [&](int c, f32x2 h) {  // rows (1, 3)
+        const f32x2 tt = fma2(PC, sub2(U[c][1], U[c][0]), fma2(PA, P1[c][1], mul2(PB, h)));  // p_target
+        record(tt, 4 * c + 1);
+        const f32x2 pn = pk2(clamp_abs(lo2(tt), 1.f), clamp_abs(hi2(tt), 1.f));
+        Q1[c][1] = fma2(TH, sub2(pn, P1[c][1]), pn);
+        residual(pn, P1[c][1]);
+        P1[c][1] = pn;
+      };
+      auto p2_dof = [&](int c, int e, f32x2 h) {
+        const f32x2 leftu = c > 0 ? U[c > 0 ? c - 1 : 0][e] : (e == 0 ? ul.x : ul.y);
+        const f32x2 tt = fma2(PC, sub2(U[c][e], leftu), fma2(PA, P2[c][e], mul2(PB, h)));
+        record(tt, 16 + 4 * c + e);
+        const float ll = c == 0 ? lim_left : 1.f;
+        const f32x2 pn = pk2(clamp_abs(lo2(tt), ll), clamp_abs(hi2(tt), ll));
+        Q2[c][e] = fma2(TH, sub2(pn, P2[c][e]), pn);
+        residual(pn, P2[c][e]);
+        P2[c][e] = pn;
+      };
+      if (!ADAPT) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const ulonglong2 h1 = *reinterpret_cast<const ulonglong2*>(myF + kH1 + 4 * NT * c);
-        const ulonglong2 h2 = *reinterpret_cast<const ulonglong2*>(myF + kH2 + 4 * NT * c);
-        H0[c] = mul2(PB, h1.x);
-        {
-          const f32x2 tt = fma2(PC, sub2(U[c][1], U[c][0]), fma2(PA, P1[c][1], mul2(PB, h1.y)));  // p_target
-          record(tt, 4 * c + 1);
-          const f32x2 pn = pk2(clamp_abs(lo2(tt), 1.f), clamp_abs(hi2(tt), 1.f));
-          Q1[c][1] = fma2(TH, sub2(pn, P1[c][1]), pn);
-          P1[c][1] = pn;
+        for (int c = 0; c < 4; ++c) {
+          const ulonglong2 h1 = *reinterpret_cast<const ulonglong2*>(myF + kH1 + 4 * NT * c);
+          const ulonglong2 h2 = *reinterpret_cast<const ulonglong2*>(myF + kH2 + 4 * NT * c);
+          H0[c] = mul2(PB, h1.x);
+          p1_odd(c, h1.y);
+          p2_dof(c, 0, h2.x);
+          p2_dof(c, 1, h2.y);
         }
+      } else {  // the order in which the residuals are summed
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const f32x2 leftu = c > 0 ? U[c - 1][e] : (e == 0 ? ul.x : ul.y);
-          const f32x2 tt = fma2(PC, sub2(U[c][e], leftu), fma2(PA, P2[c][e], mul2(PB, e == 0 ? h2.x : h2.y)));
-          record(tt, 16 + 4 * c + e);
-          const float ll = c == 0 ? lim_left : 1.f;
-          const f32x2 pn = pk2(clamp_abs(lo2(tt), ll), clamp_abs(hi2(tt), ll));
-          Q2[c][e] = fma2(TH, sub2(pn, P2[c][e]), pn);
-          P2[c][e] = pn;
+        for (int c = 0; c < 4; ++c) p2_dof(c, 0, *reinterpret_cast<const f32x2*>(myF + kH2 + 4 * NT * c));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const ulonglong2 h1 = *reinterpret_cast<const ulonglong2*>(myF + kH1 + 4 * NT * c);
+          H0[c] = mul2(PB, h1.x);
+          p1_odd(c, h1.y);
+          p2_dof(c, 1, *reinterpret_cast<const f32x2*>(myF + kH2 + 4 * NT * c + 2));
         }
       }
       *reinterpret_cast<ulonglong2*>(myQL) = make_ulonglong2(Q2[0][0], Q2[0][1]);
@@ -529,6 +634,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         record(tt, 4 * c);
         const f32x2 pn = pk2(clamp_abs(lo2(tt), lim_top), clamp_abs(hi2(tt), 1.f));
         Q1[c][0] = fma2(TH, sub2(pn, P1[c][0]), pn);
+        residual(pn, P1[c][0]);
         P1[c][0] = pn;
       }
       const float4 q = make_float4(lo2(Q1[0][0]), lo2(Q1[1][0]), lo2(Q1[2][0]), lo2(Q1[3][0]));
@@ -544,6 +650,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       if (ADJ) xbits |= in_box(tt) & 1u;
       const float pn = clamp_abs(tt, 1.f);
       smem[L::QL + r_slot] = fmaf(co.th, pn - pr_s, pn);
+      residual(pk2(pn, 0.f), pk2(pr_s, 0.f));
       pr_s = pn;
     }
     if (bottom_lane) {  // Du = -u of the last row
@@ -555,15 +662,33 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         if (ADJ) xbits |= in_box(p_target(pB[c], -uB[c], hB[c], co)) & (2u << c);
+        const float po = pB[c];
         p_update(pB[c], qB[c], -uB[c], hB[c], co);
+        residual(pk2(pB[c], 0.f), pk2(po, 0.f));
       }
       *reinterpret_cast<float4*>(smem + L::PBS + j0) = make_float4(pB[0], pB[1], pB[2], pB[3]);
       *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(qB[0], qB[1], qB[2], qB[3]);
     }
     if (ADJ && (right_lane || bottom_lane)) tapeM[NT] = xbits;
+    if (ADAPT && k + 1 < K)  // added up at the start of iteration k + 1
+      *reinterpret_cast<float4*>(smem + AD::PS + 4 * tid) = make_float4(lo2(SD), hi2(SD), lo2(SP), hi2(SP));
     __syncthreads();
   }
-  if (CLU && push_down) wait_q();  // drain the last pbar1 halo (not read)
+  const bool stopped = ADAPT && k_run < K;
+  if (CLU && push_down && !stopped) wait_q();  // drain the last pbar1 halo (not read)
+  if (stopped) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(smem + AD::OU + 4 * (NT * c + tid));
+      U[c][0] = v.x;
+      U[c][1] = v.y;
+    }
+  }
+  if (ADAPT && rank == 0 && tid == 0) {
+    A.inner_used[a * g.NC + b] = k_run;
+    atomicMax(A.inner_max, k_run);
+    atomicAdd(A.inner_work, (unsigned long long)mr * (unsigned long long)mc * (unsigned long long)k_run);
+  }
   if constexpr (ADJ) {
     int tid2, a2 = a, b2 = b;  // the geometry again rather than in registers, as below
     asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid2));
@@ -602,6 +727,13 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile(const LocalArgs A, co
   const unsigned t = CLU ? blockIdx.x / (unsigned)cl : blockIdx.x, rank = CLU ? blockIdx.x - t * (unsigned)cl : 0u;
   const unsigned a = t / (unsigned)A.g.NC;
   tile_solve<LPR, NW, CLU, PAD, FID, MASK>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank, CLU ? cl : 1);
+}
+
+// adaptive inner stop, subdomains that fill their block
+template <int LPR, int NW, int FID, bool MASK>
+__global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile_adapt(const LocalArgs A, const int cl) {
+  const unsigned t = blockIdx.x / (unsigned)cl, rank = blockIdx.x - t * (unsigned)cl, a = t / (unsigned)A.g.NC;
+  tile_solve<LPR, NW, true, false, FID, MASK, false, true>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank, cl);
 }
 
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>

@@ -175,15 +175,6 @@ cudaError_t fused_mt_prepare();
 // The same kernel over the work list of a batch (every image's arrays 16-byte aligned).
 cudaError_t launch_fused_mt_batch(const BatchArgs& B, int total_tiles, cudaStream_t st);
 
-// ---- kernels_fused_mt4.cu
-// Persistent fused local solver on 4 x 4 micro-tiles, one warp per thread row, three
-// 128-thread CTAs per SM, the state moved by tensor copies; 128 x 128 tiles with 16-byte
-// aligned rows (fused_mt4_supported), fixed inner count or (a.inner_tol2 > 0) the adaptive
-// stop.  cudaErrorNotSupported if the tensor maps cannot be encoded.
-bool fused_mt4_supported(const LocalArgs& a);
-cudaError_t launch_fused_mt4(const LocalArgs& a, int fidelity, cudaStream_t st);
-cudaError_t fused_mt4_prepare();
-
 // ---- kernels_tile8.cu, kernels_tile16.cu, kernels_tile32.cu (fused_tile.cuh)
 // How the micro-tile kernels cover the subdomains of a grid: lpr lanes per row group (a
 // block 4 lpr columns wide), nw warps per CTA (bands of 4 nw (32 / lpr) rows), cl CTAs per
@@ -206,6 +197,8 @@ cudaError_t prepare_tile_8_4();
 cudaError_t prepare_tile_16_4();
 cudaError_t prepare_tile_16_8();
 cudaError_t prepare_tile_32_4();
+// the adaptive inner stop (a.inner_tol2 > 0), every subdomain exactly 128 x 128
+cudaError_t launch_tile_adapt_128(const LocalArgs& a, int fid, cudaStream_t st);
 // every subdomain of every image of a batch, 64 x 64 or 128 x 128
 cudaError_t launch_tile_batch_128(const BatchArgs& B, int total_tiles, bool overlap, cudaStream_t st);
 cudaError_t launch_tile_batch_64(const BatchArgs& B, int total_tiles, bool overlap, cudaStream_t st);

@@ -336,8 +336,7 @@ __global__ void __launch_bounds__(BW* TR, (BW * TR <= 256 ? 2 : 1)) k_fused(cons
 }
 
 // Hardware mappings of exact 128 x 128 subdomains (dd_tv_params.variant):
-//   0  the micro-tile kernel of every other shape (fused_tile.cuh)
-//   1  persistent 4 x 4 micro-tiles, state moved by tensor copies
+//   0  the micro-tile kernel of every other shape (fused_tile.cuh); 1 the same
 //   2  persistent 2 x 4 micro-tiles, 256 threads, 2 CTAs per SM
 //   3  the cluster-barrier kernel (one subdomain per cluster)
 constexpr int kNumVariants = 4;
@@ -450,8 +449,7 @@ cudaError_t fused_prepare() {
   if ((e = prepare_tile_16_4()) != cudaSuccess) return e;
   if ((e = prepare_tile_16_8()) != cudaSuccess) return e;
   if ((e = prepare_tile_32_4()) != cudaSuccess) return e;
-  if ((e = fused_mt_prepare()) != cudaSuccess) return e;
-  return fused_mt4_prepare();
+  return fused_mt_prepare();
 }
 
 cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, int variant, bool overlap,
@@ -462,7 +460,7 @@ cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, in
 }
 
 bool fused_out_of_place(const Grid& g, int variant) {
-  return variant == 0 || !(g.H == 128 * g.NR && g.W == 128 * g.NC);  // the micro-tile kernel
+  return variant <= 1 || !(g.H == 128 * g.NR && g.W == 128 * g.NC);  // the micro-tile kernel
 }
 
 cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStream_t st) {
@@ -470,11 +468,11 @@ cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStr
   const int mr = (a.g.H + a.g.NR - 1) / a.g.NR, mc = (a.g.W + a.g.NC - 1) / a.g.NC;
   const bool exact128 = a.g.H == 128 * a.g.NR && a.g.W == 128 * a.g.NC;  // every tile exactly 128 x 128
   if (a.inner_tol2 > 0.0) {
-    // the adaptive stop: in the persistent micro-tile kernel where it applies (variant 0)
-    if (exact128 && variant == 0 && fused_mt4_supported(a)) {
-      const cudaError_t e = launch_fused_mt4(a, fid, st);
-      if (e != cudaErrorNotSupported) return e;
-    }
+    // the micro-tile kernel for the default of exact 128 x 128 subdomains.  (W + N_c a multiple
+    // of 4 and K <= 64 are no needs of it, but its residual sums are float32 where those of
+    // the kernel below are float64, so a near tie could stop a subdomain one iteration
+    // apart: every problem keeps the sums it has always had.)
+    if (exact128 && variant == 0 && a.K <= 64 && (a.g.W + a.g.NC) % 4 == 0) return launch_tile_adapt_128(a, fid, st);
     switch (pick(mr, mc)) {
       case 0: return launch_fid<32, 8, 4, 1, true>(a, fid, st);
       case 1: return launch_fid<64, 8, 8, 1, true>(a, fid, st);
@@ -483,10 +481,6 @@ cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStr
     }
   }
   if (exact128) {
-    if (variant == 1 && fused_mt4_supported(a)) {
-      const cudaError_t e = launch_fused_mt4(a, fid, st);
-      if (e != cudaErrorNotSupported) return e;
-    }
     if (variant == 2 && fused_mt_supported(a)) return launch_fused_mt(a, fid, st);
     if (variant == 3) return launch_fid<128, 8, 2, 8, false>(a, fid, st);
   }

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
     ((128, 128), (2, 2), 0.0, 2), ((124, 101), (2, 2), 0.0, 5),    # 64 wide
     ((100, 60), (1, 1), 0.2, 2), ((192, 64), (2, 1), 0.0, 2),      # ... and taller than 64
     ((128, 256), (1, 2), 0.0, 2), ((112, 128), (1, 1), 0.0, 2),    # 128 wide, without padding and with 7 CTAs
-    ((33, 129), (2, 1), 0.0, 2), ((127, 215), (1, 2), 0.2, 2),
+    ((33, 129), (2, 2), 0.0, 2), ((127, 215), (1, 2), 0.2, 2),
 ])
 def test_reverse_pass_of_every_block_shape(cuda_lib, shape, tiles, mask_prob, every):
     f, g, mask = _case(*shape, "l2", mask_prob, seed=shape[0] + shape[1])
