@@ -278,14 +278,14 @@ int dd_tv_batch_create(dd_tv_batch** out, const dd_tv_batch_image* images, int n
       (e = cudaMalloc((void**)&b->d_tile_base, sizeof(int) * n)) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->d_elem_base, sizeof(int) * (n + 1))) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->d_sigma, sizeof(float) * n)) != cudaSuccess ||
-      (e = cudaMalloc((void**)&b->d_err, sizeof(int))) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->partials, sizeof(double) * reduce_partials_count())) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->counter, sizeof(unsigned int))) != cudaSuccess ||
-      (e = cudaMalloc((void**)&b->red_out, 2 * sizeof(double))) != cudaSuccess) {
+      (e = cudaMalloc((void**)&b->red_out, 3 * sizeof(double))) != cudaSuccess) {
     bfail(nullptr, DD_TV_ENOMEM, "batch descriptors: %s", cudaGetErrorString(e));
     dd_tv_batch_destroy(b);
     return DD_TV_ENOMEM;
   }
+  b->d_err = reinterpret_cast<int*>(b->red_out + 2);  // read back with the results, in one copy
   for (int i = 0; i < n; ++i) b->host_args[i].err = b->d_err;
   if ((e = cudaMemcpy(b->d_args, b->host_args.data(), sizeof(LocalArgs) * n, cudaMemcpyHostToDevice)) ||
       (e = cudaMemcpy(b->d_strips, b->host_strips.data(), sizeof(Strips) * 2 * n, cudaMemcpyHostToDevice)) ||
@@ -317,7 +317,7 @@ int dd_tv_batch_destroy(dd_tv_batch* b) {
   if (!b) return DD_TV_OK;
   drop_batch_graphs(b);
   void* bufs[] = {b->arena, b->d_args, b->d_strips, b->d_fid, b->d_tile_img, b->d_tile_base, b->d_elem_base,
-                  b->d_sigma, b->d_err, b->partials, b->counter, b->red_out};
+                  b->d_sigma, b->partials, b->counter, b->red_out};
   for (void* q : bufs)
     if (q) cudaFree(q);
   if (b->own) cudaStreamDestroy(b->own);
@@ -376,13 +376,15 @@ int dd_tv_batch_energy(dd_tv_batch* b, int i, double* J_out) {
   const LocalArgs& A = b->host_args[i];
   BCK(launch_energy(A.g, b->fid[i], (float)b->img[i].alpha, A.c1, A.c2, A.u, A.f, nullptr, nullptr, nullptr,
                     b->partials, b->counter, b->red_out, b->stream));
-  double o[2];
-  BCK(cudaMemcpyAsync(o, b->red_out, sizeof(o), cudaMemcpyDeviceToHost, b->stream));
+  struct {
+    double value[2];
+    int err, pad;
+  } o;
+  BCK(cudaMemcpyAsync(&o, b->red_out, sizeof(o), cudaMemcpyDeviceToHost, b->stream));
   BCK(cudaStreamSynchronize(b->stream));
-  int flag = 0;
-  BCK(cudaMemcpy(&flag, b->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  const int flag = o.err;
   if (flag) return bfail(b, DD_TV_ETIMEOUT, "a device-side wait ran out (results are invalid)");
-  *J_out = o[0];
+  *J_out = o.value[0];
   return DD_TV_OK;
 }
 

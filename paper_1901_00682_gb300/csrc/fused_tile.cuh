@@ -78,6 +78,19 @@ struct TileLayout {
   static_assert(kRightThread + BAND <= NT, "a thread per right-side dof");
 };
 
+// Shared memory with an inpainting domain D, behind the layout above: a word per pixel, thread
+// order.  f is taken as 0 on D, where the prox is the identity; then L1, ubar - P(ubar - f),
+// is it with the difference times 0, and L2, ua ubar + ub f, with ua replaced by 1: the
+// words are the factor 0 or 1, or the mask that keeps ua.
+constexpr bool use_mask_words(bool clu, bool mask, bool adj, bool adapt) { return clu && mask && !adj && !adapt; }
+
+template <int LPR, int NW>
+struct MaskTileLayout {
+  using L = TileLayout<LPR, NW>;
+  static constexpr int DM = (L::MB + 4 + 3) & ~3;
+  static constexpr size_t BYTES = sizeof(float) * (DM + 16 * L::NT);
+};
+
 // Shared memory of the adaptive inner stop, behind the layout above.
 template <int LPR, int NW>
 struct AdaptTileLayout {
@@ -229,6 +242,11 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   using AD = AdaptTileLayout<LPR, NW>;
   const uint32_t mbR = smem_addr(smem + AD::MBR);
   static_assert(!ADAPT || (CLU && !PAD && !ADJ && NW > 2), "the adaptive stop: clusters of full blocks");
+  // D as words in shared memory in clusters (4096 x 4096 in 128 x 128, L1: 246 -> 239 us), as bits
+  // where other arrays need the room and in single CTAs (1024 x 768 in 64 x 64: 20.4 us, with
+  // words 22.2: registers)
+  constexpr bool kWords = use_mask_words(CLU, MASK, ADJ, ADAPT), kBits = MASK && !kWords;
+  constexpr int kDM = MaskTileLayout<LPR, NW>::DM - L::F;
 
   const Grid g = A.g;
   const int r0 = PAD ? part_start(a, g.H, g.NR) : a * CL * BAND, mr = PAD ? part_start(a + 1, g.H, g.NR) - r0 : CL * BAND;
@@ -366,7 +384,9 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         if (c == 0 && left) h2[r][c] = phat_t(p2[r][c], ll[r], tau);
         if (PAD && rgt && cpad == c) h2[r][c] = phat_s(p2[r][c], lr[r], tau);
         if (FID == FID_SEG) fv[r][c] = (fv[r][c] - A.c1) * (fv[r][c] - A.c1) - (fv[r][c] - A.c2) * (fv[r][c] - A.c2);
-        if (MASK && ((mb[r] >> (8 * c)) & 0xffu)) in_d |= 1u << (4 * c + r);
+        const bool d = MASK && ((mb[r] >> (8 * c)) & 0xffu);
+        if (kBits && d) in_d |= 1u << (4 * c + r);
+        if (kWords && d) fv[r][c] = 0.f;
       }
     }
 #pragma unroll
@@ -378,6 +398,15 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         Q2[c][e] = P2[c][e] = pk2(p2[e][c], p2[e + 2][c]);
       }
       *reinterpret_cast<float4*>(myF + 4 * NT * c) = make_float4(fv[0][c], fv[2][c], fv[1][c], fv[3][c]);
+      if (kWords) {
+        float m[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const bool d = (mb[r] >> (8 * c)) & 0xffu;
+          m[r] = FID == FID_L1 ? (d ? 0.f : 1.f) : __uint_as_float(d ? 0u : ~0u);
+        }
+        *reinterpret_cast<float4*>(myF + kDM + 4 * NT * c) = make_float4(m[0], m[2], m[1], m[3]);
+      }
       *reinterpret_cast<float4*>(myF + kH1 + 4 * NT * c) = make_float4(h1[0][c], h1[2][c], h1[1][c], h1[3][c]);
       *reinterpret_cast<float4*>(myF + kH2 + 4 * NT * c) = make_float4(h2[0][c], h2[2][c], h2[1][c], h2[3][c]);
     }
@@ -485,6 +514,8 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const ulonglong2 fc = *reinterpret_cast<const ulonglong2*>(myF + 4 * NT * c);
+        ulonglong2 dm = make_ulonglong2(0ull, 0ull);
+        if (kWords) dm = *reinterpret_cast<const ulonglong2*>(myF + kDM + 4 * NT * c);
         f32x2 ubar[2];
 #pragma unroll
         for (int ee = 0; ee < 2; ++ee) {
@@ -497,15 +528,19 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
           const f32x2 d = sub2(add2(bt, right), Q2[c][e]);  // div_px
           const f32x2 ub = fma2(SIG, d, U[c][e]);
           ubar[e] = ub;
-          const bool dl = MASK && ((in_d >> (4 * c + e)) & 1u), dh = MASK && ((in_d >> (4 * c + e + 2)) & 1u);
+          const bool dl = kBits && ((in_d >> (4 * c + e)) & 1u), dh = kBits && ((in_d >> (4 * c + e + 2)) & 1u);
+          const f32x2 de = e == 0 ? dm.x : dm.y;
           f32x2 un;
           if (FID == FID_L2) {
-            un = fma2(UBc, fg, mul2(UA, ub));
-            if (MASK) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
+            f32x2 ua = UA;
+            if (kWords) ua = (UA & de) | (0x3f8000003f800000ull & ~de);
+            un = fma2(UBc, fg, mul2(ua, ub));
+            if (kBits) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
           } else if (FID == FID_L1) {  // ubar - P_[-s,s](ubar - f)
-            const f32x2 v = sub2(ub, fg);
+            f32x2 v = sub2(ub, fg);
+            if (kWords) v = mul2(v, de);
             un = sub2(ub, pk2(clamp_abs(lo2(v), cu.s), clamp_abs(hi2(v), cu.s)));
-            if (MASK) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
+            if (kBits) un = pk2(dl ? lo2(ub) : lo2(un), dh ? hi2(ub) : hi2(un));
           } else {
             un = pk2(prox_ubar<FID>(lo2(ub), lo2(fg), dl, cu), prox_ubar<FID>(hi2(ub), hi2(fg), dh, cu));
           }
@@ -739,7 +774,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile_adapt(const LocalArgs
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
 cudaError_t prepare_tile_one() {
   return cudaFuncSetAttribute(k_tile<LPR, NW, CLU, PAD, FID, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)TileLayout<LPR, NW>::BYTES);
+                              (int)(use_mask_words(CLU, MASK, false, false) ? MaskTileLayout<LPR, NW>::BYTES : TileLayout<LPR, NW>::BYTES));
 }
 
 template <int LPR, int NW, bool CLU, bool PAD>
@@ -763,7 +798,7 @@ cudaError_t launch_tile_one(const LocalArgs& a, int cl, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(CLU ? cl : 1) * a.g.NC * a.g.NR, 1, 1);
   cfg.blockDim = dim3(32 * NW, 1, 1);
-  cfg.dynamicSmemBytes = TileLayout<LPR, NW>::BYTES;
+  cfg.dynamicSmemBytes = use_mask_words(CLU, MASK, false, false) ? MaskTileLayout<LPR, NW>::BYTES : TileLayout<LPR, NW>::BYTES;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   cfg.attrs = attr;

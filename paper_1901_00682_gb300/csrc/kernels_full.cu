@@ -13,10 +13,10 @@
 // another's results.
 //
 // What bounds it: as the local solve, latency and issue slots of the inner loop, times the
-// overlap (128 x 128 pixels computed for 108 x 104 stored at n = 10), and per launch 24 bytes
+// overlap (128 x 128 pixels computed for 108 x 108, or 104, stored at n = 10), and per launch 24 bytes
 // read and 20 written per pixel of a block.  n is at most 10: twice as many leave less than
 // half of a block to store.  Measured per 10 iterations, before (two launches per iteration)
-// and after: 1001 x 1503 218 -> 48 us.
+// and after: 1001 x 1503 218 -> 43 us, 4096 x 4096 about 2500 -> 306.
 #include "fused_tile.cuh"
 
 namespace ddtv {
@@ -27,27 +27,28 @@ using FL = TileLayout<32, 4>;
 constexpr int kBlockSide = FL::BW;
 
 // Blocks along an axis of len pixels: m of them, block q covering [start, start + 128) (or
-// the whole axis), storing [from, to).  Starts and bounds are multiples of 4 wherever they
-// can be, for 16-byte accesses.
+// the whole axis), storing [from, to).  Starts and bounds are multiples of `al` (4 for the
+// columns of an image whose rows are 16-byte aligned, else 1), but for the last start.
 struct Axis {
-  int len, m, halo4;
+  int len, m, halo, al;
   __host__ __device__ int start(int q) const {
-    const int T = (len - kBlockSide + 3) / 4;
-    const int s = m > 1 ? 4 * (int)((long long)q * T / (m - 1)) : 0;
+    const int T = (len - kBlockSide + al - 1) / al;
+    const int s = m > 1 ? al * (int)((long long)q * T / (m - 1)) : 0;
     return q > 0 && q == m - 1 ? len - kBlockSide : s;
   }
   __host__ __device__ int size() const { return len < kBlockSide ? len : kBlockSide; }
-  __host__ __device__ int from(int q) const { return q > 0 ? start(q) + halo4 : 0; }
-  __host__ __device__ int to(int q) const { return q + 1 < m ? start(q + 1) + halo4 : len; }
+  __host__ __device__ int from(int q) const { return q > 0 ? start(q) + halo : 0; }
+  __host__ __device__ int to(int q) const { return q + 1 < m ? start(q + 1) + halo : len; }
 };
 
 // n iterations: every interior bound at least n pixels inside both blocks it separates
-Axis axis_for(int len, int n) {
+Axis axis_for(int len, int n, int al) {
   Axis a;
   a.len = len;
-  a.halo4 = (n + 3) & ~3;
-  const int gap4 = (kBlockSide - a.halo4 - n) / 4;  // largest distance of two starts, in units of 4
-  a.m = len <= kBlockSide ? 1 : 1 + ((len - kBlockSide + 3) / 4 + gap4 - 1) / gap4;
+  a.al = al;
+  a.halo = (n + al - 1) / al * al;
+  const int gap = (kBlockSide - a.halo - n) / al;  // largest distance of two starts, in units of al
+  a.m = len <= kBlockSide ? 1 : 1 + ((len - kBlockSide + al - 1) / al + gap - 1) / gap;
   return a;
 }
 
@@ -107,24 +108,49 @@ __global__ void __launch_bounds__(FL::NT, 4) k_full(const FullArgs A, const Axis
   uint32_t in_d = 0;
   {
     const bool vec = (W & 3) == 0 && (c0 & 3) == 0;
-    float t[4][4];
-    auto rows = [&](const float* base, int ld, bool v, f32x2 (*X)[2]) {  // the lane's 4 x 4 pixels of an array
+    // the lane's 4 x 4 pixels of every array, all loads in flight before the first is used
+    float x[6][4][4];
+    const float* const base[6] = {A.f, A.in.u, A.in.P1, A.in.Pb1, A.in.P2, A.in.Pb2};
+    const size_t o1 = (size_t)(r0 + i0) * W + c0 + j0, o2 = (size_t)(r0 + i0) * W2 + c0 + j0;
+    if (vec && i0 + 3 < mr && j0 + 3 < mc) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-        load4(base + (size_t)(r0 + i0 + r) * ld + c0 + j0, i0 + r < mr ? mc - j0 : 0, v, t[r]);
+      for (int r = 0; r < 4; ++r) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        X[c][0] = pk2(t[0][c], t[2][c]);
-        X[c][1] = pk2(t[1][c], t[3][c]);
+        for (int q = 0; q < 4; ++q) load4(base[q] + o1 + (size_t)r * W, x[q][r]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          x[4][r][c] = base[4][o2 + (size_t)r * W2 + c];
+          x[5][r][c] = base[5][o2 + (size_t)r * W2 + c];
+        }
       }
-    };
+    } else {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int n = i0 + r < mr ? mc - j0 : 0;
+#pragma unroll
+        for (int q = 0; q < 6; ++q)
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            x[q][r][c] = c < n ? base[q][(q < 4 ? o1 + (size_t)r * W : o2 + (size_t)r * W2) + c] : 0.f;
+      }
+    }
+    float qb[4] = {0.f, 0.f, 0.f, 0.f};  // pbar1 of the row below the band (0 below the image)
+    if (w == NG - 1) load4(A.in.Pb1 + (size_t)(r0 + i0 + 4) * W + c0 + j0, r0 + i0 + 4 < A.H ? mc - j0 : 0, vec, qb);
+    float qr = 0.f;  // pbar2 right of the block (0 right of the image), in the pair order of the slots: rows 0, 2, 1, 3
+    const int ro = (l >> 1) + 2 * (l & 1);
+    if (l < 4 && mc == BW && c0 + BW < W && i0 + ro < mr) qr = A.in.Pb2[(size_t)(r0 + i0 + ro) * W2 + c0 + BW];
     f32x2 FV[4][2];
-    rows(A.f, W, vec, FV);
-    rows(A.in.u, W, vec, U);
-    rows(A.in.P1, W, vec, P1);
-    rows(A.in.Pb1, W, vec, Q1);
-    rows(A.in.P2, W2, false, P2);
-    rows(A.in.Pb2, W2, false, Q2);
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        FV[c][e] = pk2(x[0][e][c], x[0][e + 2][c]);
+        U[c][e] = pk2(x[1][e][c], x[1][e + 2][c]);
+        P1[c][e] = pk2(x[2][e][c], x[2][e + 2][c]);
+        Q1[c][e] = pk2(x[3][e][c], x[3][e + 2][c]);
+        P2[c][e] = pk2(x[4][e][c], x[4][e + 2][c]);
+        Q2[c][e] = pk2(x[5][e][c], x[5][e + 2][c]);
+      }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       if (FID == FID_SEG) {
@@ -146,19 +172,10 @@ __global__ void __launch_bounds__(FL::NT, 4) k_full(const FullArgs A, const Axis
     }
     *reinterpret_cast<float4*>(sQ1 + w * BW + j0) = make_float4(lo2(Q1[0][0]), lo2(Q1[1][0]), lo2(Q1[2][0]), lo2(Q1[3][0]));
     *reinterpret_cast<ulonglong2*>(myQL) = make_ulonglong2(Q2[0][0], Q2[0][1]);
-    if (w == NG - 1) {  // pbar1 of the row below the band (0 below the image)
-      float q[4];
-      const int gi = r0 + i0 + 4;
-      load4(A.in.Pb1 + (size_t)gi * W + c0 + j0, gi < A.H ? mc - j0 : 0, vec, q);
-      *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(q[0], q[1], q[2], q[3]);
-    }
+    if (w == NG - 1) *reinterpret_cast<float4*>(sQ1 + NG * BW + j0) = make_float4(qb[0], qb[1], qb[2], qb[3]);
     if (w == 0 && rank == 0) *reinterpret_cast<float4*>(sUB + j0) = make_float4(0.f, 0.f, 0.f, 0.f);
     if (l == 0) *reinterpret_cast<float4*>(smem + FL::UR + w * FL::SLOT) = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (l < 4) {  // pbar2 right of the block (0 right of the image), in the pair order of the slots: rows 0, 2, 1, 3
-      const int r = (l >> 1) + 2 * (l & 1);
-      smem[FL::QL + w * FL::SLOT + 4 * LPR + l] =
-          mc == BW && c0 + BW < W && i0 + r < mr ? A.in.Pb2[(size_t)(r0 + i0 + r) * W2 + c0 + BW] : 0.f;
-    }
+    if (l < 4) smem[FL::QL + w * FL::SLOT + 4 * LPR + l] = qr;
   }
   __syncthreads();
   bool timed_out = false;
@@ -292,7 +309,7 @@ __global__ void __launch_bounds__(FL::NT, 4) k_full(const FullArgs A, const Axis
 
 template <int FID, bool MASK>
 cudaError_t launch_full_one(const FullArgs& a, int n, cudaStream_t st) {
-  const Axis ar = axis_for(a.H, n), ac = axis_for(a.W, n);
+  const Axis ar = axis_for(a.H, n, 1), ac = axis_for(a.W, n, (a.W & 3) == 0 ? 4 : 1);
   const int cl = (ar.size() + FL::BAND - 1) / FL::BAND;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)cl * ac.m * ar.m, 1, 1);
