@@ -200,7 +200,8 @@ int dd_tv_current_energy(dd_tv* h, double* J_out);
  * dd_tv_set_profiling(h, 1): later dd_tv_iterate / energy calls launch their kernels
  * directly (no graph replay) and bracket every phase with CUDA events on the
  * handle's stream.  dd_tv_profile_read synchronises and writes, for each phase
- * (0 = interface multiplier update, 1 = local solves, 2 = energy reduction), the
+ * (0 = interface multiplier update where it is a launch of its own, 1 = local solves,
+ * which make the update themselves on the fused path's default, 2 = energy reduction), the
  * summed device time in milliseconds and the number of kernel launches since
  * profiling was switched on (arrays of 3; either pointer may be NULL); it then
  * resets the counters.  dd_tv_set_profiling(h, 0) returns to graph replay. */

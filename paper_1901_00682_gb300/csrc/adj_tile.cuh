@@ -537,7 +537,7 @@ template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
 __global__ void __launch_bounds__(32 * NW, NW <= 4 ? 12 / NW : 2) k_adj_tile(const LocalArgs A, const AdjArgs Z, const int cl) {
   const unsigned t = CLU ? blockIdx.x / (unsigned)cl : blockIdx.x, rank = CLU ? blockIdx.x - t * (unsigned)cl : 0u;
   const unsigned a = t / (unsigned)A.g.NC;
-  tile_solve<LPR, NW, CLU, PAD, FID, MASK, true>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank,
+  tile_solve<LPR, NW, CLU, PAD, FID, MASK, false, true>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank,
                                                  CLU ? cl : 1, &Z);
 }
 

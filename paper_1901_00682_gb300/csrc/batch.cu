@@ -190,7 +190,7 @@ int dd_tv_batch_create(dd_tv_batch** out, const dd_tv_batch_image* images, int n
   b->n = n;
   b->p = *p;
   b->img.assign(images, images + n);
-  cudaError_t e = fused_prepare();
+  cudaError_t e = fused_prepare_batch(p->tile, p->variant);
   if (e != cudaSuccess) {
     bfail(nullptr, DD_TV_ECUDA, "fused kernel set-up: %s", cudaGetErrorString(e));
     delete b;
@@ -237,6 +237,7 @@ int dd_tv_batch_create(dd_tv_batch** out, const dd_tv_batch_image* images, int n
     const double tau = m.tau > 0 ? m.tau : (m.fidelity == DD_TV_SEG ? 1.0 : 50.0);
     const double sigma = m.tau > 0 ? m.sigma : 0.5 / tau;
     LocalArgs& A = b->host_args[i];
+    A = LocalArgs{};
     A.g = Grid{m.height, m.width, NR, NC};
     A.K = p->inner_iters;
     A.tau = (float)tau;

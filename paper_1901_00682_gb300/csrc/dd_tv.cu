@@ -72,6 +72,12 @@ struct dd_tv {
   // line into the arrays above; for a whole image they equal lamh / strips.
   float* lamh_k = nullptr;
   Strips strips_k[2] = {};
+  // the local solves make the multiplier update (LocalArgs.chain): lamh, lamv are the copies of
+  // the upper / left sides, lam2 ([h | v]) those of the lower / right ones, x the extrapolated
+  // strips by parity
+  bool chain = false;
+  float *lam2 = nullptr, *x_mem = nullptr;
+  Strips x[2] = {};
   // row-block shard (dd_tv_create_shard): global tile rows [tile_row0, tile_row0 + g.NR)
   // of a problem with nr_global tile rows; its first pixel row is row0 of the image
   bool shard = false;
@@ -219,7 +225,7 @@ void build_schedule(const dd_tv_params& p, std::vector<Coef>& c) {
 }
 
 LocalArgs local_args(dd_tv* h, int write_set) {
-  LocalArgs a;
+  LocalArgs a{};
   a.g = h->g;
   a.K = h->p.inner_iters;
   a.tau = (float)h->p.tau;
@@ -282,6 +288,31 @@ void full_select(dd_tv* h) {
   h->Pb2 = s.Pb2;
 }
 
+// The chained local solve's arrays: iterate n of parity par in, n + 1 out.
+void chain_args(dd_tv* h, int par, LocalArgs* a) {
+  a->chain = 1;
+  a->sigma = (float)h->p.sigma;
+  a->lam_th = h->lamh;
+  a->lam_tv = h->lamv;
+  a->lam_sh = h->lam2;
+  a->lam_sv = h->lam2 ? h->lam2 + h->nh : nullptr;
+  a->x_in = h->x[par];
+  a->x_out = h->x[1 - par];
+}
+
+// After lamh, lamv and both strip sets of iterate h->n were set: the arrays that follow from them.
+cudaError_t chain_rebuild(dd_tv* h) {
+  if (!h->chain) return cudaSuccess;
+  const auto D2D = cudaMemcpyDeviceToDevice;
+  const int par = h->n & 1;
+  cudaError_t e;
+  if (h->nh && (e = cudaMemcpyAsync(h->lam2, h->lamh, h->nh * sizeof(float), D2D, h->stream)) != cudaSuccess) return e;
+  if (h->nv && (e = cudaMemcpyAsync(h->lam2 + h->nh, h->lamv, h->nv * sizeof(float), D2D, h->stream)) != cudaSuccess)
+    return e;
+  return launch_extrapolate(2 * (long long)(h->nh + h->nv), h->strips[par].SB, h->strips[1 - par].SB, h->x[par].SB,
+                            h->stream);
+}
+
 // One outer iteration starting from parity `par` (= n mod 2): the strips of p~^n are
 // in set par, those of p~^{n-1} in set 1 - par, and p~^{n+1}'s go to set 1 - par.
 cudaError_t outer_once(dd_tv* h, int par) {
@@ -308,6 +339,12 @@ cudaError_t outer_once(dd_tv* h, int par) {
         return e;
     }
     return cudaSuccess;
+  }
+  if (h->chain) {  // one launch: the local solves update the multipliers as they load
+    PhaseMark m(h, 1, 1);
+    LocalArgs a = local_args(h, 1 - par);
+    chain_args(h, par, &a);
+    return launch_fused_local(a, h->fid, h->p.variant, st);
   }
   {
     PhaseMark m(h, 0, (h->nh + h->nv) ? 1 : 0);
@@ -394,6 +431,7 @@ int reset_state(dd_tv* h) {
   if (h->nh) CK(cudaMemsetAsync(h->lamh, 0, h->nh * sizeof(float), st));
   if (h->nv) CK(cudaMemsetAsync(h->lamv, 0, h->nv * sizeof(float), st));
   if (h->strip_mem) CK(cudaMemsetAsync(h->strip_mem, 0, 4 * (h->nh + h->nv) * sizeof(float), st));
+  if (h->x_mem) CK(cudaMemsetAsync(h->x_mem, 0, 5 * (h->nh + h->nv) * sizeof(float), st));  // x and lam2
   if (h->Pb1) {
     CK(cudaMemsetAsync(h->Pb1, 0, h->n1 * sizeof(float), st));
     CK(cudaMemsetAsync(h->Pb2, 0, h->n2 * sizeof(float), st));
@@ -548,7 +586,7 @@ int adj_reserve(dd_tv* h, int nck, int m) {
     w->fused = tape_f > 0 && tape_f * sizeof(float) <= (4ull << 30);
     w->direct = w->fused && h->p.path == DD_TV_PATH_FUSED && fused_out_of_place(h->g, h->p.variant);
     w->nal = (int)std::max(adj_alpha_slots(h->g), adj_alpha_slots_fused(h->g));
-    if (w->fused) CK(adj_fused_prepare());
+    if (w->fused) CK(adj_fused_prepare(h->g));
     int rc;
     if ((rc = dalloc(h, &w->Au, h->npx)) || (rc = dalloc(h, &w->Ad, h->npx)) || (rc = dalloc(h, &w->Af, h->npx)) ||
         (rc = dalloc(h, &w->Aal, (size_t)w->nal)) || (rc = dalloc(h, &w->AP, nP)) || (rc = dalloc(h, &w->AQ, nP)) ||
@@ -644,6 +682,7 @@ int state_restore(dd_tv* h, const float* src, int n) {
     CK(cudaMemcpyAsync(h->strip_mem, src + ne, 4 * ne * sizeof(float), D2D, st));
   }
   h->n = n;
+  CK(chain_rebuild(h));
   return DD_TV_OK;
 }
 
@@ -925,7 +964,7 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
   }
   cudaGetDevice(&h->device);
   if (p->path == DD_TV_PATH_FUSED) {
-    cudaError_t e = fused_prepare();
+    cudaError_t e = fused_prepare(h->g, p->variant, p->inner_tol > 0.0);
     if (e != cudaSuccess) {
       std::snprintf(g_create_err, sizeof(g_create_err), "fused kernel set-up: %s", cudaGetErrorString(e));
       delete h;
@@ -999,6 +1038,20 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
       h->strips_k[s].ST += skip;
     }
   }
+  h->chain = p->path == DD_TV_PATH_FUSED && !h->shard && fused_chains(g, p->variant, p->inner_iters, p->inner_tol > 0.0);
+  if (h->chain && h->nh + h->nv) {
+    const size_t ne = h->nh + h->nv;
+    if ((rc = dalloc(h, &h->x_mem, 5 * ne))) {
+      std::snprintf(g_create_err, sizeof(g_create_err), "%s", h->err);
+      dd_tv_destroy(h);
+      return rc;
+    }
+    for (int s = 0; s < 2; ++s) {
+      float* base = h->x_mem + (size_t)s * 2 * ne;
+      h->x[s] = Strips{base, base + h->nh, base + 2 * h->nh, base + 2 * h->nh + h->nv};
+    }
+    h->lam2 = h->x_mem + 4 * ne;
+  }
   h->lamh_k = h->lamh ? h->lamh + (size_t)g.cut_top * g.W : nullptr;
   cudaError_t e;
   if ((e = cudaMemcpy(h->coef, sched.data(), sched.size() * sizeof(Coef), cudaMemcpyHostToDevice)) != cudaSuccess ||
@@ -1043,7 +1096,7 @@ int dd_tv_destroy(dd_tv* h) {
     cudaEventDestroy(m.a);
     cudaEventDestroy(m.b);
   }
-  void* bufs[] = {h->f, h->u, h->P1, h->P2, h->lamh, h->lamv, h->mask, h->strip_mem, h->coef, h->Ph1, h->Ph2,
+  void* bufs[] = {h->f, h->u, h->P1, h->P2, h->lamh, h->lamv, h->mask, h->strip_mem, h->x_mem, h->coef, h->Ph1, h->Ph2,
                   h->Pb1, h->Pb2, h->partials, h->counter, h->red_out, h->flag, h->inner_used, h->inner_max,
                   h->inner_work};
   for (void* b : bufs)
@@ -1178,6 +1231,7 @@ int dd_tv_set_state(dd_tv* h, const float* u, const float* P1, const float* P2, 
   } else {
     CK(launch_extract_strips(h->g, P1, P2, h->strips[h->n & 1], st));
     CK(launch_extract_strips(h->g, P1prev, P2prev, h->strips[1 - (h->n & 1)], st));
+    CK(chain_rebuild(h));
   }
   h->loaded = true;
   return DD_TV_OK;

@@ -107,6 +107,28 @@ struct AdaptTileLayout {
   static_assert(RED % 2 == 0 && MBR % 2 == 0, "8-byte alignment of the pairs and mbarriers");
 };
 
+// Shared memory of the multiplier update (CHAIN), behind whichever of the above the instance
+// has.  (What an instance does not need it does not ask for: four CTAs past 164 KB or 196 KB
+// leave the L1 cache less, 4096 x 4096 with a mask 240 -> 265 us.)
+template <int LPR, int NW, bool WORDS, bool ADAPT>
+struct ChainTileLayout {
+  using L = TileLayout<LPR, NW>;
+  static constexpr size_t kBefore = ADAPT   ? AdaptTileLayout<LPR, NW>::BYTES
+                                    : WORDS ? MaskTileLayout<LPR, NW>::BYTES
+                                            : L::BYTES;
+  static constexpr int OT = (int)((kBefore / sizeof(float) + 3) & ~(size_t)3);  // p~^n on the upper and lower side (BW each),
+  static constexpr int OL = OT + 2 * L::BW;    // ... on the left and right side, of the band's rows (BAND each)
+  static constexpr int LT = OL + 2 * L::BAND;  // the new multipliers of the upper and lower side (BW each)
+  static constexpr int LL = LT + 2 * L::BW;    // ... of the left and right side (BAND each)
+  static constexpr size_t BYTES = sizeof(float) * (LL + 2 * L::BAND);
+};
+
+// shared memory of an instance of the forward kernel
+template <int LPR, int NW, bool WORDS, bool ADAPT, bool CHAIN>
+constexpr size_t tile_bytes() {
+  return CHAIN ? ChainTileLayout<LPR, NW, WORDS, ADAPT>::BYTES : ChainTileLayout<LPR, NW, WORDS, ADAPT>::kBefore;
+}
+
 // four consecutive floats (16-byte aligned)
 __device__ __forceinline__ void load4(const float* p, float* v) {
   const float4 x = *reinterpret_cast<const float4*>(p);
@@ -144,7 +166,7 @@ __device__ __forceinline__ void store4(float* p, int n, bool vec, float a, float
 __device__ __forceinline__ float half_of(f32x2 v, int h) { return h ? hi2(v) : lo2(v); }
 
 // Stores the subdomain's u, p1, p2 and sides.
-template <int LPR, int NW, bool PAD>
+template <int LPR, int NW, bool PAD, bool CHAIN, class CH>
 __device__ __forceinline__ void tile_store(const LocalArgs& A, const Strips& out, int a, int b, int tid, int CL, int rank,
                                            const f32x2 (&U)[4][2], const f32x2 (&P1)[4][2], const f32x2 (&P2)[4][2],
                                            float pr_s) {
@@ -165,6 +187,60 @@ __device__ __forceinline__ void tile_store(const LocalArgs& A, const Strips& out
   // the strips of a set start at multiples of the interface edges, not of 4 floats
   const bool vec_t = vec && (reinterpret_cast<uintptr_t>(out.ST) & 15) == 0;
   const bool vec_b = vec && (reinterpret_cast<uintptr_t>(out.SB) & 15) == 0;
+  if (CHAIN) {  // 2 p~^{n+1} - p~^n of the sides and their multipliers
+    const Strips& x = A.x_out;
+    const float *oldt = smem + CH::OT + j0, *oldl = smem + CH::OL + 4 * G;
+    const float *lamt = smem + CH::LT + j0, *laml = smem + CH::LL + 4 * G;
+    if (i0 == 0 && s_top) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c < mc - j0) {
+          const ptrdiff_t e = (ptrdiff_t)(a - 1) * g.W + c0 + j0 + c;
+          x.ST[e] = fmaf(2.0f, lo2(P1[c][0]), -oldt[c]);
+          A.lam_th[e] = lamt[c];
+        }
+    }
+    const bool pad_bot = PAD && s_bot && !fill_r && mr >= i0 && mr < i0 + 4;
+    if (pad_bot || bottom_lane) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int r = mr - i0;
+        const f32x2 v = r & 1 ? P1[c][1] : P1[c][0];
+        const float pn = pad_bot ? (r >> 1 ? hi2(v) : lo2(v)) : smem[L::PBS + j0 + c];
+        const ptrdiff_t e = (ptrdiff_t)a * g.W + c0 + j0 + c;
+        if (c < mc - j0) {
+          x.SB[e] = fmaf(2.0f, pn, -oldt[BW + c]);
+          A.lam_sh[e] = lamt[BW + c];
+        }
+      }
+    }
+    if (j0 == 0 && s_lft) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (i0 + r < mr) {
+          const ptrdiff_t e = (ptrdiff_t)(b - 1) * g.H + r0 + i0 + r;
+          x.SL[e] = fmaf(2.0f, half_of(P2[0][r & 1], r >> 1), -oldl[r]);
+          A.lam_tv[e] = laml[r];
+        }
+    }
+    if (PAD && s_rgt && !fill_c && mc >= j0 && mc < j0 + 4) {
+      const int q = mc - j0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const f32x2 v = q == 0 ? P2[0][r & 1] : (q == 1 ? P2[1][r & 1] : (q == 2 ? P2[2][r & 1] : P2[3][r & 1]));
+        const ptrdiff_t e = (ptrdiff_t)b * g.H + r0 + i0 + r;
+        if (i0 + r < mr) {
+          x.SR[e] = fmaf(2.0f, half_of(v, r >> 1), -oldl[BAND + r]);
+          A.lam_sv[e] = laml[BAND + r];
+        }
+      }
+    }
+    if (right_lane) {
+      const ptrdiff_t e = (ptrdiff_t)b * g.H + r0 + rank * BAND + rr;
+      x.SR[e] = fmaf(2.0f, pr_s, -smem[CH::OL + BAND + rr]);
+      A.lam_sv[e] = smem[CH::LL + BAND + rr];
+    }
+  }
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int e = r & 1, h = r >> 1, i = i0 + r, gi = r0 + i;
@@ -229,7 +305,10 @@ __device__ __forceinline__ void tile_reverse(const LocalArgs& A, const AdjArgs& 
 // barrier.  On "stop" the u-step of iteration k + 1 is undone (each iteration first copies u
 // to shared memory), its u halo is drained and the p-step is skipped: the solve keeps k + 1
 // inner iterations, as the rule prescribes.
-template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK, bool ADJ = false, bool ADAPT = false>
+//
+// CHAIN: the multiplier update is made here as the state is loaded (LocalArgs.chain).
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK, bool CHAIN = false, bool ADJ = false,
+          bool ADAPT = false>
 __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out, const int a, const int b,
                                            const int rank, const int CL, const AdjArgs* Z = nullptr) {
   using L = TileLayout<LPR, NW>;
@@ -247,6 +326,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   // words 22.2: registers)
   constexpr bool kWords = use_mask_words(CLU, MASK, ADJ, ADAPT), kBits = MASK && !kWords;
   constexpr int kDM = MaskTileLayout<LPR, NW>::DM - L::F;
+  using CH = ChainTileLayout<LPR, NW, kWords, ADAPT>;
 
   const Grid g = A.g;
   const int r0 = PAD ? part_start(a, g.H, g.NR) : a * CL * BAND, mr = PAD ? part_start(a + 1, g.H, g.NR) - r0 : CL * BAND;
@@ -324,31 +404,63 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     const float* g2 = A.P20 + (size_t)(r0 + i0) * W2 + c0 + b + j0;
     const uint8_t* gm = MASK ? A.mask + (size_t)(r0 + i0) * g.W + c0 + j0 : nullptr;
     uint32_t mb[4] = {0, 0, 0, 0};  // mask bytes of the lane's rows
-    if (vec && i0 + 3 < mr && j0 + 3 < mc) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        load4(gu + (size_t)r * g.W, u[r]);
+    const bool whole = vec && i0 + 3 < mr && j0 + 3 < mc;
+    auto data = [&](int r) {  // f and the mask of a row
+      if (whole) {
         load4(gf + (size_t)r * g.W, fv[r]);
-        load4(g1 + (size_t)r * g.W, p1[r]);
         if (MASK) mb[r] = *reinterpret_cast<const uint32_t*>(gm + (size_t)r * g.W);
+      } else {
+        const int n = i0 + r < mr ? mc - j0 : 0;  // pixels of this lane's row
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          fv[r][c] = c < n ? gf[(size_t)r * g.W + c] : 0.f;
+          if (MASK && c < n) mb[r] |= (uint32_t)gm[(size_t)r * g.W + c] << (8 * c);
+        }
+      }
+    };
+    auto state = [&](int r) {
+      if (whole) {
+        load4(gu + (size_t)r * g.W, u[r]);
+        load4(g1 + (size_t)r * g.W, p1[r]);
 #pragma unroll
         for (int c = 0; c < 4; ++c) p2[r][c] = g2[(size_t)r * W2 + c];
-      }
-    } else {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
+      } else {
         const int i = i0 + r;
-        const int n = i < mr ? mc - j0 : 0;                                // pixels of this lane's row
+        const int n = i < mr ? mc - j0 : 0;
         const int n1 = i < mr + (s_bot ? 1 : 0) ? mc - j0 : 0;             // p1 dofs (row mr: the bottom side)
         const int n2 = i < mr ? mc + (s_rgt ? 1 : 0) - j0 : 0;             // p2 dofs (column mc: the right side)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           u[r][c] = c < n ? gu[(size_t)r * g.W + c] : 0.f;
-          fv[r][c] = c < n ? gf[(size_t)r * g.W + c] : 0.f;
           p1[r][c] = c < n1 ? g1[(size_t)r * g.W + c] : 0.f;
           p2[r][c] = c < n2 ? g2[(size_t)r * W2 + c] : 0.f;
-          if (MASK && c < n) mb[r] |= (uint32_t)gm[(size_t)r * g.W + c] << (8 * c);
         }
+      }
+    };
+    if (CHAIN) {  // the data before the previous launch has ended, the state after
+      if (whole) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) data(r);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) data(r);
+      }
+      pdl_wait();
+      if (whole) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) state(r);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) state(r);
+      }
+    } else {
+      // (one branch around all rows, so that the loads of a row do not wait for another's)
+      if (whole) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) state(r), data(r);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) state(r), data(r);
       }
     }
     // pbar1 of the row below the band: the next CTA's first row (its halo of later
@@ -361,17 +473,52 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     for (int c = 0; c < 4; ++c) qb[c] = c < nb ? A.P10[(size_t)(r0 + ib + a) * g.W + c0 + j0 + c] : 0.f;
     if (right_lane) pr_s = A.P20[(size_t)(r0 + rank * BAND + rr) * W2 + c0 + BW + b];
 
-    pdl_wait();  // the multipliers, of the sides this lane holds
+    if (!CHAIN) pdl_wait();  // the multiplier update
+    // the multipliers of the sides this lane holds
     const bool top = i0 == 0 && s_top, left = j0 == 0 && s_lft, bot = pad_r && s_bot, rgt = pad_c && s_rgt;
-    float lt[4], ll[4], lr[4];
+    const bool low = bot || bottom_fill;
+    float lt[4], ll[4], lr[4], l_r = 0.f;
+    const ptrdiff_t et = (ptrdiff_t)(a - 1) * g.W + c0 + j0, eb = (ptrdiff_t)a * g.W + c0 + j0;
+    const ptrdiff_t el = (ptrdiff_t)(b - 1) * g.H + r0 + i0, er = (ptrdiff_t)b * g.H + r0 + i0;
+    const ptrdiff_t es = (ptrdiff_t)b * g.H + r0 + rank * BAND + rr;
+    if (!CHAIN) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      lt[c] = top && c < mc - j0 ? A.lamh[(ptrdiff_t)(a - 1) * g.W + c0 + j0 + c] : 0.f;
-      lb[c] = (bot || bottom_fill) && c < mc - j0 ? A.lamh[(size_t)a * g.W + c0 + j0 + c] : 0.f;
-      ll[c] = left && i0 + c < mr ? A.lamv[(size_t)(b - 1) * g.H + r0 + i0 + c] : 0.f;
-      lr[c] = rgt && i0 + c < mr ? A.lamv[(size_t)b * g.H + r0 + i0 + c] : 0.f;
+      for (int c = 0; c < 4; ++c) {
+        lt[c] = top && c < mc - j0 ? A.lamh[et + c] : 0.f;
+        lb[c] = low && c < mc - j0 ? A.lamh[eb + c] : 0.f;
+        ll[c] = left && i0 + c < mr ? A.lamv[el + c] : 0.f;
+        lr[c] = rgt && i0 + c < mr ? A.lamv[er + c] : 0.f;
+      }
+      if (right_lane) l_r = A.lamv[es];
+    } else {
+      // lambda + sigma (x_s - x_t), on this side's copy (kernels_interface.cu lam_step); branches,
+      // so that the warps without a side skip it
+      auto step = [&](const float* lam, const float* xs, const float* xt, ptrdiff_t e, int n, float* v, float* keep) {
+        float l0[4], s0[4], t0[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          l0[c] = c < n ? lam[e + c] : 0.f;
+          s0[c] = c < n ? xs[e + c] : 0.f;
+          t0[c] = c < n ? xt[e + c] : 0.f;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = fmaf(A.sigma, s0[c] - t0[c], l0[c]);
+        *reinterpret_cast<float4*>(keep) = make_float4(v[0], v[1], v[2], v[3]);
+      };
+      // (stored to global memory at the end: a store in flight here holds up the first release
+      // operation of the loop, 4096 x 4096 343 us per outer iteration instead of 223)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) lt[c] = lb[c] = ll[c] = lr[c] = 0.f;
+      if (top) step(A.lam_th, A.x_in.SB, A.x_in.ST, et, mc - j0, lt, smem + CH::LT + j0);
+      if (low) step(A.lam_sh, A.x_in.SB, A.x_in.ST, eb, mc - j0, lb, smem + CH::LT + BW + j0);
+      if (left) step(A.lam_tv, A.x_in.SR, A.x_in.SL, el, mr - i0, ll, smem + CH::LL + 4 * G);
+      if (PAD && rgt) step(A.lam_sv, A.x_in.SR, A.x_in.SL, er, mr - i0, lr, smem + CH::LL + BAND + 4 * G);
+      if (right_lane) {
+        l_r = fmaf(A.sigma, A.x_in.SR[es] - A.x_in.SL[es], A.lam_sv[es]);
+        smem[CH::LL + BAND + rr] = l_r;
+      }
     }
-    if (right_lane) hr_s = phat_s(pr_s, A.lamv[(size_t)b * g.H + r0 + rank * BAND + rr], tau);
+    if (right_lane) hr_s = phat_s(pr_s, l_r, tau);
 
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -409,6 +556,26 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
       }
       *reinterpret_cast<float4*>(myF + kH1 + 4 * NT * c) = make_float4(h1[0][c], h1[2][c], h1[1][c], h1[3][c]);
       *reinterpret_cast<float4*>(myF + kH2 + 4 * NT * c) = make_float4(h2[0][c], h2[2][c], h2[1][c], h2[3][c]);
+    }
+    if (CHAIN) {  // p~^n of the sides, for their extrapolation at the end
+      if (top) *reinterpret_cast<float4*>(smem + CH::OT + j0) = make_float4(p1[0][0], p1[0][1], p1[0][2], p1[0][3]);
+      if (bottom_fill) *reinterpret_cast<float4*>(smem + CH::OT + BW + j0) = make_float4(qb[0], qb[1], qb[2], qb[3]);
+      if (left) *reinterpret_cast<float4*>(smem + CH::OL + 4 * G) = make_float4(p2[0][0], p2[1][0], p2[2][0], p2[3][0]);
+      if (PAD && bot) {
+        auto put = [&](int r) { *reinterpret_cast<float4*>(smem + CH::OT + BW + j0) = make_float4(p1[r][0], p1[r][1], p1[r][2], p1[r][3]); };
+        if (rpad == 0) put(0);
+        else if (rpad == 1) put(1);
+        else if (rpad == 2) put(2);
+        else put(3);
+      }
+      if (PAD && rgt) {
+        auto put = [&](int c) { *reinterpret_cast<float4*>(smem + CH::OL + BAND + 4 * G) = make_float4(p2[0][c], p2[1][c], p2[2][c], p2[3][c]); };
+        if (cpad == 0) put(0);
+        else if (cpad == 1) put(1);
+        else if (cpad == 2) put(2);
+        else put(3);
+      }
+      if (right_lane) smem[CH::OL + BAND + rr] = pr_s;
     }
     *reinterpret_cast<float4*>(sQ1 + G * BW + j0) = make_float4(p1[0][0], p1[0][1], p1[0][2], p1[0][3]);
     *reinterpret_cast<ulonglong2*>(myQL) = make_ulonglong2(P2[0][0], P2[0][1]);
@@ -747,7 +914,7 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   int tid2 = tid, a2 = a, b2 = b;
   asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid2));
   asm volatile("" : "+r"(a2), "+r"(b2));
-  tile_store<LPR, NW, PAD>(A, out, a2, b2, tid2, CL, rank, U, P1, P2, pr_s);
+  tile_store<LPR, NW, PAD, CHAIN, CH>(A, out, a2, b2, tid2, CL, rank, U, P1, P2, pr_s);
   if (CLU) {
     if (timed_out) atomicOr(A.err, 1);
     __syncwarp();
@@ -755,42 +922,47 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
   }
 }
 
-// 16 warps per SM: 128 registers per thread
-template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
-__global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile(const LocalArgs A, const int cl) {
+template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK, bool CHAIN>
+__global__ void __launch_bounds__(32 * NW, tile_warps(NW, PAD && CHAIN) / NW) k_tile(const LocalArgs A, const int cl) {
   // block x = CTA x % cl of subdomain x / cl (a 1-D grid: any number of subdomains)
   const unsigned t = CLU ? blockIdx.x / (unsigned)cl : blockIdx.x, rank = CLU ? blockIdx.x - t * (unsigned)cl : 0u;
   const unsigned a = t / (unsigned)A.g.NC;
-  tile_solve<LPR, NW, CLU, PAD, FID, MASK>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank, CLU ? cl : 1);
+  tile_solve<LPR, NW, CLU, PAD, FID, MASK, CHAIN>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank, CLU ? cl : 1);
 }
 
 // adaptive inner stop, subdomains that fill their block
-template <int LPR, int NW, int FID, bool MASK>
+template <int LPR, int NW, int FID, bool MASK, bool CHAIN>
 __global__ void __launch_bounds__(32 * NW, 16 / NW) k_tile_adapt(const LocalArgs A, const int cl) {
   const unsigned t = blockIdx.x / (unsigned)cl, rank = blockIdx.x - t * (unsigned)cl, a = t / (unsigned)A.g.NC;
-  tile_solve<LPR, NW, true, false, FID, MASK, false, true>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank, cl);
+  tile_solve<LPR, NW, true, false, FID, MASK, CHAIN, false, true>(A, A.out, (int)a, (int)(t - a * (unsigned)A.g.NC), (int)rank, cl);
 }
 
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
-cudaError_t prepare_tile_one() {
-  return cudaFuncSetAttribute(k_tile<LPR, NW, CLU, PAD, FID, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(use_mask_words(CLU, MASK, false, false) ? MaskTileLayout<LPR, NW>::BYTES : TileLayout<LPR, NW>::BYTES));
+cudaError_t prepare_tile_one(bool chain) {
+  constexpr bool words = use_mask_words(CLU, MASK, false, false);
+  auto set = [](auto kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  const cudaError_t e = set(k_tile<LPR, NW, CLU, PAD, FID, MASK, false>, tile_bytes<LPR, NW, words, false, false>());
+  return e != cudaSuccess || !chain
+             ? e
+             : set(k_tile<LPR, NW, CLU, PAD, FID, MASK, true>, tile_bytes<LPR, NW, words, false, true>());
 }
 
 template <int LPR, int NW, bool CLU, bool PAD>
-cudaError_t prepare_tile_fid() {
+cudaError_t prepare_tile_fid(bool chain) {
   cudaError_t e;
-  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L2, false>()) != cudaSuccess) return e;
-  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L2, true>()) != cudaSuccess) return e;
-  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L1, false>()) != cudaSuccess) return e;
-  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L1, true>()) != cudaSuccess) return e;
-  return prepare_tile_one<LPR, NW, CLU, PAD, FID_SEG, false>();
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L2, false>(chain)) != cudaSuccess) return e;
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L2, true>(chain)) != cudaSuccess) return e;
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L1, false>(chain)) != cudaSuccess) return e;
+  if ((e = prepare_tile_one<LPR, NW, CLU, PAD, FID_L1, true>(chain)) != cudaSuccess) return e;
+  return prepare_tile_one<LPR, NW, CLU, PAD, FID_SEG, false>(chain);
 }
 
+// the instances a grid with or without padding reaches, the chained ones if asked for
 template <int LPR, int NW, bool CLU>
-cudaError_t prepare_tile() {
-  const cudaError_t e = prepare_tile_fid<LPR, NW, CLU, false>();
-  return e != cudaSuccess ? e : prepare_tile_fid<LPR, NW, CLU, true>();
+cudaError_t prepare_tile(bool pad, bool chain) {
+  return pad ? prepare_tile_fid<LPR, NW, CLU, true>(chain) : prepare_tile_fid<LPR, NW, CLU, false>(chain);
 }
 
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
@@ -798,18 +970,20 @@ cudaError_t launch_tile_one(const LocalArgs& a, int cl, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(CLU ? cl : 1) * a.g.NC * a.g.NR, 1, 1);
   cfg.blockDim = dim3(32 * NW, 1, 1);
-  cfg.dynamicSmemBytes = use_mask_words(CLU, MASK, false, false) ? MaskTileLayout<LPR, NW>::BYTES : TileLayout<LPR, NW>::BYTES;
+  constexpr bool words = use_mask_words(CLU, MASK, false, false);
+  cfg.dynamicSmemBytes = a.chain ? tile_bytes<LPR, NW, words, false, true>() : tile_bytes<LPR, NW, words, false, false>();
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   cfg.attrs = attr;
-  if (has_interfaces(a.g)) pdl_attr(&attr[cfg.numAttrs++]);
+  if (a.chain || has_interfaces(a.g)) pdl_attr(&attr[cfg.numAttrs++]);
   if (CLU) {
     attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
     attr[cfg.numAttrs].val.clusterDim.x = cl;
     attr[cfg.numAttrs].val.clusterDim.y = 1;
     attr[cfg.numAttrs++].val.clusterDim.z = 1;
   }
-  return cudaLaunchKernelEx(&cfg, k_tile<LPR, NW, CLU, PAD, FID, MASK>, a, cl);
+  return a.chain ? cudaLaunchKernelEx(&cfg, k_tile<LPR, NW, CLU, PAD, FID, MASK, true>, a, cl)
+                 : cudaLaunchKernelEx(&cfg, k_tile<LPR, NW, CLU, PAD, FID, MASK, false>, a, cl);
 }
 
 template <int LPR, int NW, bool CLU, bool PAD>

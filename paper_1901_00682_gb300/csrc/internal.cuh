@@ -45,6 +45,16 @@ struct LocalArgs {
   const float* lamh;     // (NR-1) x W
   const float* lamv;     // (NC-1) x H
   Strips out;            // strips of p~^{n+1} (written at the end)
+  // chain != 0 (micro-tile kernel only): the local solve makes the multiplier update itself.
+  // Every side keeps its own copy of the multipliers (lam_s: lower / right sides, in the
+  // layout of lamh and lamv; lam_t: upper / left sides), which both owners of an interface
+  // update with the same operations from the extrapolated strips x_in = 2 p~^n - p~^{n-1}; x_out
+  // receives 2 p~^{n+1} - p~^n.  (With a launch of its own the update cost 2 to 3 us per outer
+  // iteration.)
+  int chain;
+  float sigma;
+  float *lam_sh, *lam_sv, *lam_th, *lam_tv;
+  Strips x_in, x_out;
   const Coef* coef;      // K coefficient sets (device)
   int* err;              // set non-zero by a kernel whose bounded wait ran out
   // adaptive inner stopping (eq. stop_inner1); inner_tol2 = 0 selects K fixed iterations
@@ -142,6 +152,9 @@ cudaError_t launch_extract_strips(const Grid& g, const float* P1, const float* P
 // P1/P2 <- 0 except the interface values, taken from the strips
 cudaError_t launch_scatter_strips(const Grid& g, Strips s, float* P1, float* P2, cudaStream_t st);
 
+// x <- 2 cur - prev over n floats (whole strip sets), the extrapolation of launch_interface
+cudaError_t launch_extrapolate(long long n, const float* cur, const float* prev, float* x, cudaStream_t st);
+
 cudaError_t launch_interface_batch(const BatchIfaceArgs& a, int total4, cudaStream_t st);
 
 // ---- kernels_fused.cu
@@ -155,9 +168,12 @@ cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, in
 // One outer iteration's local solves, all tiles, fused (returns cudaErrorInvalidValue
 // if no fused configuration fits the tile shape).
 cudaError_t launch_fused_local(const LocalArgs& a, int fidelity, int variant, cudaStream_t st);
-// Sets the shared-memory opt-in of every fused configuration on the current device
-// (called at handle creation, outside any stream capture).
-cudaError_t fused_prepare();
+// Whether the local solves should make the multiplier update themselves (LocalArgs.chain).
+bool fused_chains(const Grid& g, int variant, int K, bool adaptive);
+// Sets the shared-memory opt-in of the kernels that launch_fused_local (the batch launch) can
+// reach on the current device (called at handle creation, outside any stream capture).
+cudaError_t fused_prepare(const Grid& g, int variant, bool adaptive);
+cudaError_t fused_prepare_batch(int tile, int variant);
 // Whether launch_fused_local(a, ., variant) with a fixed inner count reads a.u0, a.P10, a.P20
 // (rather than working in place on a.u, a.P1, a.P2).
 bool fused_out_of_place(const Grid& g, int variant);
@@ -172,6 +188,7 @@ int fused_num_variants();
 bool fused_mt_supported(const LocalArgs& a);
 cudaError_t launch_fused_mt(const LocalArgs& a, int fidelity, cudaStream_t st);
 cudaError_t fused_mt_prepare();
+cudaError_t fused_mt_batch_prepare();
 // The same kernel over the work list of a batch (every image's arrays 16-byte aligned).
 cudaError_t launch_fused_mt_batch(const BatchArgs& B, int total_tiles, cudaStream_t st);
 
@@ -186,17 +203,24 @@ struct TilePlan {
 // false if a subdomain is larger than 128 x 128
 bool tile_plan(const Grid& g, TilePlan* p);
 
+// Warps of the micro-tile kernel per SM: 16 at 128 registers a thread; 12 where padding and the
+// multiplier update come together and spill (321 x 481 15.0 us per outer iteration with 16).
+constexpr int tile_warps(int nw, bool pad_chain) { return pad_chain && nw <= 4 ? 12 : 16; }
+
 // launch_tile_<lpr>_<nw>
 cudaError_t launch_tile_8_2(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
 cudaError_t launch_tile_8_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
 cudaError_t launch_tile_16_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
 cudaError_t launch_tile_16_8(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
 cudaError_t launch_tile_32_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st);
-cudaError_t prepare_tile_8_2();
-cudaError_t prepare_tile_8_4();
-cudaError_t prepare_tile_16_4();
-cudaError_t prepare_tile_16_8();
-cudaError_t prepare_tile_32_4();
+cudaError_t prepare_tile_8_2(bool pad, bool chain);
+cudaError_t prepare_tile_8_4(bool pad, bool chain);
+cudaError_t prepare_tile_16_4(bool pad, bool chain);
+cudaError_t prepare_tile_16_8(bool pad, bool chain);
+cudaError_t prepare_tile_32_4(bool pad, bool chain);
+cudaError_t prepare_tile_adapt_128(bool chain);
+cudaError_t prepare_tile_batch_128();
+cudaError_t prepare_tile_batch_64();
 // the adaptive inner stop (a.inner_tol2 > 0), every subdomain exactly 128 x 128
 cudaError_t launch_tile_adapt_128(const LocalArgs& a, int fid, cudaStream_t st);
 // every subdomain of every image of a batch, 64 x 64 or 128 x 128
@@ -265,7 +289,7 @@ cudaError_t launch_adj_fused(const LocalArgs& a, const AdjArgs& z, int fidelity,
 // floats of the fused reverse kernel's tape (0 if the tile shape is not supported)
 size_t adj_fused_tape_floats(const Grid& g, int K);
 // shared-memory opt-in of the fused reverse kernels (outside any stream capture)
-cudaError_t adj_fused_prepare();
+cudaError_t adj_fused_prepare(const Grid& g);
 // alpha partial-sum slots the fused reverse kernel uses
 long long adj_alpha_slots_fused(const Grid& g);
 // launch_adj_tile_<lpr>_<nw>
@@ -274,9 +298,11 @@ cudaError_t launch_adj_tile_8_4(const LocalArgs& a, const AdjArgs& z, int fid, i
 cudaError_t launch_adj_tile_16_4(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st);
 cudaError_t launch_adj_tile_16_8(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st);
 cudaError_t launch_adj_tile_32_4(const LocalArgs& a, const AdjArgs& z, int fid, int cl, bool pad, cudaStream_t st);
-cudaError_t prepare_adj_tile_8();
-cudaError_t prepare_adj_tile_16();
-cudaError_t prepare_adj_tile_32();
+cudaError_t prepare_adj_tile_8_2();
+cudaError_t prepare_adj_tile_8_4();
+cudaError_t prepare_adj_tile_16_4();
+cudaError_t prepare_adj_tile_16_8();
+cudaError_t prepare_adj_tile_32_4();
 
 // ---- kernels_misc.cu
 // u0 = f (0 on D) for L2/L1, 1/2 for SEG

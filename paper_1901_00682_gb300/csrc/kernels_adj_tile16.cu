@@ -10,9 +10,7 @@ cudaError_t launch_adj_tile_16_4(const LocalArgs& a, const AdjArgs& z, int fid, 
 cudaError_t launch_adj_tile_16_8(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st) {
   return launch_adj_tile<16, 8, false, true>(a, z, fid, cl, st);
 }
-cudaError_t prepare_adj_tile_16() {
-  const cudaError_t e = prepare_adj_tile<16, 4, true, true>();
-  return e != cudaSuccess ? e : prepare_adj_tile<16, 8, false, true>();
-}
+cudaError_t prepare_adj_tile_16_4() { return prepare_adj_tile<16, 4, true, true>(); }
+cudaError_t prepare_adj_tile_16_8() { return prepare_adj_tile<16, 8, false, true>(); }
 
 }  // namespace ddtv

@@ -10,9 +10,7 @@ cudaError_t launch_adj_tile_8_2(const LocalArgs& a, const AdjArgs& z, int fid, i
 cudaError_t launch_adj_tile_8_4(const LocalArgs& a, const AdjArgs& z, int fid, int cl, cudaStream_t st) {
   return launch_adj_tile<8, 4, true, true>(a, z, fid, cl, st);
 }
-cudaError_t prepare_adj_tile_8() {
-  const cudaError_t e = prepare_adj_tile<8, 2, false, true>();
-  return e != cudaSuccess ? e : prepare_adj_tile<8, 4, true, true>();
-}
+cudaError_t prepare_adj_tile_8_2() { return prepare_adj_tile<8, 2, false, true>(); }
+cudaError_t prepare_adj_tile_8_4() { return prepare_adj_tile<8, 4, true, true>(); }
 
 }  // namespace ddtv

@@ -18,11 +18,12 @@ size_t adj_fused_tape_floats(const Grid& g, int K) {
   return (size_t)g.NR * g.NC * p.cl * 32 * p.nw * kTapeWords * K;
 }
 
-cudaError_t adj_fused_prepare() {
-  cudaError_t e;
-  if ((e = prepare_adj_tile_8()) != cudaSuccess) return e;
-  if ((e = prepare_adj_tile_16()) != cudaSuccess) return e;
-  return prepare_adj_tile_32();
+cudaError_t adj_fused_prepare(const Grid& g) {
+  TilePlan p;
+  if (!tile_plan(g, &p)) return cudaErrorInvalidValue;
+  if (p.lpr == 8) return p.nw == 2 ? prepare_adj_tile_8_2() : prepare_adj_tile_8_4();
+  if (p.lpr == 16) return p.nw == 8 ? prepare_adj_tile_16_8() : prepare_adj_tile_16_4();
+  return prepare_adj_tile_32_4();
 }
 
 cudaError_t launch_adj_fused(const LocalArgs& a, const AdjArgs& z, int fid, cudaStream_t st) {

@@ -438,18 +438,52 @@ void fused_max_tile(int* rows, int* cols) {
 
 int fused_num_variants() { return kNumVariants; }
 
-cudaError_t fused_prepare() {
-  cudaError_t e;
-  if ((e = prepare_fid<32, 8, 4, 1, true>()) != cudaSuccess) return e;
-  if ((e = prepare_fid<64, 8, 8, 1, true>()) != cudaSuccess) return e;
-  if ((e = prepare_fid<128, 8, 2, 8, true>()) != cudaSuccess) return e;
-  if ((e = prepare_fid<128, 8, 2, 8, false>()) != cudaSuccess) return e;
-  if ((e = prepare_tile_8_2()) != cudaSuccess) return e;
-  if ((e = prepare_tile_8_4()) != cudaSuccess) return e;
-  if ((e = prepare_tile_16_4()) != cudaSuccess) return e;
-  if ((e = prepare_tile_16_8()) != cudaSuccess) return e;
-  if ((e = prepare_tile_32_4()) != cudaSuccess) return e;
-  return fused_mt_prepare();
+// The adaptive stop runs in the micro-tile kernel for the default of exact 128 x 128
+// subdomains.  (W + N_c a multiple of 4 and K <= 64 are no needs of it, but its residual sums
+// are float32 where those of the cluster-barrier kernel are float64, so a near tie could stop
+// a subdomain one iteration apart: every problem keeps the sums it has always had.)
+static bool adapt_in_tile(const Grid& g, int variant, int K) {
+  return g.H == 128 * g.NR && g.W == 128 * g.NC && variant == 0 && K <= 64 && (g.W + g.NC) % 4 == 0;
+}
+
+// In the micro-tile kernel and where one wave holds the launch (on the 148 SMs that
+// take clusters).  The update then saves a launch on the chain of latencies: 128 x 128 in 64 x
+// 64 11.4 -> 10.9 us per outer iteration, 512 x 512 in 128 x 128 13.0 -> 12.0, 1024 x 1024 18.6 ->
+// 17.9.  With several waves the update of the sides costs more instructions than its own
+// launch, which overlaps with the loads: 4096 x 4096 216 -> 224.
+bool fused_chains(const Grid& g, int variant, int K, bool adaptive) {
+  const bool exact128 = g.H == 128 * g.NR && g.W == 128 * g.NC;
+  TilePlan p;
+  if (!(adaptive ? adapt_in_tile(g, variant, K) : variant <= 1 || !exact128) || !tile_plan(g, &p)) return false;
+  return (long long)g.NR * g.NC * p.cl * p.nw <= 148 * tile_warps(p.nw, p.pad);
+}
+
+// Every handle prepares the kernels it can reach and no others: an attribute call per
+// kernel instance is most of what creating a small handle costs.
+cudaError_t fused_prepare(const Grid& g, int variant, bool adaptive) {
+  TilePlan p;
+  if (!tile_plan(g, &p)) return cudaErrorInvalidValue;
+  const bool exact128 = g.H == 128 * g.NR && g.W == 128 * g.NC;
+  const bool chain = fused_chains(g, variant, 1, adaptive);  // (whatever the inner count)
+  cudaError_t e = cudaSuccess;
+  if (adaptive) {
+    if (exact128 && variant == 0 && (e = prepare_tile_adapt_128(chain)) != cudaSuccess) return e;
+    switch (pick((g.H + g.NR - 1) / g.NR, (g.W + g.NC - 1) / g.NC)) {
+      case 0: return prepare_fid<32, 8, 4, 1, true>();
+      case 1: return prepare_fid<64, 8, 8, 1, true>();
+      default: return prepare_fid<128, 8, 2, 8, true>();
+    }
+  }
+  if (exact128 && variant == 3) return prepare_fid<128, 8, 2, 8, false>();
+  if (exact128 && variant == 2 && (e = fused_mt_prepare()) != cudaSuccess) return e;
+  if (p.lpr == 8) return p.nw == 2 ? prepare_tile_8_2(p.pad, chain) : prepare_tile_8_4(p.pad, chain);
+  if (p.lpr == 16) return p.nw == 8 ? prepare_tile_16_8(p.pad, chain) : prepare_tile_16_4(p.pad, chain);
+  return prepare_tile_32_4(p.pad, chain);
+}
+
+cudaError_t fused_prepare_batch(int tile, int variant) {
+  if (tile == 64) return prepare_tile_batch_64();
+  return variant == 2 ? fused_mt_batch_prepare() : prepare_tile_batch_128();
 }
 
 cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, int variant, bool overlap,
@@ -468,11 +502,7 @@ cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStr
   const int mr = (a.g.H + a.g.NR - 1) / a.g.NR, mc = (a.g.W + a.g.NC - 1) / a.g.NC;
   const bool exact128 = a.g.H == 128 * a.g.NR && a.g.W == 128 * a.g.NC;  // every tile exactly 128 x 128
   if (a.inner_tol2 > 0.0) {
-    // the micro-tile kernel for the default of exact 128 x 128 subdomains.  (W + N_c a multiple
-    // of 4 and K <= 64 are no needs of it, but its residual sums are float32 where those of
-    // the kernel below are float64, so a near tie could stop a subdomain one iteration
-    // apart: every problem keeps the sums it has always had.)
-    if (exact128 && variant == 0 && a.K <= 64 && (a.g.W + a.g.NC) % 4 == 0) return launch_tile_adapt_128(a, fid, st);
+    if (adapt_in_tile(a.g, variant, a.K)) return launch_tile_adapt_128(a, fid, st);
     switch (pick(mr, mc)) {
       case 0: return launch_fid<32, 8, 4, 1, true>(a, fid, st);
       case 1: return launch_fid<64, 8, 8, 1, true>(a, fid, st);

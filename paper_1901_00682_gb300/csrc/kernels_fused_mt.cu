@@ -924,8 +924,7 @@ cudaError_t fused_mt_prepare() {
   if ((e = prepare_mt_one<FID_L2, true>()) != cudaSuccess) return e;
   if ((e = prepare_mt_one<FID_L1, false>()) != cudaSuccess) return e;
   if ((e = prepare_mt_one<FID_L1, true>()) != cudaSuccess) return e;
-  if ((e = prepare_mt_one<FID_SEG, false>()) != cudaSuccess) return e;
-  return fused_mt_batch_prepare();
+  return prepare_mt_one<FID_SEG, false>();
 }
 
 cudaError_t launch_fused_mt(const LocalArgs& a, int fid, cudaStream_t st) {

@@ -1,7 +1,8 @@
 // Interface step of Algorithm 1: the multiplier update
 //   lambda^{n+1} = lambda^n + sigma B (2 p~^n - p~^{n-1}),
 //   (B p~)_e = p_s(e) - p_t(e)   (s the upper/left tile, t the lower/right one, Section 2.4),
-// on compact interface strips, plus the kernels that move strips in and out of the
+// on compact interface strips (where the local solve does not make it itself, LocalArgs.chain),
+// plus the kernels that move strips in and out of the
 // torn field.  The update is HBM-bound: 5 float reads and 1 write per interface edge.
 #include "internal.cuh"
 
@@ -59,6 +60,12 @@ __global__ void k_interface_v1(int nh, int nv, float sigma, const float* __restr
       lamv[q] = lam_step(lamv[q], sigma, cSR[q], pSR[q], cSL[q], pSL[q]);
     }
   }
+}
+
+__global__ void k_extrapolate(long long n, const float* __restrict__ cur, const float* __restrict__ prev,
+                              float* __restrict__ x) {
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
+    x[e] = fmaf(2.0f, cur[e], -prev[e]);
 }
 
 // strips <- interface values of (P1, P2): one thread per interface edge
@@ -168,6 +175,12 @@ cudaError_t launch_interface(const Grid& g, float sigma, Strips cur, Strips prev
   }
   return launch_pdl(k_interface_v1, grid_for(nh + nv, block), block, st, nh, nv, sigma, cur.SB, cur.ST, prev.SB,
                     prev.ST, lamh, cur.SR, cur.SL, prev.SR, prev.SL, lamv);
+}
+
+cudaError_t launch_extrapolate(long long n, const float* cur, const float* prev, float* x, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  k_extrapolate<<<grid_for(n, 256), 256, 0, st>>>(n, cur, prev, x);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_interface_batch(const BatchIfaceArgs& a, int total4, cudaStream_t st) {

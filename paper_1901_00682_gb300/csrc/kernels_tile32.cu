@@ -10,28 +10,31 @@ cudaError_t launch_adapt_one(const LocalArgs& a, int cl, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)cl * a.g.NC * a.g.NR, 1, 1);
   cfg.blockDim = dim3(128, 1, 1);
-  cfg.dynamicSmemBytes = AdaptTileLayout<32, 4>::BYTES;
+  cfg.dynamicSmemBytes = a.chain ? tile_bytes<32, 4, false, true, true>() : tile_bytes<32, 4, false, true, false>();
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   cfg.attrs = attr;
-  if (has_interfaces(a.g)) pdl_attr(&attr[cfg.numAttrs++]);
+  if (a.chain || has_interfaces(a.g)) pdl_attr(&attr[cfg.numAttrs++]);
   attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
   attr[cfg.numAttrs].val.clusterDim.x = cl;
   attr[cfg.numAttrs].val.clusterDim.y = 1;
   attr[cfg.numAttrs++].val.clusterDim.z = 1;
-  return cudaLaunchKernelEx(&cfg, k_tile_adapt<32, 4, FID, MASK>, a, cl);
+  return a.chain ? cudaLaunchKernelEx(&cfg, k_tile_adapt<32, 4, FID, MASK, true>, a, cl)
+                 : cudaLaunchKernelEx(&cfg, k_tile_adapt<32, 4, FID, MASK, false>, a, cl);
 }
 
+template <bool CHAIN>
 cudaError_t prepare_adapt() {
   auto set = [](auto kern) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AdaptTileLayout<32, 4>::BYTES);
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)tile_bytes<32, 4, false, true, CHAIN>());
   };
   cudaError_t e;
-  if ((e = set(k_tile_adapt<32, 4, FID_L2, false>)) != cudaSuccess) return e;
-  if ((e = set(k_tile_adapt<32, 4, FID_L2, true>)) != cudaSuccess) return e;
-  if ((e = set(k_tile_adapt<32, 4, FID_L1, false>)) != cudaSuccess) return e;
-  if ((e = set(k_tile_adapt<32, 4, FID_L1, true>)) != cudaSuccess) return e;
-  return set(k_tile_adapt<32, 4, FID_SEG, false>);
+  if ((e = set(k_tile_adapt<32, 4, FID_L2, false, CHAIN>)) != cudaSuccess) return e;
+  if ((e = set(k_tile_adapt<32, 4, FID_L2, true, CHAIN>)) != cudaSuccess) return e;
+  if ((e = set(k_tile_adapt<32, 4, FID_L1, false, CHAIN>)) != cudaSuccess) return e;
+  if ((e = set(k_tile_adapt<32, 4, FID_L1, true, CHAIN>)) != cudaSuccess) return e;
+  return set(k_tile_adapt<32, 4, FID_SEG, false, CHAIN>);
 }
 
 }  // namespace
@@ -49,12 +52,9 @@ cudaError_t launch_tile_adapt_128(const LocalArgs& a, int fid, cudaStream_t st) 
 cudaError_t launch_tile_32_4(const LocalArgs& a, int fid, int cl, bool pad, cudaStream_t st) {
   return launch_tile<32, 4, true>(a, fid, cl, pad, st);
 }
-cudaError_t prepare_tile_32_4() {
-  cudaError_t e;
-  if ((e = prepare_adapt()) != cudaSuccess) return e;
-  if ((e = prepare_tile_batch<32, 4, 8>()) != cudaSuccess) return e;
-  return prepare_tile<32, 4, true>();
-}
+cudaError_t prepare_tile_32_4(bool pad, bool chain) { return prepare_tile<32, 4, true>(pad, chain); }
+cudaError_t prepare_tile_batch_128() { return prepare_tile_batch<32, 4, 8>(); }
+cudaError_t prepare_tile_adapt_128(bool chain) { return chain ? prepare_adapt<true>() : prepare_adapt<false>(); }
 cudaError_t launch_tile_batch_128(const BatchArgs& B, int total_tiles, bool overlap, cudaStream_t st) {
   return launch_tile_batch<32, 4, 8>(B, total_tiles, overlap, st);
 }
