@@ -82,10 +82,11 @@ typedef struct {
   int energy_every;       /* with outer_tol: evaluate J every energy_every outer iterations  */
   int path;               /* dd_tv_path                                                    */
   int variant;            /* fused path, hardware mapping of exact 128 x 128 subdomains:
-                             0 the micro-tile kernel of every other tile shape
-                             (default); 1 the same; 2 persistent 2 x 4 micro-tiles; 3
-                             one cluster per subdomain with cluster barriers.  The
-                             arithmetic and results do not depend on it               */
+                             0 the micro-tile kernel of every other tile shape, or 1
+                             where that is faster (default); 1 persistent 4 x 4
+                             micro-tiles, state moved by tensor copies; 2 persistent 2
+                             x 4 micro-tiles; 3 one cluster per subdomain with cluster
+                             barriers.  The arithmetic and results do not depend on it */
   double inner_tol;       /* >= 0.  0: every local solve runs inner_iters iterations.  > 0:
                              adaptive inner stopping (Section 5, eq. stop_inner1): a
                              subdomain stops after the first inner iteration k with
@@ -201,7 +202,7 @@ int dd_tv_current_energy(dd_tv* h, double* J_out);
  * directly (no graph replay) and bracket every phase with CUDA events on the
  * handle's stream.  dd_tv_profile_read synchronises and writes, for each phase
  * (0 = interface multiplier update where it is a launch of its own, 1 = local solves,
- * which make the update themselves on the fused path's default, 2 = energy reduction), the
+ * which make the update themselves where one wave holds them, 2 = energy reduction), the
  * summed device time in milliseconds and the number of kernel launches since
  * profiling was switched on (arrays of 3; either pointer may be NULL); it then
  * resets the counters.  dd_tv_set_profiling(h, 0) returns to graph replay. */

@@ -964,7 +964,7 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
   }
   cudaGetDevice(&h->device);
   if (p->path == DD_TV_PATH_FUSED) {
-    cudaError_t e = fused_prepare(h->g, p->variant, p->inner_tol > 0.0);
+    cudaError_t e = fused_prepare(h->g, p->variant, p->inner_iters, p->inner_tol * p->inner_tol);
     if (e != cudaSuccess) {
       std::snprintf(g_create_err, sizeof(g_create_err), "fused kernel set-up: %s", cudaGetErrorString(e));
       delete h;
@@ -1038,7 +1038,7 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
       h->strips_k[s].ST += skip;
     }
   }
-  h->chain = p->path == DD_TV_PATH_FUSED && !h->shard && fused_chains(g, p->variant, p->inner_iters, p->inner_tol > 0.0);
+  h->chain = p->path == DD_TV_PATH_FUSED && !h->shard && fused_chains(g, p->variant, p->inner_iters, p->inner_tol * p->inner_tol);
   if (h->chain && h->nh + h->nv) {
     const size_t ne = h->nh + h->nv;
     if ((rc = dalloc(h, &h->x_mem, 5 * ne))) {

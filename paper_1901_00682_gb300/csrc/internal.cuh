@@ -169,10 +169,10 @@ cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, in
 // if no fused configuration fits the tile shape).
 cudaError_t launch_fused_local(const LocalArgs& a, int fidelity, int variant, cudaStream_t st);
 // Whether the local solves should make the multiplier update themselves (LocalArgs.chain).
-bool fused_chains(const Grid& g, int variant, int K, bool adaptive);
+bool fused_chains(const Grid& g, int variant, int K, double inner_tol2);
 // Sets the shared-memory opt-in of the kernels that launch_fused_local (the batch launch) can
 // reach on the current device (called at handle creation, outside any stream capture).
-cudaError_t fused_prepare(const Grid& g, int variant, bool adaptive);
+cudaError_t fused_prepare(const Grid& g, int variant, int K, double inner_tol2);
 cudaError_t fused_prepare_batch(int tile, int variant);
 // Whether launch_fused_local(a, ., variant) with a fixed inner count reads a.u0, a.P10, a.P20
 // (rather than working in place on a.u, a.P1, a.P2).
@@ -191,6 +191,15 @@ cudaError_t fused_mt_prepare();
 cudaError_t fused_mt_batch_prepare();
 // The same kernel over the work list of a batch (every image's arrays 16-byte aligned).
 cudaError_t launch_fused_mt_batch(const BatchArgs& B, int total_tiles, cudaStream_t st);
+
+// ---- kernels_fused_mt4.cu
+// Persistent fused local solver on 4 x 4 micro-tiles, one warp per thread row, three
+// 128-thread CTAs per SM, the state moved by tensor copies; 128 x 128 tiles with 16-byte
+// aligned rows (fused_mt4_supported), in place, fixed inner count or (a.inner_tol2 > 0) the
+// adaptive stop.  cudaErrorNotSupported if the tensor maps cannot be encoded.
+bool fused_mt4_supported(const LocalArgs& a);
+cudaError_t launch_fused_mt4(const LocalArgs& a, int fidelity, cudaStream_t st);
+cudaError_t fused_mt4_prepare(bool adaptive);
 
 // ---- kernels_tile8.cu, kernels_tile16.cu, kernels_tile32.cu (fused_tile.cuh)
 // How the micro-tile kernels cover the subdomains of a grid: lpr lanes per row group (a

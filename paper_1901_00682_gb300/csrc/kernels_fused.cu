@@ -336,7 +336,8 @@ __global__ void __launch_bounds__(BW* TR, (BW * TR <= 256 ? 2 : 1)) k_fused(cons
 }
 
 // Hardware mappings of exact 128 x 128 subdomains (dd_tv_params.variant):
-//   0  the micro-tile kernel of every other shape (fused_tile.cuh); 1 the same
+//   0  the micro-tile kernel of every other shape (fused_tile.cuh), or 1 where that is faster
+//   1  persistent 4 x 4 micro-tiles, state moved by tensor copies
 //   2  persistent 2 x 4 micro-tiles, 256 threads, 2 CTAs per SM
 //   3  the cluster-barrier kernel (one subdomain per cluster)
 constexpr int kNumVariants = 4;
@@ -438,34 +439,77 @@ void fused_max_tile(int* rows, int* cols) {
 
 int fused_num_variants() { return kNumVariants; }
 
-// The adaptive stop runs in the micro-tile kernel for the default of exact 128 x 128
-// subdomains.  (W + N_c a multiple of 4 and K <= 64 are no needs of it, but its residual sums
-// are float32 where those of the cluster-barrier kernel are float64, so a near tie could stop
-// a subdomain one iteration apart: every problem keeps the sums it has always had.)
-static bool adapt_in_tile(const Grid& g, int variant, int K) {
-  return g.H == 128 * g.NR && g.W == 128 * g.NC && variant == 0 && K <= 64 && (g.W + g.NC) % 4 == 0;
+namespace {
+
+bool exact_128(const Grid& g) { return g.H == 128 * g.NR && g.W == 128 * g.NC; }
+
+// Whether one wave holds a launch of the micro-tile kernel (on the 148 SMs that take
+// clusters).
+bool one_wave(const Grid& g, const TilePlan& p) {
+  return (long long)g.NR * g.NC * p.cl * p.nw <= 148 * tile_warps(p.nw, p.pad);
 }
 
-// In the micro-tile kernel and where one wave holds the launch (on the 148 SMs that
-// take clusters).  The update then saves a launch on the chain of latencies: 128 x 128 in 64 x
-// 64 11.4 -> 10.9 us per outer iteration, 512 x 512 in 128 x 128 13.0 -> 12.0, 1024 x 1024 18.6 ->
-// 17.9.  With several waves the update of the sides costs more instructions than its own
-// launch, which overlaps with the loads: 4096 x 4096 216 -> 224.
-bool fused_chains(const Grid& g, int variant, int K, bool adaptive) {
-  const bool exact128 = g.H == 128 * g.NR && g.W == 128 * g.NC;
+// The persistent 4 x 4 kernel: variant 1, and the default of launches of several waves with
+// few inner iterations.  It has the next subdomain's loads on their way while this one
+// iterates, where a CTA of the micro-tile kernel waits for its own; with four CTAs per SM
+// instead of three that one iterates faster.  us per outer iteration, persistent / micro-tile:
+//
+//   state beyond L2     K = 1        2           3            4            10
+//   4096 x 4096     82 / 94    94 / 108   111 / 118    127 / 130    231 / 216
+//   2560 x 2560     35 / 40    42 / 46     49 / 50      55 / 56
+//   ... with a mask 40 / 44    47 / 50     54 / 54      62 / 59
+//   state in L2
+//   2048 x 2048     23.1 / 24.2  27.7 / 28.4  32.4 / 31.2  36.0 / 35.4
+//   ... with a mask 24.5 / 24.7  29.9 / 28.3  34.7 / 32.9
+//
+// The adaptive stop runs few inner iterations where the tolerance is loose (400 outer
+// iterations of at most 10; of them all but the first end after one): 4096 x 4096 1e-3 130 /
+// 161, 1e-4 173 / 194, 3e-5 220 / 231, 1e-5 277 / 276, 1e-6 345 / 331; with a mask 1e-4
+// 210 / 216, 3e-5 293 / 283; 2048 x 2048 1e-3 37 / 36, 1e-4 48 / 46.
+bool use_mt4(const Grid& g, int variant, int K, double inner_tol2, bool masked) {
   TilePlan p;
-  if (!(adaptive ? adapt_in_tile(g, variant, K) : variant <= 1 || !exact128) || !tile_plan(g, &p)) return false;
-  return (long long)g.NR * g.NC * p.cl * p.nw <= 148 * tile_warps(p.nw, p.pad);
+  if (!exact_128(g) || K > 64 || (g.W + g.NC) % 4 != 0 || !tile_plan(g, &p)) return false;
+  if (variant == 1) return inner_tol2 == 0.0;
+  if (variant != 0 || one_wave(g, p)) return false;
+  // u, f, p1 and p2, read by every launch (67 MB at 2048 x 2048, 105 MB at 2560 x 2560)
+  const bool beyond_l2 = 16ll * g.H * g.W > 96ll << 20;
+  if (inner_tol2 > 0.0) return beyond_l2 && inner_tol2 >= 2e-5 * 2e-5;
+  return K < (beyond_l2 ? (masked ? 3 : 5) : (masked ? 0 : 3));
+}
+
+// The adaptive stop in one of the micro-tile kernels: the default of exact 128 x 128
+// subdomains.  (W + N_c a multiple of 4 and K <= 64 are no needs of fused_tile.cuh, but its
+// residual sums are float32 where those of the cluster-barrier kernel are float64, so a near
+// tie could stop a subdomain one iteration apart: every problem keeps the sums it has always
+// had.)
+bool adapt_in_tile(const Grid& g, int variant, int K) {
+  return exact_128(g) && variant == 0 && K <= 64 && (g.W + g.NC) % 4 == 0;
+}
+
+}  // namespace
+
+// In the micro-tile kernel and where one wave holds the launch.  The update then saves a
+// launch on the chain of latencies: 128 x 128 in 64 x 64 11.4 -> 10.9 us per outer iteration,
+// 512 x 512 in 128 x 128 12.7 -> 11.9, 1024 x 1024 18.6 -> 18.1.  With several waves the update of
+// the sides costs more instructions than its own launch, which overlaps with the loads: 4096
+// x 4096 216 -> 224.
+bool fused_chains(const Grid& g, int variant, int K, double inner_tol2) {
+  TilePlan p;
+  if (!tile_plan(g, &p) || !one_wave(g, p)) return false;
+  return inner_tol2 > 0.0 ? adapt_in_tile(g, variant, K) : variant == 0 || !exact_128(g);
 }
 
 // Every handle prepares the kernels it can reach and no others: an attribute call per
 // kernel instance is most of what creating a small handle costs.
-cudaError_t fused_prepare(const Grid& g, int variant, bool adaptive) {
+cudaError_t fused_prepare(const Grid& g, int variant, int K, double inner_tol2) {
   TilePlan p;
   if (!tile_plan(g, &p)) return cudaErrorInvalidValue;
-  const bool exact128 = g.H == 128 * g.NR && g.W == 128 * g.NC;
-  const bool chain = fused_chains(g, variant, 1, adaptive);  // (whatever the inner count)
+  const bool exact128 = exact_128(g), chain = fused_chains(g, variant, K, inner_tol2);
+  const bool adaptive = inner_tol2 > 0.0;
   cudaError_t e = cudaSuccess;
+  // (whatever a later load brings: without a mask the persistent kernel is taken wherever it
+  // is with one)
+  if (use_mt4(g, variant, K, inner_tol2, false) && (e = fused_mt4_prepare(adaptive)) != cudaSuccess) return e;
   if (adaptive) {
     if (exact128 && variant == 0 && (e = prepare_tile_adapt_128(chain)) != cudaSuccess) return e;
     switch (pick((g.H + g.NR - 1) / g.NR, (g.W + g.NC - 1) / g.NC)) {
@@ -493,14 +537,19 @@ cudaError_t launch_fused_batch(const BatchArgs& B, int total_tiles, int tile, in
   return tile == 64 ? launch_tile_batch_64(B, total_tiles, overlap, st) : cudaErrorInvalidValue;
 }
 
-bool fused_out_of_place(const Grid& g, int variant) {
-  return variant <= 1 || !(g.H == 128 * g.NR && g.W == 128 * g.NC);  // the micro-tile kernel
+bool fused_out_of_place(const Grid& g, int variant) {  // in the micro-tile kernel
+  return variant <= 1 || !exact_128(g);
 }
 
 cudaError_t launch_fused_local(const LocalArgs& a, int fid, int variant, cudaStream_t st) {
   // largest tile of the (ragged) partition
   const int mr = (a.g.H + a.g.NR - 1) / a.g.NR, mc = (a.g.W + a.g.NC - 1) / a.g.NC;
-  const bool exact128 = a.g.H == 128 * a.g.NR && a.g.W == 128 * a.g.NC;  // every tile exactly 128 x 128
+  const bool exact128 = exact_128(a.g);  // every tile exactly 128 x 128
+  // (only the micro-tile kernel works out of place)
+  if (a.u0 == a.u && use_mt4(a.g, variant, a.K, a.inner_tol2, a.mask != nullptr) && fused_mt4_supported(a)) {
+    const cudaError_t e = launch_fused_mt4(a, fid, st);
+    if (e != cudaErrorNotSupported) return e;
+  }
   if (a.inner_tol2 > 0.0) {
     if (adapt_in_tile(a.g, variant, a.K)) return launch_tile_adapt_128(a, fid, st);
     switch (pick(mr, mc)) {

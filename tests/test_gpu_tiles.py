@@ -67,3 +67,15 @@ def test_loads_share_the_captured_loop(cuda_lib, path):
                 torch.cuda.synchronize()
             for k in a:
                 assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("n,K,fid,mask", [
+    (1280, 1, "l2", False), (1280, 2, "seg", False), (1280, 2, "l1", True),      # state in L2
+    (2560, 1, "l1", True), (2560, 3, "l2", True), (2560, 4, "l2", False), (2560, 5, "seg", False)])
+def test_launches_of_several_waves_equal_plain_path(cuda_lib, n, K, fid, mask):
+    """128 x 128 subdomains on both sides of the lines between the persistent and the
+    micro-tile kernel."""
+    from paper_1901_00682_gb300 import _lib as L
+    a, b = (_state(L, n, n, n // 128, n // 128, fid, mask, K, 3, path) for path in ("fused", "plain"))
+    for k in a:
+        assert torch.equal(a[k], b[k]), k
