@@ -1,7 +1,7 @@
 // Fused local solver with cluster barriers: the adaptive inner stop of every subdomain
 // shape but exact 128 x 128, and variant 3 of those; and the choice among the fused
 // kernels (launch_fused_local).  A fixed inner count runs the micro-tile kernel of
-// fused_tile.cuh.
+// fused_tile.cuh or, where use_mt4() says so, the persistent one of kernels_fused_mt4.cu.
 //
 // All inner iterations of one outer iteration of Algorithm 1 for every subdomain in one
 // launch (Section 5, local problem eq. local, solved by the
