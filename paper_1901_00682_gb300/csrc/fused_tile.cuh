@@ -437,31 +437,23 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
         }
       }
     };
-    if (CHAIN) {  // the data before the previous launch has ended, the state after
-      if (whole) {
+    // the data, which no launch of the loop writes, before the previous launch has ended; the state
+    // and the multipliers after.  (Branches around all rows, so that the loads of a row do not wait
+    // for another's.)
+    if (whole) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) data(r);
-      } else {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) data(r);
-      }
-      pdl_wait();
-      if (whole) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) state(r);
-      } else {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) state(r);
-      }
+      for (int r = 0; r < 4; ++r) data(r);
     } else {
-      // (one branch around all rows, so that the loads of a row do not wait for another's)
-      if (whole) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) state(r), data(r);
-      } else {
+      for (int r = 0; r < 4; ++r) data(r);
+    }
+    pdl_wait();
+    if (whole) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) state(r), data(r);
-      }
+      for (int r = 0; r < 4; ++r) state(r);
+    } else {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) state(r);
     }
     // pbar1 of the row below the band: the next CTA's first row (its halo of later
     // iterations), the bottom side of a subdomain that fills the block, or 0
@@ -473,7 +465,6 @@ __device__ __forceinline__ void tile_solve(const LocalArgs& A, const Strips out,
     for (int c = 0; c < 4; ++c) qb[c] = c < nb ? A.P10[(size_t)(r0 + ib + a) * g.W + c0 + j0 + c] : 0.f;
     if (right_lane) pr_s = A.P20[(size_t)(r0 + rank * BAND + rr) * W2 + c0 + BW + b];
 
-    if (!CHAIN) pdl_wait();  // the multiplier update
     // the multipliers of the sides this lane holds
     const bool top = i0 == 0 && s_top, left = j0 == 0 && s_lft, bot = pad_r && s_bot, rgt = pad_c && s_rgt;
     const bool low = bot || bottom_fill;

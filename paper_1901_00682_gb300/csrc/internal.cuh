@@ -128,9 +128,10 @@ struct AdjArgs {
 // writes are visible (at once in a kernel launched without the attribute).
 //
 // The outer iteration is a chain of short kernels: multiplier update, local solves, update,
-// ...  The update waits before its first access and triggers after that wait, so a
-// local solve that starts early knows the previous local solve complete: it loads its
-// state at once and waits only before it reads the multipliers and before it ends.
+// ...  Every one of them waits before its first access to what another of them writes; ahead
+// of the wait it sets itself up and loads the data (f, the mask, the coefficients), which none
+// of them writes.  The wait is also what makes the results of the kernels before the
+// predecessor visible: that they have completed is not enough.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
