@@ -534,19 +534,17 @@ int load_common(dd_tv* h, const float* f, const uint8_t* mask, cudaMemcpyKind ki
   if (!h) return DD_TV_EINVAL;
   if (!f) return fail(h, DD_TV_EINVAL, "f is NULL");
   if (mask && h->fid == DD_TV_SEG) return fail(h, DD_TV_EINVAL, "an inpainting mask is not defined for DD_TV_SEG");
+  if (mask && !h->mask) {  // first: without room for it the handle stays as it was
+    int rc = dalloc(h, &h->mask, h->npx);
+    if (rc) return rc;
+  }
   CK(cudaMemcpyAsync(h->f, f, h->npx * sizeof(float), kind, h->stream));
+  if (mask) CK(cudaMemcpyAsync(h->mask, mask, h->npx, kind, h->stream));
   // the graphs of the outer loop hold the handle's own arrays and read the coefficients from
   // device memory; only a mask coming or going changes their kernels (capturing them again
   // for every load took 130 us of a 0.55 ms solve of 512 x 512 in 32 x 32 subdomains)
   if (h->has_mask != (mask != nullptr)) drop_graphs(h);
   h->has_mask = mask != nullptr;
-  if (mask) {
-    if (!h->mask) {
-      int rc = dalloc(h, &h->mask, h->npx);
-      if (rc) return rc;
-    }
-    CK(cudaMemcpyAsync(h->mask, mask, h->npx, kind, h->stream));
-  }
   ++h->gen;
   return reset_state(h);
 }

@@ -1,0 +1,88 @@
+"""The host side of the solver on a CUDA runtime of host memory (fake_cuda.cpp): which kernels
+a call launches on which arrays, also after an allocation that fails and in graphs."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1901_00682_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_1901_00682_gb300 import _lib, build
+    nvcc = subprocess.run(["which", build._nvcc()], capture_output=True, text=True).stdout.strip()
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    so = str(tmp_path_factory.mktemp("host") / "libhost.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", include, "-x", "c++",
+                    os.path.join(HERE, "fake_cuda.cpp"), os.path.join(CSRC, "dd_tv.cu"), "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    for name, (res, args) in _lib.SIGNATURES.items():
+        if hasattr(lib, name):
+            getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
+    lib.fake_log.restype = ctypes.c_char_p
+    lib.fake_fail_allocations.argtypes = [ctypes.c_size_t]
+    return lib
+
+
+@pytest.fixture
+def lib(fake):
+    yield fake
+    fake.fake_fail_allocations(0)
+    fake.fake_fail_prepare(0)
+
+
+class Handle:
+    def __init__(self, lib, *args, **kw):
+        from paper_1901_00682_gb300 import _lib
+        self.lib, self.h = lib, ctypes.c_void_p()
+        d = _lib.Params()
+        lib.dd_tv_default_params(ctypes.byref(d))
+        for k, v in dict(alpha=10.0, **kw).items():
+            setattr(d, k, v)
+        d.height, d.width, d.sub_rows, d.sub_cols = args
+        self.shape = args[:2]
+        self.rc = lib.dd_tv_create(ctypes.byref(self.h), ctypes.byref(d))
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        self.lib.dd_tv_destroy(self.h)
+
+    def load(self, f, mask=None):
+        return self.lib.dd_tv_load(self.h, f.ctypes.data, None if mask is None else mask.ctypes.data)
+
+    def launches(self, n_outer):
+        """The launches of n_outer outer iterations."""
+        self.lib.fake_clear_log()
+        assert self.lib.dd_tv_iterate(self.h, n_outer) == 0
+        return self.lib.fake_log().decode().split("\n")[:-1]
+
+    def u(self):
+        out = np.empty(self.shape, np.float32)
+        assert self.lib.dd_tv_get_u(self.h, out.ctypes.data) == 0
+        return out
+
+
+@pytest.mark.parametrize("path,kernels", [(0, {"interface", "local"}), (2, {"full"})])
+def test_load_that_fails_leaves_the_handle_as_it_was(lib, path, kernels):
+    """The first masked load finds no memory for the mask: the captured loop of the unmasked
+    problem goes on, and a later masked load does not replay it."""
+    H, W = 96, 64
+    f, g, m = np.zeros((H, W), np.float32), np.ones((H, W), np.float32), np.ones((H, W), np.uint8)
+    with Handle(lib, H, W, 2, 1, path=path) as s:
+        assert s.load(f) == 0
+        lib.fake_fail_allocations(m.nbytes)
+        assert s.load(g, m) == 2   # ENOMEM
+        lib.fake_fail_allocations(0)
+        assert s.u()[-1, -1] == 0
+        assert set(s.launches(8)) == kernels
+        assert s.load(g, m) == 0
+        masked = [k for k in s.launches(8) if k != "interface"]
+        assert masked and all(k.endswith(" masked") for k in masked)
+        assert s.load(f) == 0
+        assert set(s.launches(8)) == kernels
