@@ -87,8 +87,9 @@ struct dd_tv {
   // plain path: phat and pbar; full-dimension path: pbar (carried across iterations)
   float *Ph1 = nullptr, *Ph2 = nullptr, *Pb1 = nullptr, *Pb2 = nullptr;
   // full-dimension path: the two sets its launches go back and forth between (u, P1, ...
-  // above point into the one that holds the current iterate); full_mem is set 1
+  // above point into full[full_cur], which holds the current iterate); full_mem is set 1
   FullSet full[2] = {};
+  int full_cur = 0;
   float* full_mem = nullptr;
   double* partials = nullptr;
   unsigned int* counter = nullptr;
@@ -98,7 +99,8 @@ struct dd_tv {
   int* inner_max = nullptr;              // 1
   unsigned long long* inner_work = nullptr;  // 1
 
-  cudaGraphExec_t chunk[2] = {nullptr, nullptr};  // kGraphChunk outer iterations from parity 0 / 1
+  // kGraphChunk outer iterations from parity 0 / 1 (full-dimension path: from set 0 / 1)
+  cudaGraphExec_t chunk[2] = {nullptr, nullptr};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 
   // measurement hooks: event pairs bracketing each phase while profiling is on
@@ -276,16 +278,23 @@ struct PhaseMark {
 // Full-dimension path: launches of one outer iteration (of inner_iters iterations).
 int full_launches(const dd_tv* h) { return (h->p.inner_iters + full_max_steps() - 1) / full_max_steps(); }
 
-// Points the handle's state at the set that holds iterate h->n (set 0 at n = 0, the other
-// one after every launch).
-void full_select(dd_tv* h) {
-  if (!h->full_mem) return;
-  const FullSet& s = h->full[h->n & full_launches(h) & 1];
+// Points the handle's state at one of the two sets.
+void full_select(dd_tv* h, int set) {
+  const FullSet& s = h->full[set];
+  h->full_cur = set;
   h->u = s.u;
   h->P1 = s.P1;
   h->P2 = s.P2;
   h->Pb1 = s.Pb1;
   h->Pb2 = s.Pb2;
+}
+
+// Whether the caller is capturing the handle's stream into a graph of its own.
+bool capturing(const dd_tv* h) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
 }
 
 // The chained local solve's arrays: iterate n of parity par in, n + 1 out.
@@ -315,22 +324,23 @@ cudaError_t chain_rebuild(dd_tv* h) {
 
 // One outer iteration starting from parity `par` (= n mod 2): the strips of p~^n are
 // in set par, those of p~^{n-1} in set 1 - par, and p~^{n+1}'s go to set 1 - par.
-cudaError_t outer_once(dd_tv* h, int par) {
+// in_place: full-dimension path, leave the iterate in the set of arrays that holds it.
+cudaError_t outer_once(dd_tv* h, int par, bool in_place = false) {
   cudaError_t e;
   const cudaStream_t st = h->stream;
-  if (h->p.path == DD_TV_PATH_FULLDIM && h->full_mem) {
+  if (h->p.path == DD_TV_PATH_FULLDIM && h->full_mem && !in_place) {
     const int L = full_launches(h), K = h->p.inner_iters;
     PhaseMark m(h, 1, L);
-    int cur = par & L & 1;
-    for (int q = 0; q < L; ++q, cur ^= 1) {
-      const int n = (int)((long long)(q + 1) * K / L - (long long)q * K / L);
+    for (int q = 0; q < L; ++q) {
+      const int n = (int)((long long)(q + 1) * K / L - (long long)q * K / L), cur = h->full_cur;
       const FullArgs a{h->g.H, h->g.W, (float)h->p.c1, (float)h->p.c2, h->f, h->has_mask ? h->mask : nullptr,
                        h->coef, h->flag, h->full[cur], h->full[1 - cur]};
       if ((e = launch_full(a, h->fid, n, st)) != cudaSuccess) return e;
+      full_select(h, 1 - cur);
     }
     return cudaSuccess;
   }
-  if (h->p.path == DD_TV_PATH_FULLDIM) {  // no room for the second set: a launch per half-step, in place
+  if (h->p.path == DD_TV_PATH_FULLDIM) {  // a launch per half-step (also without room for the second set)
     LocalArgs a = local_args(h, 0);
     PhaseMark m(h, 1, 2 * a.K);
     for (int k = 0; k < a.K; ++k) {
@@ -379,44 +389,53 @@ void drop_graphs(dd_tv* h) {
     }
 }
 
-int capture_chunk(dd_tv* h, int par) {
+// Captures chunk[c], of kGraphChunk outer iterations from parity par (an even number of
+// launches: it leaves the full-dimension iterate in the set it found it in).
+int capture_chunk(dd_tv* h, int c, int par) {
   cudaGraph_t graph = nullptr;
   CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+  const int set = h->full_cur;
   cudaError_t e = cudaSuccess;
   for (int q = 0; q < kGraphChunk && e == cudaSuccess; ++q) e = outer_once(h, (par + q) & 1);
   cudaError_t e2 = cudaStreamEndCapture(h->stream, &graph);
+  if (h->full_mem) full_select(h, set);
   if (e != cudaSuccess || e2 != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
     return fail(h, DD_TV_ECUDA, "graph capture failed: %s",
                 cudaGetErrorString(e != cudaSuccess ? e : e2));
   }
-  e = cudaGraphInstantiate(&h->chunk[par], graph, 0);
+  e = cudaGraphInstantiate(&h->chunk[c], graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
-    h->chunk[par] = nullptr;
+    h->chunk[c] = nullptr;
     return fail(h, DD_TV_ECUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
   }
   return DD_TV_OK;
 }
 
 int run_outer(dd_tv* h, int count) {
+  // a caller's graph finds the full-dimension iterate where it left it, at every replay: if its
+  // launches went to the other set of arrays an odd number of times, the last iteration is run in
+  // place
+  const int set = h->full_cur;
+  const bool keep_set = h->full_mem && full_launches(h) % 2 && capturing(h);
   int done = 0;
   while (done < count) {
     const int par = h->n & 1;
     if (count - done >= kGraphChunk && !h->prof) {
-      if (!h->chunk[par]) {
-        int rc = capture_chunk(h, par);
+      const int c = h->full_mem ? h->full_cur : par;
+      if (!h->chunk[c]) {
+        int rc = capture_chunk(h, c, par);
         if (rc) return rc;
       }
-      CK(cudaGraphLaunch(h->chunk[par], h->stream));
+      CK(cudaGraphLaunch(h->chunk[c], h->stream));
       h->n += kGraphChunk;
       done += kGraphChunk;
     } else {
-      CK(outer_once(h, par));
+      CK(outer_once(h, par, keep_set && done + 1 == count && h->full_cur == set));
       h->n += 1;
       done += 1;
     }
-    full_select(h);
   }
   return DD_TV_OK;
 }
@@ -424,7 +443,6 @@ int run_outer(dd_tv* h, int count) {
 int reset_state(dd_tv* h) {
   const cudaStream_t st = h->stream;
   h->n = 0;
-  full_select(h);
   CK(launch_init_u(h->g, h->fid, h->f, h->has_mask ? h->mask : nullptr, h->u, st));
   CK(cudaMemsetAsync(h->P1, 0, h->n1 * sizeof(float), st));
   CK(cudaMemsetAsync(h->P2, 0, h->n2 * sizeof(float), st));
@@ -1086,8 +1104,7 @@ int dd_tv_destroy(dd_tv* h) {
   adj_free(h->adj);
   h->adj = nullptr;
   if (h->full_mem) {  // u, P1, ... back to the arrays allocated one by one
-    h->n = 0;
-    full_select(h);
+    full_select(h, 0);
     cudaFree(h->full_mem);
   }
   for (auto& m : h->marks) {
@@ -1217,7 +1234,6 @@ int dd_tv_set_state(dd_tv* h, const float* u, const float* P1, const float* P2, 
   const cudaStream_t st = h->stream;
   const auto D2D = cudaMemcpyDeviceToDevice;
   h->n = outer_count;
-  full_select(h);
   CK(cudaMemcpyAsync(h->u, u, h->npx * sizeof(float), D2D, st));
   CK(cudaMemcpyAsync(h->P1, P1, h->n1 * sizeof(float), D2D, st));
   CK(cudaMemcpyAsync(h->P2, P2, h->n2 * sizeof(float), D2D, st));

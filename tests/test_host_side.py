@@ -86,3 +86,29 @@ def test_load_that_fails_leaves_the_handle_as_it_was(lib, path, kernels):
         assert masked and all(k.endswith(" masked") for k in masked)
         assert s.load(f) == 0
         assert set(s.launches(8)) == kernels
+
+
+@pytest.mark.parametrize("K", [1, 7, 10, 15])
+@pytest.mark.parametrize("n_outer", [1, 2, 3])
+@pytest.mark.parametrize("before", [0, 1, 5])
+def test_full_dimension_iterations_replay_from_a_callers_graph(lib, K, n_outer, before):
+    """Outer iterations captured into a caller's graph advance the iterate at every replay,
+    whichever set of arrays held it, and the handle goes on from there."""
+    H, W = 70, 60
+    f = np.zeros((H, W), np.float32)
+    with Handle(lib, H, W, 1, 1, path=2, inner_iters=K) as s:
+        assert s.load(f) == 0
+        s.launches(before)
+        graph, run, out = ctypes.c_void_p(), ctypes.c_void_p(), np.empty_like(f)
+        assert lib.cudaStreamBeginCapture(None, 0) == 0
+        assert lib.dd_tv_iterate(s.h, n_outer) == 0
+        assert lib.dd_tv_get_u(s.h, ctypes.c_void_p(out.ctypes.data)) == 0
+        assert lib.cudaStreamEndCapture(None, ctypes.byref(graph)) == 0
+        assert lib.cudaGraphInstantiate(ctypes.byref(run), graph, ctypes.c_ulonglong(0)) == 0
+        lib.cudaGraphDestroy(graph)
+        for r in (1, 2, 3):
+            assert lib.cudaGraphLaunch(run, None) == 0
+            assert out[0, 0] == K * (before + r * n_outer)
+        lib.cudaGraphExecDestroy(run)
+        s.launches(6)
+        assert s.u()[0, 0] == K * (before + 3 * n_outer + 6)
