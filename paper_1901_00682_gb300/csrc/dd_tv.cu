@@ -1009,6 +1009,7 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
   }
   if (p->path != DD_TV_PATH_FUSED) {
     if ((rc = dalloc(h, &h->Pb1, h->n1)) || (rc = dalloc(h, &h->Pb2, h->n2))) {
+      std::snprintf(g_create_err, sizeof(g_create_err), "%s", h->err);
       dd_tv_destroy(h);
       return rc;
     }
@@ -1018,12 +1019,21 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
     // runs a launch per half-step in place
     auto up = [](size_t n) { return (n + 63) & ~(size_t)63; };
     const size_t n = up(h->npx) + 2 * up(h->n1) + 2 * up(h->n2);
-    if (cudaMalloc((void**)&h->full_mem, n * sizeof(float)) != cudaSuccess ||
-        cudaMemset(h->full_mem, 0, n * sizeof(float)) != cudaSuccess || full_prepare() != cudaSuccess) {
+    const cudaError_t room = cudaMalloc((void**)&h->full_mem, n * sizeof(float));
+    if (room == cudaErrorMemoryAllocation) {
       cudaGetLastError();
-      if (h->full_mem) cudaFree(h->full_mem);
       h->full_mem = nullptr;
     } else {
+      cudaError_t e = room;
+      if (e == cudaSuccess) e = cudaMemset(h->full_mem, 0, n * sizeof(float));
+      if (e == cudaSuccess) e = full_prepare();
+      if (e != cudaSuccess) {
+        std::snprintf(g_create_err, sizeof(g_create_err), "full-dimension kernel set-up: %s", cudaGetErrorString(e));
+        if (room == cudaSuccess) cudaFree(h->full_mem);
+        h->full_mem = nullptr;
+        dd_tv_destroy(h);
+        return DD_TV_ECUDA;
+      }
       float* m = h->full_mem;
       h->full[0] = FullSet{h->u, h->P1, h->P2, h->Pb1, h->Pb2};
       h->full[1].u = m;
@@ -1035,6 +1045,7 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
   }
   if (p->path == DD_TV_PATH_PLAIN) {
     if ((rc = dalloc(h, &h->Ph1, h->n1)) || (rc = dalloc(h, &h->Ph2, h->n2))) {
+      std::snprintf(g_create_err, sizeof(g_create_err), "%s", h->err);
       dd_tv_destroy(h);
       return rc;
     }

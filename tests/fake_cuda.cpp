@@ -20,6 +20,7 @@ using Work = std::vector<std::function<void()>>;
 Work* g_capture = nullptr;   // the capture under way
 std::string g_log;
 size_t g_fail_bytes = 0;     // an allocation of at least this size fails (0: none does)
+int g_fail_at = 0;           // the allocation that fails, counted from here (0: none does)
 cudaError_t g_prepare_error = cudaSuccess;
 
 cudaError_t enqueue(std::function<void()> f) {
@@ -44,10 +45,11 @@ extern "C" {
 const char* fake_log() { return g_log.c_str(); }
 void fake_clear_log() { g_log.clear(); }
 void fake_fail_allocations(size_t at_least_bytes) { g_fail_bytes = at_least_bytes; }
+void fake_fail_allocation(int k) { g_fail_at = k; }
 void fake_fail_prepare(int error) { g_prepare_error = (cudaError_t)error; }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
-  if (g_fail_bytes && n >= g_fail_bytes) return cudaErrorMemoryAllocation;
+  if ((g_fail_bytes && n >= g_fail_bytes) || (g_fail_at && --g_fail_at == 0)) return cudaErrorMemoryAllocation;
   *p = std::calloc(n, 1);
   return cudaSuccess;
 }

@@ -32,6 +32,7 @@ def fake(tmp_path_factory):
 def lib(fake):
     yield fake
     fake.fake_fail_allocations(0)
+    fake.fake_fail_allocation(0)
     fake.fake_fail_prepare(0)
 
 
@@ -112,3 +113,45 @@ def test_full_dimension_iterations_replay_from_a_callers_graph(lib, K, n_outer, 
         lib.cudaGraphExecDestroy(run)
         s.launches(6)
         assert s.u()[0, 0] == K * (before + 3 * n_outer + 6)
+
+
+HALF_STEPS = ["ustep", "pstep"]
+
+
+def test_full_dimension_without_room_for_the_second_set(lib):
+    """Only then the path runs a launch per half-step in place; state and results as otherwise."""
+    H, W, K = 70, 60, 3
+    f = np.zeros((H, W), np.float32)
+    lib.fake_fail_allocations(2 * 4 * H * W)   # more than any single array
+    with Handle(lib, H, W, 1, 1, path=2, inner_iters=K) as s:
+        assert s.rc == 0
+        lib.fake_fail_allocations(0)
+        assert s.load(f) == 0
+        assert s.launches(1) == HALF_STEPS * K
+        assert s.launches(6) == HALF_STEPS * (6 * K)
+        assert s.u()[0, 0] == 7 * K
+    with Handle(lib, H, W, 1, 1, path=2, inner_iters=K) as s:
+        assert s.load(f) == 0
+        assert s.launches(7) == ["full"] * 7
+
+
+@pytest.mark.parametrize("path", [0, 2])
+def test_create_reports_a_kernel_set_up_that_fails(lib, path):
+    lib.fake_fail_prepare(98)   # cudaErrorInvalidDeviceFunction
+    with Handle(lib, 70, 60, 1, 1, path=path) as s:
+        assert s.rc == 3 and not s.h.value   # ECUDA
+        assert b"set-up" in lib.dd_tv_last_error(None)
+
+
+@pytest.mark.parametrize("path,n", [(0, 9), (1, 16), (2, 12)])
+def test_create_reports_each_allocation_that_fails(lib, path, n):
+    """Every allocation of a new handle in turn finds no memory."""
+    codes = []
+    for k in range(1, 40):
+        lib.fake_fail_allocation(k)
+        with Handle(lib, 70, 60, 2, 2, path=path) as s:
+            codes.append(s.rc)
+            assert (s.rc == 0) == bool(s.h.value)
+            if s.rc:
+                assert b"cudaMalloc" in lib.dd_tv_last_error(None)
+    assert codes.count(2) >= n and set(codes) == {0, 2}
