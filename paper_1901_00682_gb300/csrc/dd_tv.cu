@@ -278,6 +278,15 @@ struct PhaseMark {
 // Full-dimension path: launches of one outer iteration (of inner_iters iterations).
 int full_launches(const dd_tv* h) { return (h->p.inner_iters + full_max_steps() - 1) / full_max_steps(); }
 
+// Whether a launch per half-step beats the blocks of kernels_full.cu: a single iteration per
+// launch, on rows that are not 16-byte aligned (the blocks load and store 11 arrays' worth of
+// scalars for it) and a state that stays in L2 between launches.  us per iteration, half-steps /
+// blocks: 90 x 97 5.2 / 6.2, 300 x 337 5.7 / 6.8, 1001 x 1503 22.5 / 25.9, 2047 x 2049 62 / 64, but 4095 x
+// 4097 287 / 202; two iterations 2047 x 2049 124 / 67; aligned rows 1024 x 1024 17.5 / 14.4.
+bool full_half_steps(const dd_tv* h) {
+  return h->p.inner_iters == 1 && h->g.W % 4 != 0 && h->npx <= (size_t)4 << 20;
+}
+
 // Points the handle's state at one of the two sets.
 void full_select(dd_tv* h, int set) {
   const FullSet& s = h->full[set];
@@ -340,7 +349,7 @@ cudaError_t outer_once(dd_tv* h, int par, bool in_place = false) {
     }
     return cudaSuccess;
   }
-  if (h->p.path == DD_TV_PATH_FULLDIM) {  // a launch per half-step (also without room for the second set)
+  if (h->p.path == DD_TV_PATH_FULLDIM) {  // a launch per half-step
     LocalArgs a = local_args(h, 0);
     PhaseMark m(h, 1, 2 * a.K);
     for (int k = 0; k < a.K; ++k) {
@@ -1014,7 +1023,7 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
       return rc;
     }
   }
-  if (p->path == DD_TV_PATH_FULLDIM) {
+  if (p->path == DD_TV_PATH_FULLDIM && !full_half_steps(h)) {
     // the second set, every array on a 256-byte boundary; without room for it the path
     // runs a launch per half-step in place
     auto up = [](size_t n) { return (n + 63) & ~(size_t)63; };

@@ -16,7 +16,9 @@
 // overlap (128 x 128 pixels computed for 108 x 108, or 104, stored at n = 10), and per launch 24 bytes
 // read and 20 written per pixel of a block.  n is at most 10: twice as many leave less than
 // half of a block to store.  Measured per 10 iterations, before (two launches per iteration)
-// and after: 1001 x 1503 218 -> 43 us, 4096 x 4096 about 2500 -> 306.
+// and after: 1001 x 1503 218 -> 43 us, 4096 x 4096 2474 -> 306, with a mask 2607 -> 350 (394 with
+// a byte load per pixel of the mask); one iteration of 1024 x 1024 17.5 -> 14.4, with a mask 17.5 ->
+// 15.7 (17.9 with byte loads), of unaligned rows dd_tv.cu full_half_steps.
 #include "fused_tile.cuh"
 
 namespace ddtv {
@@ -163,12 +165,22 @@ __global__ void __launch_bounds__(FL::NT, 4) k_full(const FullArgs A, const Axis
       }
       *reinterpret_cast<ulonglong2*>(myF + 4 * NT * c) = make_ulonglong2(FV[c][0], FV[c][1]);
     }
-    if (MASK) {
+    if (MASK) {  // a word per row where the rows are aligned
+      if (vec && i0 + 3 < mr && j0 + 3 < mc) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < 4; ++r) {
+          const uint32_t m = *reinterpret_cast<const uint32_t*>(A.mask + o1 + (size_t)r * W);
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (i0 + r < mr && j0 + c < mc && A.mask[(size_t)(r0 + i0 + r) * W + c0 + j0 + c]) in_d |= 1u << (4 * c + r);
+          for (int c = 0; c < 4; ++c)
+            if ((m >> (8 * c)) & 0xffu) in_d |= 1u << (4 * c + r);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (i0 + r < mr && j0 + c < mc && A.mask[o1 + (size_t)r * W + c]) in_d |= 1u << (4 * c + r);
+      }
     }
     *reinterpret_cast<float4*>(sQ1 + w * BW + j0) = make_float4(lo2(Q1[0][0]), lo2(Q1[1][0]), lo2(Q1[2][0]), lo2(Q1[3][0]));
     *reinterpret_cast<ulonglong2*>(myQL) = make_ulonglong2(Q2[0][0], Q2[0][1]);

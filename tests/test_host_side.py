@@ -155,3 +155,12 @@ def test_create_reports_each_allocation_that_fails(lib, path, n):
             if s.rc:
                 assert b"cudaMalloc" in lib.dd_tv_last_error(None)
     assert codes.count(2) >= n and set(codes) == {0, 2}
+
+
+@pytest.mark.parametrize("H,W,K,half_steps", [(70, 61, 1, True), (70, 60, 1, False), (70, 61, 2, False),
+                                              (2047, 2049, 1, True), (2049, 2049, 1, False)])
+def test_single_full_dimension_iterations_of_unaligned_rows_run_half_steps(lib, H, W, K, half_steps):
+    f = np.zeros((H, W), np.float32)
+    with Handle(lib, H, W, 1, 1, path=2, inner_iters=K) as s:
+        assert s.load(f) == 0
+        assert s.launches(5) == (HALF_STEPS if half_steps else ["full"]) * 5
