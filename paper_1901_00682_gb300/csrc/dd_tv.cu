@@ -74,9 +74,9 @@ struct dd_tv {
   Strips strips_k[2] = {};
   // the local solves make the multiplier update (LocalArgs.chain): lamh, lamv are the copies of
   // the upper / left sides, lam2 ([h | v]) those of the lower / right ones, x the extrapolated
-  // strips by parity
+  // strips by parity (both behind the strip sets in strip_mem)
   bool chain = false;
-  float *lam2 = nullptr, *x_mem = nullptr;
+  float* lam2 = nullptr;
   Strips x[2] = {};
   // row-block shard (dd_tv_create_shard): global tile rows [tile_row0, tile_row0 + g.NR)
   // of a problem with nr_global tile rows; its first pixel row is row0 of the image
@@ -320,15 +320,10 @@ void chain_args(dd_tv* h, int par, LocalArgs* a) {
 
 // After lamh, lamv and both strip sets of iterate h->n were set: the arrays that follow from them.
 cudaError_t chain_rebuild(dd_tv* h) {
-  if (!h->chain) return cudaSuccess;
-  const auto D2D = cudaMemcpyDeviceToDevice;
+  if (!h->chain || h->nh + h->nv == 0) return cudaSuccess;
   const int par = h->n & 1;
-  cudaError_t e;
-  if (h->nh && (e = cudaMemcpyAsync(h->lam2, h->lamh, h->nh * sizeof(float), D2D, h->stream)) != cudaSuccess) return e;
-  if (h->nv && (e = cudaMemcpyAsync(h->lam2 + h->nh, h->lamv, h->nv * sizeof(float), D2D, h->stream)) != cudaSuccess)
-    return e;
-  return launch_extrapolate(2 * (long long)(h->nh + h->nv), h->strips[par].SB, h->strips[1 - par].SB, h->x[par].SB,
-                            h->stream);
+  return launch_chain_rebuild((int)h->nh, (int)h->nv, h->strips[par].SB, h->strips[1 - par].SB, h->x[par].SB, h->lamh,
+                              h->lamv, h->lam2, h->stream);
 }
 
 // One outer iteration starting from parity `par` (= n mod 2): the strips of p~^n are
@@ -457,8 +452,7 @@ int reset_state(dd_tv* h) {
   CK(cudaMemsetAsync(h->P2, 0, h->n2 * sizeof(float), st));
   if (h->nh) CK(cudaMemsetAsync(h->lamh, 0, h->nh * sizeof(float), st));
   if (h->nv) CK(cudaMemsetAsync(h->lamv, 0, h->nv * sizeof(float), st));
-  if (h->strip_mem) CK(cudaMemsetAsync(h->strip_mem, 0, 4 * (h->nh + h->nv) * sizeof(float), st));
-  if (h->x_mem) CK(cudaMemsetAsync(h->x_mem, 0, 5 * (h->nh + h->nv) * sizeof(float), st));  // x and lam2
+  if (h->strip_mem) CK(cudaMemsetAsync(h->strip_mem, 0, (h->chain ? 9 : 4) * (h->nh + h->nv) * sizeof(float), st));
   if (h->Pb1) {
     CK(cudaMemsetAsync(h->Pb1, 0, h->n1 * sizeof(float), st));
     CK(cudaMemsetAsync(h->Pb2, 0, h->n2 * sizeof(float), st));
@@ -1003,11 +997,12 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
   h->nlh = (size_t)(g.NR - 1) + g.cut_top + g.cut_bot;
   h->nh = h->nlh * g.W;
   h->nv = (size_t)(g.NC - 1) * g.H;
+  h->chain = p->path == DD_TV_PATH_FUSED && !h->shard && fused_chains(g, p->variant, p->inner_iters, p->inner_tol * p->inner_tol);
   std::vector<Coef> sched;
   build_schedule(*p, sched);
   if ((rc = dalloc(h, &h->f, h->npx)) || (rc = dalloc(h, &h->u, h->npx)) || (rc = dalloc(h, &h->P1, h->n1)) ||
       (rc = dalloc(h, &h->P2, h->n2)) || (rc = dalloc(h, &h->lamh, h->nh)) || (rc = dalloc(h, &h->lamv, h->nv)) ||
-      (rc = dalloc(h, &h->strip_mem, 4 * (h->nh + h->nv))) || (rc = dalloc(h, &h->coef, sched.size())) ||
+      (rc = dalloc(h, &h->strip_mem, (h->chain ? 9 : 4) * (h->nh + h->nv))) || (rc = dalloc(h, &h->coef, sched.size())) ||
       (rc = dalloc(h, &h->partials, (size_t)std::max(reduce_partials_count(), sum_f64_partials_count()))) ||
       (rc = dalloc(h, &h->counter, 1)) || (rc = dalloc(h, &h->red_out, 2)) || (rc = dalloc(h, &h->flag, 1)) ||
       (rc = dalloc(h, &h->inner_used, (size_t)h->g.NR * h->g.NC)) || (rc = dalloc(h, &h->inner_max, 1)) ||
@@ -1074,19 +1069,12 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
       h->strips_k[s].ST += skip;
     }
   }
-  h->chain = p->path == DD_TV_PATH_FUSED && !h->shard && fused_chains(g, p->variant, p->inner_iters, p->inner_tol * p->inner_tol);
-  if (h->chain && h->nh + h->nv) {
-    const size_t ne = h->nh + h->nv;
-    if ((rc = dalloc(h, &h->x_mem, 5 * ne))) {
-      std::snprintf(g_create_err, sizeof(g_create_err), "%s", h->err);
-      dd_tv_destroy(h);
-      return rc;
-    }
+  if (h->chain && h->strip_mem) {  // behind the strip sets: x likewise, then lam2
     for (int s = 0; s < 2; ++s) {
-      float* base = h->x_mem + (size_t)s * 2 * ne;
+      float* base = h->strip_mem + (size_t)(s + 2) * 2 * (h->nh + h->nv);
       h->x[s] = Strips{base, base + h->nh, base + 2 * h->nh, base + 2 * h->nh + h->nv};
     }
-    h->lam2 = h->x_mem + 4 * ne;
+    h->lam2 = h->strip_mem + 8 * (h->nh + h->nv);
   }
   h->lamh_k = h->lamh ? h->lamh + (size_t)g.cut_top * g.W : nullptr;
   cudaError_t e;
@@ -1131,7 +1119,7 @@ int dd_tv_destroy(dd_tv* h) {
     cudaEventDestroy(m.a);
     cudaEventDestroy(m.b);
   }
-  void* bufs[] = {h->f, h->u, h->P1, h->P2, h->lamh, h->lamv, h->mask, h->strip_mem, h->x_mem, h->coef, h->Ph1, h->Ph2,
+  void* bufs[] = {h->f, h->u, h->P1, h->P2, h->lamh, h->lamv, h->mask, h->strip_mem, h->coef, h->Ph1, h->Ph2,
                   h->Pb1, h->Pb2, h->partials, h->counter, h->red_out, h->flag, h->inner_used, h->inner_max,
                   h->inner_work};
   for (void* b : bufs)
@@ -1263,8 +1251,7 @@ int dd_tv_set_state(dd_tv* h, const float* u, const float* P1, const float* P2, 
     CK(cudaMemcpyAsync(h->Pb1, P1prev, h->n1 * sizeof(float), D2D, st));
     CK(cudaMemcpyAsync(h->Pb2, P2prev, h->n2 * sizeof(float), D2D, st));
   } else {
-    CK(launch_extract_strips(h->g, P1, P2, h->strips[h->n & 1], st));
-    CK(launch_extract_strips(h->g, P1prev, P2prev, h->strips[1 - (h->n & 1)], st));
+    CK(launch_extract_strips(h->g, P1, P2, h->strips[h->n & 1], P1prev, P2prev, h->strips[1 - (h->n & 1)], st));
     CK(chain_rebuild(h));
   }
   h->loaded = true;

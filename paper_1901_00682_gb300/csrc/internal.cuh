@@ -148,13 +148,15 @@ inline bool has_interfaces(const Grid& g) { return g.NR > 1 || g.NC > 1 || g.cut
 // lambda += sigma ((2 cur_s - prev_s) - (2 cur_t - prev_t)) on every interface edge.
 cudaError_t launch_interface(const Grid& g, float sigma, Strips cur, Strips prev, float* lamh, float* lamv,
                              cudaStream_t st);
-// strips <- interface values of the torn field (P1, P2)
-cudaError_t launch_extract_strips(const Grid& g, const float* P1, const float* P2, Strips s, cudaStream_t st);
+// s <- interface values of the torn field (P1, P2), t <- those of (R1, R2)
+cudaError_t launch_extract_strips(const Grid& g, const float* P1, const float* P2, Strips s, const float* R1,
+                                  const float* R2, Strips t, cudaStream_t st);
 // P1/P2 <- 0 except the interface values, taken from the strips
 cudaError_t launch_scatter_strips(const Grid& g, Strips s, float* P1, float* P2, cudaStream_t st);
 
-// x <- 2 cur - prev over n floats (whole strip sets), the extrapolation of launch_interface
-cudaError_t launch_extrapolate(long long n, const float* cur, const float* prev, float* x, cudaStream_t st);
+// x <- 2 cur - prev (whole strip sets), the extrapolation of launch_interface; lam2 <- [lamh | lamv]
+cudaError_t launch_chain_rebuild(int nh, int nv, const float* cur, const float* prev, float* x, const float* lamh,
+                                 const float* lamv, float* lam2, cudaStream_t st);
 
 cudaError_t launch_interface_batch(const BatchIfaceArgs& a, int total4, cudaStream_t st);
 

@@ -62,14 +62,19 @@ __global__ void k_interface_v1(int nh, int nv, float sigma, const float* __restr
   }
 }
 
-__global__ void k_extrapolate(long long n, const float* __restrict__ cur, const float* __restrict__ prev,
-                              float* __restrict__ x) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
+__global__ void k_chain_rebuild(int nh, int nv, const float* __restrict__ cur, const float* __restrict__ prev,
+                                float* __restrict__ x, const float* __restrict__ lamh, const float* __restrict__ lamv,
+                                float* __restrict__ lam2) {
+  const long long ne = (long long)nh + nv;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < 2 * ne; e += (long long)gridDim.x * blockDim.x) {
     x[e] = fmaf(2.0f, cur[e], -prev[e]);
+    if (e < ne) lam2[e] = e < nh ? lamh[e] : lamv[e - nh];
+  }
 }
 
-// strips <- interface values of (P1, P2): one thread per interface edge
-__global__ void k_extract(Grid g, const float* __restrict__ P1, const float* __restrict__ P2, Strips s) {
+// s <- interface values of (P1, P2), t <- of (R1, R2): one thread per interface edge
+__global__ void k_extract(Grid g, const float* __restrict__ P1, const float* __restrict__ P2, Strips s,
+                          const float* __restrict__ R1, const float* __restrict__ R2, Strips t) {
   const int nh = (g.NR - 1) * g.W, nv = (g.NC - 1) * g.H;
   const int W2 = g.W + g.NC;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nh + nv; e += gridDim.x * blockDim.x) {
@@ -78,11 +83,15 @@ __global__ void k_extract(Grid g, const float* __restrict__ P1, const float* __r
       const int rs = part_start(a + 1, g.H, g.NR) + a;  // bottom side of tile row a
       s.SB[e] = P1[(size_t)rs * g.W + j];
       s.ST[e] = P1[(size_t)(rs + 1) * g.W + j];
+      t.SB[e] = R1[(size_t)rs * g.W + j];
+      t.ST[e] = R1[(size_t)(rs + 1) * g.W + j];
     } else {
       const int q = e - nh, b = q / g.H, i = q % g.H;
       const int cs = part_start(b + 1, g.W, g.NC) + b;  // right side of tile column b
       s.SR[q] = P2[(size_t)i * W2 + cs];
       s.SL[q] = P2[(size_t)i * W2 + cs + 1];
+      t.SR[q] = R2[(size_t)i * W2 + cs];
+      t.SL[q] = R2[(size_t)i * W2 + cs + 1];
     }
   }
 }
@@ -177,9 +186,11 @@ cudaError_t launch_interface(const Grid& g, float sigma, Strips cur, Strips prev
                     prev.ST, lamh, cur.SR, cur.SL, prev.SR, prev.SL, lamv);
 }
 
-cudaError_t launch_extrapolate(long long n, const float* cur, const float* prev, float* x, cudaStream_t st) {
+cudaError_t launch_chain_rebuild(int nh, int nv, const float* cur, const float* prev, float* x, const float* lamh,
+                                 const float* lamv, float* lam2, cudaStream_t st) {
+  const long long n = 2 * ((long long)nh + nv);
   if (n == 0) return cudaSuccess;
-  k_extrapolate<<<grid_for(n, 256), 256, 0, st>>>(n, cur, prev, x);
+  k_chain_rebuild<<<grid_for(n, 256), 256, 0, st>>>(nh, nv, cur, prev, x, lamh, lamv, lam2);
   return cudaGetLastError();
 }
 
@@ -188,10 +199,11 @@ cudaError_t launch_interface_batch(const BatchIfaceArgs& a, int total4, cudaStre
   return launch_pdl(k_interface_batch, grid_for(total4, 256), 256, st, a, total4);
 }
 
-cudaError_t launch_extract_strips(const Grid& g, const float* P1, const float* P2, Strips s, cudaStream_t st) {
+cudaError_t launch_extract_strips(const Grid& g, const float* P1, const float* P2, Strips s, const float* R1,
+                                  const float* R2, Strips t, cudaStream_t st) {
   const int n = (g.NR - 1) * g.W + (g.NC - 1) * g.H;
   if (n == 0) return cudaSuccess;
-  k_extract<<<grid_for(n, 256), 256, 0, st>>>(g, P1, P2, s);
+  k_extract<<<grid_for(n, 256), 256, 0, st>>>(g, P1, P2, s, R1, R2, t);
   return cudaGetLastError();
 }
 

@@ -20,10 +20,13 @@ using Work = std::vector<std::function<void()>>;
 Work* g_capture = nullptr;   // the capture under way
 std::string g_log;
 size_t g_fail_bytes = 0;     // an allocation of at least this size fails (0: none does)
+int g_operations = 0;        // put on the stream (copies, memsets, launches)
+bool g_chain = false;        // the local solves make the multiplier update
 int g_fail_at = 0;           // the allocation that fails, counted from here (0: none does)
 cudaError_t g_prepare_error = cudaSuccess;
 
 cudaError_t enqueue(std::function<void()> f) {
+  ++g_operations;
   if (g_capture) g_capture->push_back(std::move(f));
   else f();
   return cudaSuccess;
@@ -45,6 +48,8 @@ extern "C" {
 const char* fake_log() { return g_log.c_str(); }
 void fake_clear_log() { g_log.clear(); }
 void fake_fail_allocations(size_t at_least_bytes) { g_fail_bytes = at_least_bytes; }
+int fake_operations() { return g_operations; }
+void fake_chain(int on) { g_chain = on; }
 void fake_fail_allocation(int k) { g_fail_at = k; }
 void fake_fail_prepare(int error) { g_prepare_error = (cudaError_t)error; }
 
@@ -131,7 +136,7 @@ cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 namespace ddtv {
 
 // ---- local solves (one launch each), multiplier updates
-bool fused_chains(const Grid&, int, int, double) { return false; }
+bool fused_chains(const Grid&, int, int, double) { return g_chain; }
 cudaError_t fused_prepare(const Grid&, int, int, double) { return g_prepare_error; }
 bool fused_out_of_place(const Grid&, int) { return true; }
 void fused_max_tile(int* r, int* c) { *r = *c = 128; }
@@ -140,12 +145,14 @@ cudaError_t launch_fused_local(const LocalArgs& a, int, int, cudaStream_t) { ret
 cudaError_t launch_interface(const Grid&, float, Strips, Strips, float*, float*, cudaStream_t) {
   return launch("interface");
 }
-cudaError_t launch_extract_strips(const Grid&, const float*, const float*, Strips, cudaStream_t) {
+cudaError_t launch_extract_strips(const Grid&, const float*, const float*, Strips, const float*, const float*, Strips,
+                                  cudaStream_t) {
   return launch("extract");
 }
 cudaError_t launch_scatter_strips(const Grid&, Strips, float*, float*, cudaStream_t) { return launch("scatter"); }
-cudaError_t launch_extrapolate(long long, const float*, const float*, float*, cudaStream_t) {
-  return launch("extrapolate");
+cudaError_t launch_chain_rebuild(int, int, const float*, const float*, float*, const float*, const float*, float*,
+                                 cudaStream_t) {
+  return launch("rebuild");
 }
 cudaError_t launch_init_u(const Grid& g, int, const float* f, const uint8_t*, float* u, cudaStream_t) {
   return launch("init", [=] { std::memcpy(u, f, sizeof(float) * g.H * g.W); });

@@ -34,6 +34,7 @@ def lib(fake):
     fake.fake_fail_allocations(0)
     fake.fake_fail_allocation(0)
     fake.fake_fail_prepare(0)
+    fake.fake_chain(0)
 
 
 class Handle:
@@ -164,3 +165,27 @@ def test_single_full_dimension_iterations_of_unaligned_rows_run_half_steps(lib, 
     with Handle(lib, H, W, 1, 1, path=2, inner_iters=K) as s:
         assert s.load(f) == 0
         assert s.launches(5) == (HALF_STEPS if half_steps else ["full"]) * 5
+
+
+def _operations(lib, call):
+    before = lib.fake_operations()
+    assert call() == 0
+    return lib.fake_operations() - before
+
+
+@pytest.mark.parametrize("sub", [(2, 2), (3, 1), (1, 3), (1, 1)])
+def test_chained_update_costs_loads_and_set_state_nothing(lib, sub):
+    """The arrays that the local solves' own multiplier update needs are set without more copies
+    and launches than a handle without it takes (one for what follows from the strips)."""
+    H, W = 70, 60
+    f, ops = np.ones((H, W), np.float32), []
+    P1, P2 = np.zeros((H + sub[0], W), np.float32), np.zeros((H, W + sub[1]), np.float32)
+    lam = np.zeros(4 * (H + W), np.float32)
+    for chain in (0, 1):
+        lib.fake_chain(chain)
+        with Handle(lib, H, W, *sub) as s:
+            state = [a.ctypes.data for a in (f, P1, P2, lam, lam, P1, P2)]
+            ops.append((_operations(lib, lambda: s.load(f)), _operations(lib, lambda: lib.dd_tv_set_state(s.h, *state, 3))))
+    assert ops[1][0] == ops[0][0]
+    assert ops[1][1] <= ops[0][1] + (sub != (1, 1))
+    assert ops[1][1] <= 3 + (sub[0] > 1) + (sub[1] > 1) + 2
