@@ -17,7 +17,8 @@ def fake(tmp_path_factory):
     nvcc = subprocess.run(["which", build._nvcc()], capture_output=True, text=True).stdout.strip()
     include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     so = str(tmp_path_factory.mktemp("host") / "libhost.so")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", include, "-x", "c++",
+    # (-Bsymbolic: its own runtime, whichever other one the process has loaded)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", include, "-x", "c++",
                     os.path.join(HERE, "fake_cuda.cpp"), os.path.join(CSRC, "dd_tv.cu"), "-o", so], check=True)
     lib = ctypes.CDLL(so)
     for name, (res, args) in _lib.SIGNATURES.items():
