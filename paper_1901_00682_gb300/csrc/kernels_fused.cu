@@ -455,12 +455,12 @@ bool one_wave(const Grid& g, const TilePlan& p) {
 // instead of three that one iterates faster.  us per outer iteration, persistent / micro-tile:
 //
 //   state beyond L2     K = 1        2           3            4            10
-//   4096 x 4096     82 / 94    94 / 108   111 / 118    127 / 130    231 / 216
+//   4096 x 4096     80 / 94    93 / 108   111 / 118    127 / 130    231 / 217
 //   2560 x 2560     35 / 40    42 / 46     49 / 50      55 / 56
 //   ... with a mask 40 / 44    47 / 50     54 / 54      62 / 59
 //   state in L2
-//   2048 x 2048     23.1 / 24.2  27.7 / 28.4  32.4 / 31.2  36.0 / 35.4
-//   ... with a mask 24.5 / 24.7  29.9 / 28.3  34.7 / 32.9
+//   2048 x 2048     22.6 / 24.2  27.2 / 28.4  31.8 / 31.2  35.9 / 35.4
+//   ... with a mask 24.4 / 24.7  29.4 / 28.3  34.3 / 32.9
 //
 // The adaptive stop runs few inner iterations where the tolerance is loose (400 outer
 // iterations of at most 10; of them all but the first end after one): 4096 x 4096 1e-3 130 /

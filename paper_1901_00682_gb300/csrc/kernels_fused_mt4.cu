@@ -31,8 +31,8 @@
 // With the next subdomain on its way while this one iterates a launch keeps the memory busy
 // throughout, which counts where it runs few inner iterations over a state larger than L2;
 // with more of them the micro-tile kernel of fused_tile.cuh is faster (use_mt4() in
-// kernels_fused.cu has both sides' times).  4096 x 4096: 81 us per outer iteration at K = 1
-// (470 MB of state, 5.8 TB/s), 231 at K = 10.
+// kernels_fused.cu has both sides' times).  4096 x 4096: 80 us per outer iteration at K = 1
+// (470 MB of state, 5.9 TB/s), 231 at K = 10.
 //
 // ADAPT: adaptive inner stopping (Section 5, eq. stop_inner1).
 // Every thread sums (p^{k+1} - p^k)^2 and (p^{k+1})^2 over its dofs in the p-step of
@@ -188,8 +188,10 @@ __device__ __forceinline__ void fused_mt4_body(const LocalArgs& A, const Mt4Maps
     remote_q1 = map_rank(smem_addr(sQ1 + NW * BW + j0), rank - 1);
     remote_mbQ = map_rank(mbQ, rank - 1);
   }
-  pdl_trigger();  // (the next update; this grid itself starts after the one before it: were its
-                  // clusters placed beside an update's blocks, some would wait for a second round)
+  // (no pdl_trigger: the next update's blocks would wait beside these clusters for the whole of the
+  // launch, 4096 x 4096 at K = 1 80.9 us per outer iteration instead of 80.4, 2048 x 2048 22.7 instead of
+  // 22.4.  And this grid itself starts after the update before it: were its clusters placed beside
+  // an update's blocks, some would wait for a second round)
   if (tid == 0) {
     mbar_init(mbU, 1);
     mbar_init(mbQ, 1);
