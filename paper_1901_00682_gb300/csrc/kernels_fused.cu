@@ -511,7 +511,7 @@ cudaError_t fused_prepare(const Grid& g, int variant, int K, double inner_tol2) 
   // is with one)
   if (use_mt4(g, variant, K, inner_tol2, false) && (e = fused_mt4_prepare(adaptive)) != cudaSuccess) return e;
   if (adaptive) {
-    if (exact128 && variant == 0 && (e = prepare_tile_adapt_128(chain)) != cudaSuccess) return e;
+    if (adapt_in_tile(g, variant, K)) return prepare_tile_adapt_128(chain);
     switch (pick((g.H + g.NR - 1) / g.NR, (g.W + g.NC - 1) / g.NC)) {
       case 0: return prepare_fid<32, 8, 4, 1, true>();
       case 1: return prepare_fid<64, 8, 8, 1, true>();
