@@ -1,6 +1,6 @@
 // Device helpers shared by the fused kernels: shared-memory and cluster addressing,
 // DSMEM stores, the split cluster barrier, packed float32 pairs, bounded mbarrier
-// waits, asynchronous copies, and the shared-memory layouts of the 128 x 128 kernels.
+// waits and asynchronous copies.
 #pragma once
 
 #include "internal.cuh"
@@ -90,45 +90,11 @@ __device__ __forceinline__ void p_update_lim(float& p, float& pbar, float du, fl
   p = pn;
 }
 
-// ---------------------------------------------------------------------------
-// Full-tile kernel: every subdomain is exactly 128 x 128 (the partition of the
-// benchmark workloads).  Same arithmetic as k_fused, without any per-pixel
-// boundary test: the band's halo rows live in the shared arrays (row 0 of sU is
-// the row above the band, row TR of sQ1 the row below it), the tile's bottom side
-// is the "row below" of the last CTA, and the right side's dofs are updated by
-// lanes 0..R-1 of each thread row's first warp (one dof per lane).
-template <int R, int TR>
-struct FullLayout {
-  static constexpr int BW = 128;
-  static constexpr int BAND = TR * R;
-  static constexpr int US = BW + 1;                    // u row stride; index 0 = zero pad
-  static constexpr int QS = BW + 1;                    // pbar2 row stride; index 128 = right side
-  static constexpr int U = 0;                          // (BAND + 1) x US: row 0 = row above the band
-  static constexpr int Q2 = U + (BAND + 1) * US;       // BAND x QS
-  static constexpr int Q1 = Q2 + BAND * QS;            // (TR + 1) x BW: first-row pbar1 per thread row; row TR = below
-  static constexpr int F = Q1 + (TR + 1) * BW;         // BAND x BW
-  static constexpr int PR = F + BAND * BW;             // BAND right-side p
-  static constexpr int HR = PR + BAND;                 // BAND right-side phat
-  static constexpr int CO = (HR + BAND + 3) & ~3;      // kMaxSmemCoef x 8 coefficients (16-byte aligned)
-  static constexpr int FLOATS = CO + 8 * 64;
-  static constexpr size_t BYTES = sizeof(float) * FLOATS;
-  static constexpr int kMaxSmemCoef = 64;
-};
-
 constexpr unsigned kWaitLimit = 1000;
 constexpr unsigned kSuspendHintNs = 1000000;
 
 __device__ __forceinline__ void mbar_init(uint32_t addr, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(addr), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_local(uint32_t addr) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.release.cta.shared::cta.b64 st, [%0];\n\t}" ::"r"(addr)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint32_t addr, uint32_t parity) {
@@ -147,18 +113,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity) {
   for (unsigned it = 0; it < kWaitLimit; ++it)
     if (mbar_try_wait(addr, parity)) return true;
   return false;
-}
-
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z),
-               "f"(v.w)
-               : "memory");
-}
-
-__device__ __forceinline__ void st_async_f32(uint32_t remote_addr, float v, uint32_t remote_mbar) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(remote_addr),
-               "r"(__float_as_uint(v)), "r"(remote_mbar)
-               : "memory");
 }
 
 // two floats into a neighbour CTA's shared memory (8-byte aligned), counted on its mbarrier
@@ -208,7 +162,6 @@ struct FidC {
 struct BatchTiles {
   const BatchArgs& B;
   int total;
-  static constexpr bool kBatch = true;
   __device__ int count() const { return total; }
   __device__ int inner() const { return B.args[0].K; }
   __device__ int image(int t) const { return B.tile_img[t]; }

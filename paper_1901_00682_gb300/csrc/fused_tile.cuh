@@ -281,8 +281,6 @@ __device__ __forceinline__ uint32_t in_box(float x) {
   return m;
 }
 
-constexpr int kTapeWords = 18;  // of the reverse pass, per thread and inner iteration
-
 // Reverse of the K iterations whose tape lies at `tape` (adj_tile.cuh).
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
 __device__ __forceinline__ void tile_reverse(const LocalArgs& A, const AdjArgs& Z, const int a, const int b, const int tid,

@@ -214,6 +214,8 @@ struct TilePlan {
 };
 // false if a subdomain is larger than 128 x 128
 bool tile_plan(const Grid& g, TilePlan* p);
+// words of the reverse pass's tape, per thread and inner iteration
+constexpr int kTapeWords = 18;
 
 // Warps of the micro-tile kernel per SM: 16 at 128 registers a thread; 12 where padding and the
 // multiplier update come together and spill (321 x 481 15.0 us per outer iteration with 16).

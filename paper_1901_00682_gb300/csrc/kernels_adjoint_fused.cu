@@ -4,12 +4,6 @@
 
 namespace ddtv {
 
-namespace {
-
-constexpr size_t kTapeWords = 18;  // per thread and inner iteration (fused_tile.cuh)
-
-}  // namespace
-
 long long adj_alpha_slots_fused(const Grid& g) { return (long long)g.NR * g.NC * 8; }
 
 size_t adj_fused_tape_floats(const Grid& g, int K) {
