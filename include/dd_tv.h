@@ -62,7 +62,12 @@ typedef enum {
 typedef enum {
   DD_TV_PATH_FUSED = 0,  /* interface kernel + fused subdomain-per-cluster local solver */
   DD_TV_PATH_PLAIN = 1,  /* one global-memory kernel per step (comparator)              */
-  DD_TV_PATH_FULLDIM = 2 /* undecomposed primal-dual iteration, N = 1 (Section 5 "CP")  */
+  DD_TV_PATH_FULLDIM = 2 /* undecomposed primal-dual iteration, N = 1 (Section 5 "CP");
+                            the handle holds two sets of u, p and the extrapolated p,
+                            20 bytes per pixel each, where there is memory for both
+                            (one set, and slower, where there is not; one also with
+                            inner_iters 1, a width that is no multiple of 4 and at
+                            most 4 Mpixel, where that is the faster way)               */
 } dd_tv_path;
 
 typedef struct {
@@ -145,7 +150,12 @@ int dd_tv_solve_device(dd_tv* h, const float* f_dev, const uint8_t* mask_dev, fl
 /* Stepping interface.  dd_tv_load copies f (and mask) from device memory into the
  * handle and initialises the state as dd_tv_solve does; dd_tv_iterate runs n_outer
  * outer iterations on the resident state (asynchronous); dd_tv_get_u copies the
- * current u to u_dev. */
+ * current u to u_dev.  A load that fails for want of memory leaves the handle as it was.
+ *
+ * dd_tv_iterate calls of fewer than 4 outer iterations (longer ones replay graphs of the
+ * handle's own) and dd_tv_get_u can be captured into a caller's CUDA graph.  Every replay
+ * then advances the iterate, on the decomposed paths if the graph runs an even number of
+ * outer iterations (they keep two sets of interface values in turn). */
 int dd_tv_load(dd_tv* h, const float* f_dev, const uint8_t* mask_dev);
 int dd_tv_iterate(dd_tv* h, int n_outer);
 int dd_tv_get_u(dd_tv* h, float* u_dev);
@@ -365,8 +375,11 @@ long long dd_tv_batch_pixels(const dd_tv_batch* b);
  * interface values of p~^{n-1}) before every checkpoint_every-th outer iteration in
  * handle-owned device memory: ceil(n_outer / m) + m states of about
  * 4 (3 H W + 5 (interface edges)) bytes each (m = min(checkpoint_every, n_outer)),
- * plus the reverse pass's tape and adjoint fields (about (4 + 2) inner_iters + 60
- * bytes per pixel), allocated on the first call and kept (and grown) until
+ * plus the adjoint fields (about 40 bytes per pixel) and the reverse pass's tape: 4.5
+ * inner_iters bytes per pixel of the blocks that cover the subdomains (32, 64 or 128
+ * wide, so up to four times the image's for small or uneven ones), and about (4 + 2)
+ * inner_iters + 20 per pixel for subdomains larger than 128 x 128 or beyond 4 GiB of
+ * tape.  All of it is allocated on the first call and kept (and grown) until
  * dd_tv_adjoint_release or dd_tv_destroy.  Writes u_N to u_dev (device, H x W).
  * Asynchronous on the handle's stream.  checkpoint_every < 1 returns DD_TV_EINVAL.
  *

@@ -530,9 +530,11 @@ __device__ __forceinline__ void tile_reverse(const LocalArgs& A, const AdjArgs& 
   tile_reverse_store<LPR, NW, PAD>(A.g, Z, a2, b2, tid2, rank, CL, Au, T1, T2, t_r, h_r, acc);
 }
 
-// 12 warps per SM: the reverse loop does not fit the forward's 128 registers (with 16 warps,
-// forward and backward of 250 x 261 take 2610 us instead of 2340, of two 1024 x 1024 3840
-// instead of 3600)
+// CTAs of up to 4 warps run 12 warps per SM: the reverse loop does not fit the forward's 128
+// registers (with 16 warps, forward and backward of 250 x 261 take 2610 us instead of 2340, of two
+// 1024 x 1024 3840 instead of 3600).  Those of 8 warps (64 x 64 subdomains) run two per SM at 128
+// registers, with 136 to 220 bytes of spills per thread: at the 168 of the others only one would
+// fit.
 template <int LPR, int NW, bool CLU, bool PAD, int FID, bool MASK>
 __global__ void __launch_bounds__(32 * NW, NW <= 4 ? 12 / NW : 2) k_adj_tile(const LocalArgs A, const AdjArgs Z, const int cl) {
   const unsigned t = CLU ? blockIdx.x / (unsigned)cl : blockIdx.x, rank = CLU ? blockIdx.x - t * (unsigned)cl : 0u;

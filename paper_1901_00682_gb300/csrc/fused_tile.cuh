@@ -32,10 +32,10 @@
 // the kernels it replaced (the cluster-barrier kernel, a column of 8 pixels per thread;
 // for exact 128 x 128 subdomains the persistent clusters of kernels_fused_mt4.cu with
 // three CTAs per SM): 1080 x 1920 in 120 x 128 subdomains 106 -> 41 us, 2160 x 3840
-// 448 -> 137, 2999 x 3001 in 125 x 125/126 477 -> 158, 4096 x 4096 in 64 x 64 572 -> 213 and in
-// 32 x 32 527 -> 187, 512 x 512 in 32 x 32 19.1 -> 8.4, 128 x 128 in 64 x 64 21.1 -> 10.9, 321 x
-// 481 in 107 x 120/121 25.8 -> 14.0; in 128 x 128 subdomains 512 x 512 14.0 -> 11.9, 1024 x 1024
-// 22.7 -> 18.1, 4096 x 4096 231 -> 216 (K = 10; where the persistent kernel is the faster
+// 446 -> 139, 2999 x 3001 in 125 x 125/126 473 -> 161, 4096 x 4096 in 64 x 64 571 -> 214 and in
+// 32 x 32 526 -> 197, 512 x 512 in 32 x 32 19.6 -> 8.3, 128 x 128 in 64 x 64 22.1 -> 10.8, 321 x
+// 481 in 107 x 120/121 26.2 -> 13.9; in 128 x 128 subdomains 512 x 512 14.4 -> 11.8, 1024 x 1024
+// 22.8 -> 18.1, 4096 x 4096 230 -> 217 (K = 10; where the persistent kernel is the faster
 // one, use_mt4() in kernels_fused.cu), a batch of 64 images (168 Mpixel) 2730 -> 2300; with
 // the adaptive stop, 1024 x 1024 and 18.7 inner iterations on average, 54 -> 43.
 //
