@@ -87,7 +87,8 @@ struct dd_tv {
   // plain path: phat and pbar; full-dimension path: pbar (carried across iterations)
   float *Ph1 = nullptr, *Ph2 = nullptr, *Pb1 = nullptr, *Pb2 = nullptr;
   // full-dimension path: the two sets its launches go back and forth between (u, P1, ...
-  // above point into full[full_cur], which holds the current iterate); full_mem is set 1
+  // above point into full[full_cur], which holds the current iterate); full_mem holds set 1 and the
+  // pbar of set 0
   FullSet full[2] = {};
   int full_cur = 0;
   float* full_mem = nullptr;
@@ -1011,18 +1012,11 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
     dd_tv_destroy(h);
     return rc;
   }
-  if (p->path != DD_TV_PATH_FUSED) {
-    if ((rc = dalloc(h, &h->Pb1, h->n1)) || (rc = dalloc(h, &h->Pb2, h->n2))) {
-      std::snprintf(g_create_err, sizeof(g_create_err), "%s", h->err);
-      dd_tv_destroy(h);
-      return rc;
-    }
-  }
   if (p->path == DD_TV_PATH_FULLDIM && !full_half_steps(h)) {
-    // the second set, every array on a 256-byte boundary; without room for it the path
-    // runs a launch per half-step in place
+    // pbar and the second set in one allocation, every array on a 256-byte boundary; without
+    // room for it the path runs a launch per half-step in place
     auto up = [](size_t n) { return (n + 63) & ~(size_t)63; };
-    const size_t n = up(h->npx) + 2 * up(h->n1) + 2 * up(h->n2);
+    const size_t np = up(h->n1) + up(h->n2), n = up(h->npx) + 3 * np;
     const cudaError_t room = cudaMalloc((void**)&h->full_mem, n * sizeof(float));
     if (room == cudaErrorMemoryAllocation) {
       cudaGetLastError();
@@ -1030,7 +1024,7 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
     } else {
       cudaError_t e = room;
       if (e == cudaSuccess) e = cudaMemset(h->full_mem, 0, n * sizeof(float));
-      if (e == cudaSuccess) e = full_prepare();
+      if (e == cudaSuccess) e = full_prepare(h->fid);
       if (e != cudaSuccess) {
         std::snprintf(g_create_err, sizeof(g_create_err), "full-dimension kernel set-up: %s", cudaGetErrorString(e));
         if (room == cudaSuccess) cudaFree(h->full_mem);
@@ -1039,12 +1033,27 @@ int create_impl(dd_tv** out, const dd_tv_params* p, int a0, int a1) {
         return DD_TV_ECUDA;
       }
       float* m = h->full_mem;
+      auto take = [&](size_t len) {
+        float* at = m;
+        m += up(len);
+        return at;
+      };
+      h->Pb1 = take(h->n1);
+      h->Pb2 = take(h->n2);
       h->full[0] = FullSet{h->u, h->P1, h->P2, h->Pb1, h->Pb2};
-      h->full[1].u = m;
-      h->full[1].P1 = m += up(h->npx);
-      h->full[1].P2 = m += up(h->n1);
-      h->full[1].Pb1 = m += up(h->n2);
-      h->full[1].Pb2 = m += up(h->n1);
+      FullSet& s = h->full[1];
+      s.u = take(h->npx);
+      s.P1 = take(h->n1);
+      s.P2 = take(h->n2);
+      s.Pb1 = take(h->n1);
+      s.Pb2 = take(h->n2);
+    }
+  }
+  if (p->path != DD_TV_PATH_FUSED && !h->full_mem) {
+    if ((rc = dalloc(h, &h->Pb1, h->n1)) || (rc = dalloc(h, &h->Pb2, h->n2))) {
+      std::snprintf(g_create_err, sizeof(g_create_err), "%s", h->err);
+      dd_tv_destroy(h);
+      return rc;
     }
   }
   if (p->path == DD_TV_PATH_PLAIN) {
@@ -1111,8 +1120,9 @@ int dd_tv_destroy(dd_tv* h) {
   drop_graphs(h);
   adj_free(h->adj);
   h->adj = nullptr;
-  if (h->full_mem) {  // u, P1, ... back to the arrays allocated one by one
+  if (h->full_mem) {  // u, P1, P2 back to the arrays allocated one by one
     full_select(h, 0);
+    h->Pb1 = h->Pb2 = nullptr;
     cudaFree(h->full_mem);
   }
   for (auto& m : h->marks) {

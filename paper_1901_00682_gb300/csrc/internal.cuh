@@ -246,7 +246,8 @@ cudaError_t launch_tile_batch_64(const BatchArgs& B, int total_tiles, bool overl
 // the image boundary are 0 and not written)
 cudaError_t launch_full(const FullArgs& a, int fidelity, int n, cudaStream_t st);
 int full_max_steps();
-cudaError_t full_prepare();
+// shared-memory opt-in of the instances of a fidelity (outside any stream capture)
+cudaError_t full_prepare(int fidelity);
 
 // ---- kernels_plain.cu
 // phat = p~ -+ tau lambda on the interface sides, pbar = p~; full arrays.

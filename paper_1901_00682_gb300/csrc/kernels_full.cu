@@ -352,16 +352,16 @@ cudaError_t launch_full(const FullArgs& a, int fid, int n, cudaStream_t st) {
   }
 }
 
-cudaError_t full_prepare() {
+cudaError_t full_prepare(int fid) {
   cudaError_t e;
   auto set = [](auto kern) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FL::BYTES);
   };
-  if ((e = set(k_full<FID_L2, false>)) != cudaSuccess) return e;
-  if ((e = set(k_full<FID_L2, true>)) != cudaSuccess) return e;
-  if ((e = set(k_full<FID_L1, false>)) != cudaSuccess) return e;
-  if ((e = set(k_full<FID_L1, true>)) != cudaSuccess) return e;
-  return set(k_full<FID_SEG, false>);
+  switch (fid) {
+    case FID_L2: return (e = set(k_full<FID_L2, false>)) != cudaSuccess ? e : set(k_full<FID_L2, true>);
+    case FID_L1: return (e = set(k_full<FID_L1, false>)) != cudaSuccess ? e : set(k_full<FID_L1, true>);
+    default: return set(k_full<FID_SEG, false>);
+  }
 }
 
 }  // namespace ddtv

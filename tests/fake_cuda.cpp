@@ -22,6 +22,7 @@ std::string g_log;
 size_t g_fail_bytes = 0;     // an allocation of at least this size fails (0: none does)
 int g_operations = 0;        // put on the stream (copies, memsets, launches)
 bool g_chain = false;        // the local solves make the multiplier update
+int g_allocations = 0;
 int g_fail_at = 0;           // the allocation that fails, counted from here (0: none does)
 cudaError_t g_prepare_error = cudaSuccess;
 
@@ -48,12 +49,14 @@ extern "C" {
 const char* fake_log() { return g_log.c_str(); }
 void fake_clear_log() { g_log.clear(); }
 void fake_fail_allocations(size_t at_least_bytes) { g_fail_bytes = at_least_bytes; }
+int fake_allocations() { return g_allocations; }
 int fake_operations() { return g_operations; }
 void fake_chain(int on) { g_chain = on; }
 void fake_fail_allocation(int k) { g_fail_at = k; }
 void fake_fail_prepare(int error) { g_prepare_error = (cudaError_t)error; }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
+  ++g_allocations;
   if ((g_fail_bytes && n >= g_fail_bytes) || (g_fail_at && --g_fail_at == 0)) return cudaErrorMemoryAllocation;
   *p = std::calloc(n, 1);
   return cudaSuccess;
@@ -159,7 +162,7 @@ cudaError_t launch_init_u(const Grid& g, int, const float* f, const uint8_t*, fl
 }
 
 // ---- full-dimension and plain paths
-cudaError_t full_prepare() { return g_prepare_error; }
+cudaError_t full_prepare(int) { return g_prepare_error; }
 int full_max_steps() { return 10; }
 cudaError_t launch_full(const FullArgs& a, int, int n, cudaStream_t) {
   const float* in = a.in.u;

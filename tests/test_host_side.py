@@ -190,3 +190,14 @@ def test_chained_update_costs_loads_and_set_state_nothing(lib, sub):
     assert ops[1][0] == ops[0][0]
     assert ops[1][1] <= ops[0][1] + (sub != (1, 1))
     assert ops[1][1] <= 3 + (sub[0] > 1) + (sub[1] > 1) + 2
+
+
+def test_second_set_of_arrays_takes_no_allocation_of_its_own(lib):
+    """Creating a full-dimension handle allocates no more often with it than without."""
+    n = []
+    for W in (60, 61):   # two sets; one (single iterations of unaligned rows)
+        before = lib.fake_allocations()
+        with Handle(lib, 70, W, 1, 1, path=2, inner_iters=1) as s:
+            assert s.rc == 0
+            n.append(lib.fake_allocations() - before)
+    assert n[0] <= n[1]
