@@ -36,7 +36,7 @@
 // 32 x 32 526 -> 197, 512 x 512 in 32 x 32 19.6 -> 8.3, 128 x 128 in 64 x 64 22.1 -> 10.8, 321 x
 // 481 in 107 x 120/121 26.2 -> 13.9; in 128 x 128 subdomains 512 x 512 14.4 -> 11.8, 1024 x 1024
 // 22.8 -> 18.1, 4096 x 4096 230 -> 217 (K = 10; where the persistent kernel is the faster
-// one, use_mt4() in kernels_fused.cu), a batch of 64 images (168 Mpixel) 2730 -> 2300; with
+// one, use_mt4() in kernels_fused.cu), a batch of 64 images (168 Mpixel) 2730 -> 2320; with
 // the adaptive stop, 1024 x 1024 and 18.7 inner iterations on average, 54 -> 43.
 //
 // Every value is computed with the operations of the scalar iteration in its order

@@ -26,7 +26,7 @@ __global__ void k_interface_v4(int nh4, int nv4, float sigma, const float4* __re
                                const float4* __restrict__ pSR, const float4* __restrict__ pSL,
                                float4* __restrict__ lamv) {
   pdl_wait();     // the previous local solves
-  pdl_trigger();  // the next ones may start: they wait for this kernel before they read lambda
+  pdl_trigger();  // the next ones may start, and wait for this kernel before they load the state
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nh4 + nv4; e += gridDim.x * blockDim.x) {
     const bool h = e < nh4;
     const int q = h ? e : e - nh4;
@@ -51,7 +51,7 @@ __global__ void k_interface_v1(int nh, int nv, float sigma, const float* __restr
                                const float* __restrict__ pSR, const float* __restrict__ pSL,
                                float* __restrict__ lamv) {
   pdl_wait();     // the previous local solves
-  pdl_trigger();  // the next ones may start: they wait for this kernel before they read lambda
+  pdl_trigger();  // the next ones may start, and wait for this kernel before they load the state
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nh + nv; e += gridDim.x * blockDim.x) {
     if (e < nh) {
       lamh[e] = lam_step(lamh[e], sigma, cSB[e], pSB[e], cST[e], pST[e]);
@@ -118,7 +118,7 @@ __global__ void k_scatter(Grid g, Strips s, float* __restrict__ P1, float* __res
 // float4 elements of all images are numbered consecutively, image by image.
 __global__ void k_interface_batch(BatchIfaceArgs B, int total4) {
   pdl_wait();     // the previous local solves
-  pdl_trigger();  // the next ones may start: they wait for this kernel before they read lambda
+  pdl_trigger();  // the next ones may start, and wait for this kernel before they load the state
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total4; e += gridDim.x * blockDim.x) {
     int lo = 0, hi = B.n_img;  // find the image: elem_base[img] <= e < elem_base[img + 1]
     while (hi - lo > 1) {
